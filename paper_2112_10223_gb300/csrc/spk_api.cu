@@ -518,10 +518,10 @@ SPK_API spkadd_status spkadd_batch_symbolic(spkadd_handle* h, int64_t* nnz_B) {
 // The numeric kernels of every problem, writing through `out`.
 static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
   cudaError_t ce = cudaSuccess;
-  const int cta_items = h->h_ctr.n_windows;
   int item_launches = 0;
-  if (cta_items > 0)
-    ce = spk::launch_num_cta(h->in, h->dt_mode, h->f32_kinds, h->d_win, cta_items, h->d_wsort, h->h_ctr.kind_n,
+  if (h->h_ctr.n_windows + h->h_ctr.n_hwin > 0)
+    ce = spk::launch_num_cta(h->in, h->dt_mode, h->f32_kinds, h->d_win, h->win_cap, h->h_ctr.n_windows,
+                             h->h_ctr.n_hwin, h->d_wsort, h->h_ctr.kind_n,
                              h->d_offs, h->d_colptr, out,
                              h->opt.window_max > h->opt.cta_max ? h->opt.window_max : h->opt.cta_max,
                              h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
@@ -656,7 +656,7 @@ SPK_API spkadd_status spkadd_get_info(spkadd_handle* h, spkadd_info* info) {
   info->cols_warp = c.n_warp;
   info->cols_cta = c.n_cta;
   info->cols_heavy = (int64_t)c.n_heavy + c.n_big;
-  info->windows = c.n_windows;
+  info->windows = (int64_t)c.n_windows + c.n_hwin;
   info->windows_split = c.n_search;
   info->cols_unique = c.n_unique;
   info->workspace_bytes = (int64_t)(h->ws_bytes + h->offs_bytes);

@@ -35,15 +35,16 @@ struct Window {
 
 struct Counters {
   int32_t n_warp, n_cta, n_heavy;
-  int32_t n_windows;    // Window records appended
+  int32_t n_windows;    // Window records of CTA-class columns, from the record array's start
   int32_t n_search;     // of those, split windows needing per-input offsets
   int32_t n_unique;     // warp columns whose input rows are all distinct (u_j == s_j)
   int32_t err;
   int32_t n_big;        // heavy columns with s_j > BIG_S (listed apart, counted in n_heavy too)
   int32_t heavy_next;   // work counter of the heavy-column symbolic kernels
-  int32_t kind_n[4];    // batches of several problem kinds: thread-block items per kind
-  int32_t kind_fill[4]; //   and their placement counters
-  int32_t pad[3];
+  int32_t n_hwin;       // Window records of heavy columns, from the record array's end
+  int32_t kind_n[8];    // batches of several problem kinds: thread-block items per kind (CTA-class, then heavy)
+  int32_t kind_fill[8]; //   and their placement counters
+  int32_t pad[2];
 };
 
 // Float sums.  A float sum of t terms, in any order, errs by at most

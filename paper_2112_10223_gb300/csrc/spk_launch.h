@@ -62,15 +62,16 @@ cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const
 // larger float, bit 3 double); f32_kinds holds bits 0-2 of the float problems.
 int num_cta_kinds(int dt, int f32_kinds);
 // Several kinds: copies the symbolic phase's window records (at most `cap`)
-// into wsort grouped by kind; ctr->kind_n gets the count of each.
+// into wsort grouped by class and kind; ctr->kind_n gets the count of each.
 cudaError_t launch_kind_sort(const Inputs& in, const Window* win, int cap, Window* wsort, Counters* ctr_w,
                              const DeviceInfo& dev, cudaStream_t st);
-// One launch per kind present: over win[0, n_win) when the batch has one
-// kind, else over the kind's group of wsort (host copy of kind_n).
-cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int n_win,
-                           const Window* wsort, const int32_t* kind_n, const int32_t* offs, const int64_t* col_ptr,
-                           const Outs& out, int window_max, int accumulator, Counters* ctr_w, const DeviceInfo& dev,
-                           cudaStream_t st, int* launches);
+// One launch per class and kind present: over the n_cta records at win's start
+// and the n_heavy ones at its end (win_cap records) when the batch has one
+// kind, else over the groups of wsort (host copy of kind_n).
+cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int64_t win_cap, int n_cta,
+                           int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
+                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
+                           const DeviceInfo& dev, cudaStream_t st, int* launches);
 // Per-problem column pointers of B (a batch): out_cp[q][j] = col_ptr[colbase + j] - col_ptr[colbase].
 cudaError_t launch_out_colptr(const Inputs& in, const Outs& o, const int64_t* col_ptr, int sms, cudaStream_t st);
 // Per-problem nnz(B): nnz[q] = col_ptr[colbase + n] - col_ptr[colbase].

@@ -24,14 +24,15 @@
 // rows span more is processed slab by slab, with per-input binary searches
 // for each slab's entries.
 //
-// A second layout, the compact word table (k_num_compact, below), keeps only
-// a summary bit per 32-row word and a table of the item's non-empty words, so
-// its shared memory follows window_max instead of the slab; the launcher runs
-// whichever layout has more blocks resident per SM.
+// k_num_items (below) is this accumulator with the entries' rows in registers,
+// as a flat bitmap or a compact word table; k_num_bitmap, which walks the
+// entries once per pass, runs only for block_accumulator = 1 on slabs of more
+// than 2^17 rows, whose bitmap fills the SM.
 #include <mutex>
 #include <type_traits>
 
 #include "spk_common.cuh"
+#include "spk_items.cuh"
 #include "spk_launch.h"
 
 namespace spk {
@@ -154,7 +155,6 @@ template <typename V, typename A, bool PHASED, int BLOCK, int U>
 __device__ __forceinline__ void bitmap_item(const Inputs& in, const Window& W, const Inst* I, const int32_t* offs,
                                             int32_t* __restrict__ out_row, V* __restrict__ out_val,
                                             const BitmapSmem& sm, int slab_log2, Counters* ctr_w) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int k = I->k, off = I->ptr_off, j = W.col - I->colbase;
   A* acc = reinterpret_cast<A*>(sm.acc);
   const int64_t S = (int64_t)1 << slab_log2;
@@ -281,46 +281,117 @@ __device__ __forceinline__ void bitmap_item(const Inputs& in, const Window& W, c
 }
 
 // ---------------------------------------------------------------------------
-// Compact word table: the same exact-rank accumulator for items whose rows
-// span a large slab but are few (at most umax distinct rows).  The flat
-// bitmap's size follows the slab (128 KB at 2^20 rows); here only the
-// summary follows the slab (one bit per 32-row word: 4 KB at 2^20) and the
-// row bits live in a table of the non-empty words, which has at most umax
-// entries.  Shared memory drops to about a quarter, so several items are in
-// flight per SM instead of one.  One more pass over the item's entries:
+// Items in registers (spk_items.cuh): the same exact-rank accumulator, with a
+// layout picked per item slab:
 //
-//   pass A1  every entry sets its word's summary bit
-//   rank 1   popcount prefix over the summary: word w gets the compact
-//            index c(w) = prefix(w / 32) + popcount(summary bits below w);
-//            nel[c] = w lists the non-empty words in row order
-//   pass A2  every entry sets its bit in cw[c(w)]
-//   rank 2   popcount prefix over cw: wpre[c]
-//   pass B   acc[wpre[c] + popcount(cw[c] & bits below r)] += value
-//   write    words expanded to rows in rank order, values copied out
+//   flat     (at most 2^17 rows) one bit per row
+//     pass A   every entry sets its row's bit
+//     rank     popcount prefix over all words: wpre[w]
+//     pass B   acc[wpre[w] + popcount(bits of w below r)] += value
+//   compact  (up to 2^20 rows, at most umax of them present) a summary bit
+//            per 32-row word, and a table of the non-empty words in row order
+//     pass A1  every entry sets its word's summary bit
+//     rank 1   popcount prefix over the summary: word w gets the compact index
+//              c(w) = spre[w / 32] + popcount(summary bits below w)
+//     pass A2  every entry sets its row's bit in cw[c(w)]
+//     rank 2   popcount prefix over cw: wpre[c]
+//     pass B   acc[wpre[c] + popcount(cw[c] & bits below r)] += value
+//   write    values copied out in rank order; then the words expanded to rows
+//            in the accumulator's slots (free once the values are out) and
+//            copied out, so both are written coalesced
+//
+// The rows are read once, into registers, for items of one chunk; the value
+// segments start toward L2 while the rows are ranked.
+// What bounds it: issue slots and shared-memory wavefronts at once (60% and 55%
+// busy on 2^15 columns of 2048 entries, 128 distinct rows; the rest is barriers).
+// Measured against three walks over the entries with a segment search each:
+// 131072 such columns (float) 3.23 -> 2.14 ms, R-MAT scale 20 k = 64 12.7 ->
+// 10.6 ms, 65537 unordered ragged columns 1.20 -> 0.60 ms.
 // ---------------------------------------------------------------------------
-struct CompactSmem {
-  uint32_t* summ;  // NSW: one bit per 32-row word of the slab (kept zero between slabs)
-  uint16_t* spre;  // NSW: exclusive popcount prefix of the summary words
-  uint32_t* cw;    // umax: row bits of the non-empty words, in row order (kept zero)
-  uint16_t* wpre;  // umax: exclusive popcount prefix of cw
-  uint16_t* nel;   // umax: word index of each compact word
-  unsigned char* acc;
-  int* red;        // BLOCK/32 + 1 scan slots
-  int NSW, umax;
+constexpr int FLAT_LOG2 = 17;  // rows of a flat slab: 16 KB of bits
+constexpr int FLAT_ROWS = 1 << FLAT_LOG2;
+
+// A flat bitmap word's place: four pad words after every 16, so that threads
+// owning 16 consecutive words each start their 16-byte loads on their own banks.
+__host__ __device__ constexpr int pad_word(int w) { return w + ((w >> 4) << 2); }
+
+// Shared-memory layout.  WIDE: slabs above FLAT_ROWS occur (both forms may run).
+template <bool WIDE, int B>
+struct ItemLayout {
+  int wflat;      // words of the flat bitmap
+  int zero;       // words kept zero between slabs: flat bits, or summary + compact words
+  int pre;        // bytes of prefixes: flat wpre, or spre + compact wpre
+  size_t acc;     // bytes of the accumulator (at least 4 per rank: it holds the rows at the end)
+  __host__ __device__ ItemLayout(int slab_log2, int umax, int asize) {
+    const int fl = slab_log2 < FLAT_LOG2 ? slab_log2 : FLAT_LOG2;
+    wflat = 1 << (fl - 5);
+    if (wflat < 4 * B) wflat = 4 * B;
+    zero = pad_word(wflat);
+    pre = 2 * wflat;
+    if (WIDE) {
+      if (zero < 1024 + umax) zero = 1024 + umax;
+      if (pre < 2 * (1024 + umax)) pre = 2 * (1024 + umax);
+    }
+    zero = (zero + 3) & ~3;
+    pre = (pre + 15) & ~15;
+    acc = ((size_t)umax * asize + 15) & ~(size_t)15;
+  }
+  __host__ __device__ size_t bytes() const { return acc + (size_t)zero * 4 + pre + sizeof(ItemMap<B>) + 2 * sizeof(Window); }
 };
 
-// Compact index of the non-empty 32-row word w.
-__device__ __forceinline__ int compact_index(const CompactSmem& sm, uint32_t w) {
-  const uint32_t x = w >> 5;
-  return (int)sm.spre[x] + __popc(sm.summ[x] & ((1u << (w & 31)) - 1u));
+template <int B>
+struct ItemSmem {
+  unsigned char* acc;
+  uint32_t* zero;  // flat bits / summary, then cw
+  uint16_t* pre;   // flat wpre / spre, then compact wpre
+  ItemMap<B>* map;
+  Window* win;     // this item's record and the next one's, by turns
+  int umax;
+};
+
+// Input i's part of the item of window W in column j.
+__device__ __forceinline__ void window_seg(const Inputs& in, const Window& W, const int32_t* offs, int off, int j, int i,
+                                           int* beg, int* end) {
+  if (W.search < 0) {
+    const int32_t* cp = in.cp[off + i];
+    *beg = __ldg(cp + j);
+    *end = __ldg(cp + j + 1);
+  } else {
+    const int32_t* o = offs + ((int64_t)W.search * in.kmax + i) * 2;
+    *beg = o[0];
+    *end = o[1];
+  }
 }
 
-template <typename V, typename A, bool PHASED, int BLOCK, int U>
-__device__ __forceinline__ void compact_item(const Inputs& in, const Window& W, const Inst* I, const int32_t* offs,
-                                             int32_t* __restrict__ out_row, V* __restrict__ out_val,
-                                             const CompactSmem& sm, int slab_log2, Counters* ctr_w) {
+// One item, the record at sm.win[turn].  F holds the bounds of its first segment
+// table (read while the previous item ran) and leaves with those of the next
+// item, whose record (null: none) goes to sm.win[turn ^ 1].
+template <typename V, typename A, bool PHASED, bool WIDE, int B>
+__device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, int turn, ItemBounds<B>& F,
+                                         const int32_t* offs, int32_t* __restrict__ out_row, V* __restrict__ out_val,
+                                         const ItemSmem<B>& sm, int slab_log2, int flat_rows, Counters* ctr_w) {
+  constexpr int KT = ItemMap<B>::KT, CAP = ItemMap<B>::CAP;
+  const int tid = threadIdx.x;
+  const Window& W = sm.win[turn];
+  const Inst* I = in.inst + inst_of(in, W.col);
   const int k = I->k, off = I->ptr_off, j = W.col - I->colbase;
+  int next_word = 0;
+  if (next && tid < (int)(sizeof(Window) / 4)) next_word = reinterpret_cast<const int32_t*>(next)[tid];
+  auto next_bounds = [&]() {
+    const Window& Wn = sm.win[turn ^ 1];
+    const Inst* In = in.inst + inst_of(in, Wn.col);
+    const int jn = Wn.col - In->colbase, offn = In->ptr_off;
+    auto segn = [&](int i, int* beg, int* end) { window_seg(in, Wn, offs, offn, jn, i, beg, end); };
+    return item_bounds<B>(0, min(In->k, KT), segn);
+  };
   A* acc = reinterpret_cast<A*>(sm.acc);
+  ItemMap<B>& M = *sm.map;
+  uint32_t* bits = sm.zero;      // flat
+  uint16_t* wpre = sm.pre;
+  uint32_t* summ = sm.zero;      // compact
+  uint32_t* cw = sm.zero + 1024;
+  uint16_t* spre = sm.pre;
+  uint16_t* cpre = sm.pre + 1024;
   const int64_t S = (int64_t)1 << slab_log2;
   const int64_t span = (int64_t)W.r_hi - W.r_lo;
   const int nsl = span <= 0 ? 0 : (int)((span + S - 1) >> slab_log2);
@@ -330,175 +401,373 @@ __device__ __forceinline__ void compact_item(const Inputs& in, const Window& W, 
     const int lo = W.r_lo + (int)(t * S);
     const int hi = (int)min((int64_t)W.r_hi, (int64_t)lo + S);
     const uint32_t width = (uint32_t)(hi - lo);
-    auto seg = [&](int i, int* beg, int* len) {
+    const bool flat = !WIDE || width <= (uint32_t)flat_rows;
+    // The item's entries of input i that fall in [lo, hi).
+    auto seg = [&](int i, int* beg, int* end) {
       int b, e;
-      if (W.search < 0) {
-        const int32_t* cp = in.cp[off + i];
-        b = __ldg(cp + j);
-        e = __ldg(cp + j + 1);
-      } else {
-        const int32_t* o = offs + ((int64_t)W.search * in.kmax + i) * 2;
-        b = o[0];
-        e = o[1];
-      }
-      if (nsl > 1 && in.sorted) {
+      window_seg(in, W, offs, off, j, i, &b, &e);
+      if (nsl > 1 && in.sorted) {  // unordered inputs: the whole segment, rows outside the slab skipped
         const int32_t* ri = in.ri[off + i];
         b = lower_bound_i32(ri, b, e, lo);
         e = lower_bound_i32(ri, b, e, hi);
       }
       *beg = b;
-      *len = e - b;
+      *end = e;
     };
-    auto none = [](uint32_t, int32_t, V) {};
-    // Pass A1: summary bits (a read first: dense items hit few words often).
-    int n_ent = 0;  // PHASED: entries this thread met in the slab
-    auto mark = [&](int32_t r, V) -> uint32_t {
-      const uint32_t rr = (uint32_t)(r - lo);
-      if (rr < width) {
-        if constexpr (PHASED) ++n_ent;
-        const uint32_t w = rr >> 5, bit = 1u << (w & 31);
-        if (!(sm.summ[w >> 5] & bit)) atomicOr(&sm.summ[w >> 5], bit);
-      }
-      return 0u;
-    };
-    SegCache sc{0, 0, false};
-    block_for_each_entry<false, V, BLOCK, U, decltype(seg), decltype(mark), decltype(none), true>(in, k, off, seg,
-                                                                                                  mark, none, sc);
-    __syncthreads();
+    uint32_t r[ITEM_SLOTS];  // rows less lo
+    ItemSlots<B> L;
+    int total = 0;  // positions of the current segment table
+    L.ns = 0;
+    const int nib = (k + KT - 1) / KT;
+    bool single = false;  // the whole item sits in r[]
     int s_ent = 0;
-    if constexpr (PHASED) block_excl_scan<BLOCK>(n_ent, sm.red, &s_ent);
-    // Rank 1: thread t owns summary words [t*ps, t*ps + ps).
+    auto table = [&](int ib, bool first, int* red) {
+      const int k_lo = ib * KT, nk = min(KT, k - k_lo);
+      if (!(first && ib == 0 && nsl == 1)) F = item_bounds<B>(k_lo, nk, seg);
+      if (!first) {
+        total = item_table<sizeof(V), false, false>(M, in, off, k_lo, nk, F, red);
+        return;
+      }
+      total = item_table<sizeof(V), true, true>(M, in, off, k_lo, nk, F, red);
+      if (t == 0 && ib == 0 && next && tid < (int)(sizeof(Window) / 4))  // (every thread is past the previous item)
+        reinterpret_cast<int32_t*>(&sm.win[turn ^ 1])[tid] = next_word;
+      s_ent += total;
+      single = nib == 1 && total <= CAP;
+    };
+    const uint32_t wmax = width - 1u;
+    // Loaded rows to rows less lo; those outside the slab become 0xffffffff.
+    auto relative = [&]() {
+#pragma unroll
+      for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+        if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+        for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
+          r[q] -= (uint32_t)lo;
+          r[q] = r[q] <= wmax ? r[q] : 0xffffffffu;
+        }
+      }
+    };
+    // Compact index of a row's word.
+    auto compact = [&](uint32_t c) {
+      const uint32_t wd = c >> 5;
+      return (int)spre[wd >> 5] + __popc(summ[wd >> 5] & ((1u << (wd & 31)) - 1u));
+    };
+    // Runs op over every chunk of rows.  A single-chunk item is loaded by the
+    // first call only; others reload their rows (and rebuild the map) each time.
+    auto rows_pass = [&](bool first, auto&& op) {
+      if (!first && single) {
+        op();
+        return;
+      }
+      for (int ib = 0; ib < nib; ++ib) {
+        if (first || nib > 1) {
+          if (nib > 1) __syncthreads();
+          table(ib, first, M.red[0]);
+          if (!first) __syncthreads();
+        }
+        for (int c0 = 0; total > 0; c0 += CAP) {
+          if (!first || c0 > 0) item_map(M, c0);
+          __syncthreads();
+          L.init(c0, total);
+          item_rows(M, L, c0, r);
+          relative();
+          op();
+          if (single) break;
+          __syncthreads();
+          item_unmap(M);
+          __syncthreads();
+          if (total - c0 <= CAP) break;
+        }
+      }
+    };
+    int slab_u = 0, ne = 0;
+    bool fits;
     const int nwords = (int)((width + 31) >> 5);
-    const int nsw = (nwords + 31) >> 5;
-    const int ps = (nsw + BLOCK - 1) / BLOCK;
-    const int x0 = min(nsw, (int)threadIdx.x * ps), x1 = min(nsw, x0 + ps);
-    int loc = 0;
-    for (int x = x0; x < x1; ++x) loc += __popc(sm.summ[x]);
-    int ne;
-    int c = block_excl_scan<BLOCK>(loc, sm.red, &ne);
-    const bool ne_fits = ne <= sm.umax && !bad;
-    if (ne_fits) {
-      for (int x = x0; x < x1; ++x) {
-        sm.spre[x] = (uint16_t)c;
-        for (uint32_t bits = sm.summ[x]; bits; bits &= bits - 1) sm.nel[c++] = (uint16_t)(x * 32 + __ffs(bits) - 1);
+    // Ownership of words for the rank scans: `per` consecutive words a thread.
+    const int per = nwords <= 4 * B ? 4 : (nwords <= 8 * B ? 8 : 16);
+    // The passes have no branches: addresses come from the row clamped into
+    // the slab, and only the atomic itself is predicated.
+    rows_pass(true, [&]() {
+#pragma unroll
+      for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+        if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+        for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
+          const uint32_t c = min(r[q], wmax);
+          uint32_t* w = flat ? &bits[pad_word((int)(c >> 5))] : &summ[c >> 10];
+          const uint32_t bit = 1u << (flat ? c & 31 : (c >> 5) & 31);
+          if (r[q] <= wmax) atomicOr(w, bit);
+        }
       }
-    } else {
-      bad = true;
-    }
+    });
     __syncthreads();
-    int slab_u = 0;
-    bool fits = false;
-    if (ne_fits) {
-      // Pass A2: row bits of the compact words.
-      auto setbit = [&](int32_t r, V) -> uint32_t {
-        const uint32_t rr = (uint32_t)(r - lo);
-        if (rr < width) {
-          const int cc = compact_index(sm, rr >> 5);
-          const uint32_t bit = 1u << (rr & 31);
-          if (cc < ne && !(sm.cw[cc] & bit)) atomicOr(&sm.cw[cc], bit);
+    if (t == nsl - 1 && nib == 1 && next) F = next_bounds();  // used when the next item starts
+    if (flat) {
+      const uint4* own = reinterpret_cast<const uint4*>(bits + pad_word(tid * per));
+      int loc = 0;
+      if (tid * per < nwords)
+        for (int x = 0; x < per / 4; ++x) {
+          const uint4 w = own[x];
+          loc += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
         }
-        return 0u;
-      };
-      block_for_each_entry<false, V, BLOCK, U>(in, k, off, seg, setbit, none, sc);
+      int run = item_scan<B>(loc, M.red[1], &slab_u);
+      fits = u_done + slab_u <= sm.umax && !bad;
+      if (tid * per < nwords)
+        for (int x = 0; x < per / 4; ++x) {
+          const uint4 w = own[x];
+          const int a1 = run + __popc(w.x), a2 = a1 + __popc(w.y), a3 = a2 + __popc(w.z);
+          uint2 p;
+          p.x = (uint32_t)run | ((uint32_t)a1 << 16);
+          p.y = (uint32_t)a2 | ((uint32_t)a3 << 16);
+          *reinterpret_cast<uint2*>(wpre + tid * per + 4 * x) = p;
+          run = a3 + __popc(w.w);
+        }
+    } else {
+      // Rank 1: thread t < 256 owns summary words [4t, 4t + 4) (1024 in all).
+      const bool sum4 = tid < 256;
+      uint4 w = make_uint4(0u, 0u, 0u, 0u);
+      if (sum4) w = *reinterpret_cast<const uint4*>(summ + 4 * tid);
+      const int n0 = __popc(w.x), n1 = __popc(w.y), n2 = __popc(w.z);
+      const int run1 = item_scan<B>(n0 + n1 + n2 + __popc(w.w), M.red[1], &ne);
+      uint2 p;
+      p.x = (uint32_t)run1 | ((uint32_t)(run1 + n0) << 16);
+      p.y = (uint32_t)(run1 + n0 + n1) | ((uint32_t)(run1 + n0 + n1 + n2) << 16);
+      if (sum4) *reinterpret_cast<uint2*>(spre + 4 * tid) = p;
       __syncthreads();
-      // Rank 2: thread t owns compact words [t*pc, t*pc + pc).
-      const int pc = (ne + BLOCK - 1) / BLOCK;
-      const int c0 = min(ne, (int)threadIdx.x * pc), c1 = min(ne, c0 + pc);
-      int rl = 0;
-      for (int cc = c0; cc < c1; ++cc) rl += __popc(sm.cw[cc]);
-      int rank = block_excl_scan<BLOCK>(rl, sm.red, &slab_u);
-      fits = u_done + slab_u <= sm.umax;
+      fits = ne <= sm.umax && !bad;
       if (fits) {
-        for (int cc = c0; cc < c1; ++cc) {
-          sm.wpre[cc] = (uint16_t)rank;
-          rank += __popc(sm.cw[cc]);
-        }
-        for (int q = threadIdx.x; q < slab_u; q += BLOCK) acc[q] = A(0);
-      } else {
-        bad = true;
+        rows_pass(false, [&]() {
+#pragma unroll
+          for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+            if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+            for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
+              const uint32_t c = min(r[q], wmax);
+              const int cc = compact(c);
+              if (r[q] <= wmax && cc < ne) atomicOr(&cw[cc], 1u << (c & 31));
+            }
+          }
+        });
+        __syncthreads();
+        const int pc = ne <= 4 * B ? 4 : (ne <= 8 * B ? 8 : 16);
+        int loc = 0;
+        for (int c = tid * pc; c < min(ne, tid * pc + pc); ++c) loc += __popc(cw[c]);
+        int run = item_scan<B>(loc, M.red[0], &slab_u);
+        fits = u_done + slab_u <= sm.umax;
+        if (fits)
+          for (int c = tid * pc; c < min(ne, tid * pc + pc); ++c) {
+            cpre[c] = (uint16_t)run;
+            run += __popc(cw[c]);
+          }
       }
-      __syncthreads();
     }
-    if (fits) {
-      // Pass B: values at their rank.
-      auto add = [&](int32_t r, V v) -> uint32_t {
-        const uint32_t rr = (uint32_t)(r - lo);
-        if (rr < width) {
-          const int cc = compact_index(sm, rr >> 5);
-          if (cc < ne) {
-            const uint32_t bits = sm.cw[cc], b = rr & 31;
-            const int q = (int)sm.wpre[cc] + __popc(bits & ((1u << b) - 1u));
-            if (((bits >> b) & 1u) && q < slab_u) atomicAdd(&acc[q], (A)v);
+    if (fits)
+      for (int q = tid; q < slab_u; q += B) acc[q] = A(0);
+    else
+      bad = true;
+    __syncthreads();
+    // Ranks past the symbolic count are never written (B holds W.u rows
+    // here); they can only arise if the inputs changed between the passes.
+    const int lim = min(slab_u, W.u - u_done);
+    int32_t* orow = out_row + u_done;
+    V* oval = out_val + u_done;
+    const bool phased = PHASED && s_ent - slab_u >= FP32_ACC_TERMS;
+    const bool by_entry = single && !phased;  // rows are written from r[]
+    if (fits && slab_u > 0) {
+      // Pass B.
+      for (int ib = 0; ib < nib; ++ib) {
+        const int nk = min(KT, k - ib * KT);
+        if (nib > 1) {
+          __syncthreads();
+          table(ib, false, M.red[1]);
+          __syncthreads();
+        }
+        const int nph = phased ? (nk + FP32_PHASE_INPUTS - 1) / FP32_PHASE_INPUTS : 1;
+        for (int ph = 0; ph < nph; ++ph) {
+          const int e_lo = phased ? M.phase[ph] : 0;
+          const int e_hi = phased && ph + 1 < nph ? M.phase[ph + 1] : total;
+          for (int c0 = 0; e_lo < e_hi; c0 += CAP) {
+            if (c0 + (CAP - 1) >= e_lo) {
+              if (!single) {
+                item_map(M, c0);
+                __syncthreads();
+                L.init(c0, total);
+                item_rows(M, L, c0, r);
+                relative();
+              }
+#pragma unroll
+              for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+                if (q0 >= L.ns) break;  // (warp-uniform)
+                uint32_t rank[ITEM_GROUP];
+                V v[ITEM_GROUP];
+#pragma unroll
+                for (int x = 0; x < ITEM_GROUP; ++x)
+                  v[x] = __ldg(reinterpret_cast<const V*>(M.seg[item_seg(M, L, q0 + x)].y) + (c0 + L.pos(q0 + x)));
+#pragma unroll
+                for (int x = 0; x < ITEM_GROUP; ++x) {
+                  const int q = q0 + x;
+                  const uint32_t c = min(r[q], wmax);
+                  uint32_t wbits;
+                  int base;
+                  if (flat) {
+                    wbits = bits[pad_word((int)(c >> 5))];
+                    base = wpre[c >> 5];
+                  } else {
+                    const int cc = min(ne - 1, compact(c));
+                    wbits = cw[cc];
+                    base = cpre[cc];
+                  }
+                  rank[x] = (uint32_t)(base + __popc(wbits & ((1u << (c & 31)) - 1u)));
+                  if (r[q] > wmax) rank[x] = 0xffffffffu;
+                  // Row and rank together (20 + 12 bits) for the rows' write below.
+                  if (by_entry) r[q] = r[q] <= wmax ? c | (rank[x] << 20) : 0xffffffffu;
+                  bool ok = L.live(q);
+                  if (PHASED && phased) {
+                    const int e = c0 + L.run + 32 * q + (tid & 31);
+                    ok = ok && e >= e_lo && e < e_hi;
+                  }
+                  if (!ok) rank[x] = 0xffffffffu;
+                }
+#pragma unroll
+                for (int x = 0; x < ITEM_GROUP; ++x)
+                  if (rank[x] < (uint32_t)slab_u) atomicAdd(&acc[rank[x]], (A)v[x]);
+              }
+              if (!single) {
+                __syncthreads();
+                item_unmap(M);
+                __syncthreads();
+              }
+            }
+            if (single || e_hi - c0 <= CAP) break;
+          }
+          if (phased) {
+            // The phase's sums join B's values (the first phase stores them).
+            __syncthreads();
+            for (int q = tid; q < slab_u; q += B) {
+              if (q < lim) oval[q] = ib + ph == 0 ? (V)acc[q] : oval[q] + (V)acc[q];
+              acc[q] = A(0);
+            }
+            __syncthreads();
           }
         }
-        return 0u;
-      };
-      // Ranks past the symbolic count are never written (B holds W.u rows here).
-      const bool written = add_values<V, A, PHASED, BLOCK, U>(in, k, off, seg, add, sc, acc, out_val + u_done, slab_u,
-                                                              min(slab_u, W.u - u_done), s_ent);
-      __syncthreads();
-      // Values copied out first; then the rows, expanded from the words into
-      // the accumulator's slots (free once the values are out; a word's rows
-      // go to consecutive ranks), so that both are written coalesced.
-      const int lim = min(slab_u, W.u - u_done);
-      int32_t* orow = out_row + u_done;
-      V* oval = out_val + u_done;
-      if (!written)
-        for (int q = threadIdx.x; q < lim; q += BLOCK) oval[q] = (V)acc[q];
-      __syncthreads();
-      int32_t* rows = reinterpret_cast<int32_t*>(acc);  // slab_u <= umax slots of at least 4 bytes
-      for (int cc = threadIdx.x; cc < ne; cc += BLOCK) {
-        int q = sm.wpre[cc];
-        const int rbase = lo + ((int)sm.nel[cc] << 5);
-        for (uint32_t bits = sm.cw[cc]; bits; bits &= bits - 1) rows[q++] = rbase + __ffs(bits) - 1;
       }
       __syncthreads();
-      for (int q = threadIdx.x; q < lim; q += BLOCK) orow[q] = rows[q];
-      u_done += slab_u;
+      if (!phased)
+        for (int q = tid; q < lim; q += B) oval[q] = (V)acc[q];
+      // The non-empty words in row order, in the segment table's place (free now).
+      uint16_t* nel = reinterpret_cast<uint16_t*>(M.seg);
+      if (!flat && !by_entry && tid < 256) {
+        const uint4 w4 = *reinterpret_cast<const uint4*>(summ + 4 * tid);
+        int c = spre[4 * tid];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          for (uint32_t wb = x == 0 ? w4.x : x == 1 ? w4.y : x == 2 ? w4.z : w4.w; wb; wb &= wb - 1)
+            nel[c++] = (uint16_t)((4 * tid + x) * 32 + __ffs(wb) - 1);
+      }
       __syncthreads();
+      int32_t* rows = reinterpret_cast<int32_t*>(acc);  // slab_u <= umax slots of at least 4 bytes
+      if (by_entry) {
+        // Every entry writes its row at its rank (equal rows write the same).
+        // All ones marks a slot without a row; its rank, 4095, is below slab_u
+        // only for a whole column of 4096 rows, where every entry has one.
+#pragma unroll
+        for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+          if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+          for (int q = q0; q < q0 + ITEM_GROUP; ++q)
+            if ((r[q] >> 20) < (uint32_t)slab_u) rows[r[q] >> 20] = lo + (int)(r[q] & 0xfffffu);
+        }
+      } else if (flat) {
+        for (int w = tid; w < nwords; w += B) {
+          int q = wpre[w];
+          for (uint32_t wb = bits[pad_word(w)]; wb; wb &= wb - 1) rows[q++] = lo + (w << 5) + __ffs(wb) - 1;
+        }
+      } else {
+        for (int c = tid; c < ne; c += B) {
+          int q = cpre[c];
+          const int rbase = lo + ((int)nel[c] << 5);
+          for (uint32_t wb = cw[c]; wb; wb &= wb - 1) rows[q++] = rbase + __ffs(wb) - 1;
+        }
+      }
+      item_unmap(M);
+      __syncthreads();
+      for (int q = tid; q < lim; q += B) orow[q] = rows[q];
+      u_done += slab_u;
+    } else {
+      item_unmap(M);
     }
-    // Clear the compact words, then this thread's summary words.
-    if (ne_fits)
-      for (int cc = threadIdx.x; cc < ne; cc += BLOCK) sm.cw[cc] = 0u;
-    for (int x = x0; x < x1; ++x) sm.summ[x] = 0u;
-    __syncthreads();
+    // Zero words again, each thread its own (every reader is past the last barrier).
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    if (flat) {
+      uint4* mine = reinterpret_cast<uint4*>(bits + pad_word(tid * per));
+      if (tid * per < nwords)
+        for (int x = 0; x < per / 4; ++x) mine[x] = z;
+    } else {
+      if (tid < 256) *reinterpret_cast<uint4*>(summ + 4 * tid) = z;
+      for (int c = tid; c < min(ne, sm.umax); c += B) cw[c] = 0u;
+    }
+    // (The next slab's or item's table has two barriers before anything here is reused.)
   }
-  if (threadIdx.x == 0 && (bad || u_done != W.u)) atomicOr(&ctr_w->err, ERR_INTERNAL);
+  if (next && k > KT) F = next_bounds();  // (tables of more inputs go through F)
+  if (tid == 0 && (bad || u_done != W.u)) atomicOr(&ctr_w->err, ERR_INTERNAL);
 }
 
-template <int DT, int ACC, int BLOCK, int U>
-__global__ void __launch_bounds__(BLOCK, (DT == 0 && ACC == 0) ? 0 : 3) k_num_compact(Inputs in, const Window* __restrict__ win, int nwin,
-                                                       const int32_t* __restrict__ offs,
-                                                       const int64_t* __restrict__ col_ptr, Outs o, int slab_log2,
-                                                       int umax, int only_dtype, Counters* ctr_w) {
+// DT: 0 = float values, 1 = double values; ACC: 0 sums in the value type, 1
+// float sums in phases, 2 float values summed in double.  B: threads per block,
+// 256 for CTA-class columns (at most 4096 entries: one chunk, four blocks per
+// SM), 384 for the windows of heavy columns (window_max distinct rows, mostly
+// under 6144 entries; 512 threads measured 808 against 750 us on 96 columns of
+// 480,000 entries, since more warps run with part of their slots).
+constexpr int CTA_ITEM_BLOCK = 256, HEAVY_ITEM_BLOCK = 384;
+
+template <int DT, int ACC, bool WIDE, int B>
+__global__ void __launch_bounds__(B, B == CTA_ITEM_BLOCK ? 4 : 2)
+    k_num_items(Inputs in, const Window* __restrict__ win, int nwin, const int32_t* __restrict__ offs,
+                const int64_t* __restrict__ col_ptr, Outs o, int slab_log2, int umax, int flat_rows, int only_dtype,
+                Counters* ctr_w) {
   using V = typename std::conditional<DT == 1, double, float>::type;
   using A = typename std::conditional<DT == 1 || ACC == 2, double, float>::type;  // accumulator
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  __shared__ int red[BLOCK / 32 + 1];
-  CompactSmem sm;
-  sm.NSW = 1 << (slab_log2 - 10);
+  const ItemLayout<WIDE, B> L(slab_log2, umax, (int)sizeof(A));
+  ItemSmem<B> sm;
   sm.umax = umax;
   sm.acc = sm_raw;
-  sm.summ = reinterpret_cast<uint32_t*>(sm.acc + (size_t)umax * sizeof(A));
-  sm.cw = sm.summ + sm.NSW;
-  sm.spre = reinterpret_cast<uint16_t*>(sm.cw + umax);
-  sm.wpre = sm.spre + sm.NSW;
-  sm.nel = sm.wpre + umax;
-  sm.red = red;
-  for (int x = threadIdx.x; x < sm.NSW; x += BLOCK) sm.summ[x] = 0u;
-  for (int x = threadIdx.x; x < umax; x += BLOCK) sm.cw[x] = 0u;
+  sm.zero = reinterpret_cast<uint32_t*>(sm.acc + L.acc);
+  sm.pre = reinterpret_cast<uint16_t*>(sm.zero + L.zero);
+  sm.map = reinterpret_cast<ItemMap<B>*>(reinterpret_cast<unsigned char*>(sm.pre) + L.pre);
+  sm.win = reinterpret_cast<Window*>(sm.map + 1);
+  for (int x = threadIdx.x; x < L.zero; x += B) sm.zero[x] = 0u;
+  item_unmap(*sm.map);
+  // While an item runs, the next one's record and segment bounds are on their
+  // way.  (The item filter only checks: every record belongs to this launch.)
+  const int step = gridDim.x;
+  int wi = blockIdx.x;
+  if (wi >= nwin) return;
+  if (threadIdx.x < sizeof(Window) / 4)
+    reinterpret_cast<int32_t*>(sm.win)[threadIdx.x] = reinterpret_cast<const int32_t*>(win + wi)[threadIdx.x];
   __syncthreads();
-  Window Wn{};
-  if (blockIdx.x < nwin) Wn = win[blockIdx.x];
-  for (int wi = blockIdx.x; wi < nwin; wi += gridDim.x) {
-    const Window W = Wn;
-    if (wi + (int)gridDim.x < nwin) Wn = win[wi + gridDim.x];
+  ItemBounds<B> F;
+  {
+    const Window& W = sm.win[0];
+    const Inst* I = in.inst + inst_of(in, W.col);
+    const int j = W.col - I->colbase, off = I->ptr_off;
+    auto seg = [&](int i, int* beg, int* end) { window_seg(in, W, offs, off, j, i, beg, end); };
+    F = item_bounds<B>(0, min(I->k, ItemMap<B>::KT), seg);
+  }
+  for (int turn = 0;; turn ^= 1) {
+    const Window& W = sm.win[turn];
     const int q = inst_of(in, W.col);
     const Inst* I = in.inst + q;
-    if (only_dtype >= 0 && !item_selected(only_dtype, I)) continue;
+    if ((only_dtype >= 0 && !item_selected(only_dtype, I)) || W.r_hi <= W.r_lo) {  // (cannot happen)
+      if (threadIdx.x == 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
+      return;
+    }
     const int64_t out = col_ptr[W.col] - (in.col_inst ? col_ptr[I->colbase] : 0) + W.out_off;
-    compact_item<V, A, ACC == 1, BLOCK, U>(in, W, I, offs, out_row_of(o, q) + out, static_cast<V*>(out_val_of(o, q)) + out, sm,
-                              slab_log2, ctr_w);
+    const bool more = wi + step < nwin;
+    reg_item<V, A, ACC == 1, WIDE, B>(in, more ? win + wi + step : nullptr, turn, F, offs, out_row_of(o, q) + out,
+                                      static_cast<V*>(out_val_of(o, q)) + out, sm, slab_log2, flat_rows, ctr_w);
+    if (!more) break;
+    wi += step;
   }
 }
 
@@ -582,12 +851,6 @@ static size_t bitmap_smem_bytes(int slab_log2, int umax, size_t vsize) {
          (size_t)umax * 2 + 16;
 }
 
-// Shared bytes of the compact-table kernel.
-static size_t compact_smem_bytes(int slab_log2, int umax, size_t vsize) {
-  const size_t nsw = (size_t)1 << (slab_log2 - 10);
-  return (size_t)umax * vsize + nsw * 4 + (size_t)umax * 4 + nsw * 2 + (size_t)umax * 4 + 16;
-}
-
 template <typename K>
 static cudaError_t launch_items(K kern, int block, int blocks_per_sm, const Inputs& in, const Window* win, int n_win,
                                 const int32_t* offs, const int64_t* col_ptr, const Outs& out, int slab_log2, int umax,
@@ -602,95 +865,100 @@ static cudaError_t launch_items(K kern, int block, int blocks_per_sm, const Inpu
   return cudaGetLastError();
 }
 
-// accumulator: 0 = automatic, 1 = flat bitmap, 2 = compact word table.
-// Automatic takes the compact table when more of its blocks are resident per
-// SM (the flat bitmap's size follows the slab, the table's follows umax):
-// items are latency chains, so items in flight per SM decide the rate.
+template <int DT, int ACC, bool WIDE, int B>
+static cudaError_t launch_reg_items(const Inputs& in, const Window* win, int n_win, const int32_t* offs,
+                                    const int64_t* col_ptr, const Outs& out, int slab_log2, int umax, int flat_rows,
+                                    int only_dtype, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
+  auto kern = k_num_items<DT, ACC, WIDE, B>;
+  const size_t smem = ItemLayout<WIDE, B>(slab_log2, umax, (DT == 1 || ACC == 2) ? 8 : 4).bytes();
+  const int bps = resident_blocks((const void*)kern, B, smem);
+  if (bps < 1) return cudaErrorInvalidConfiguration;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int grid = dev.sms * bps;
+  if (grid > n_win) grid = n_win;
+  if (grid < 1) return cudaSuccess;
+  kern<<<grid, B, smem, st>>>(in, win, n_win, offs, col_ptr, out, slab_log2, umax, flat_rows, only_dtype, ctr_w);
+  return cudaGetLastError();
+}
+
+// accumulator: 0 = automatic (slabs of at most FLAT_ROWS rows flat, larger
+// ones compact), 1 = flat bitmap, 2 = compact word table.  A flat bitmap of
+// more than FLAT_ROWS rows fills the SM: one 1024-thread block.
 template <int DT, int ACC>
-static cudaError_t launch_num_cta_t(const Inputs& in, const Window* win, int n_win, const int32_t* offs,
+static cudaError_t launch_num_cta_t(const Inputs& in, const Window* win, int n_win, bool heavy, const int32_t* offs,
                                     const int64_t* col_ptr, const Outs& out, int umax, int accumulator,
                                     int only_dtype, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
   constexpr size_t VS = (DT == 1 || ACC == 2) ? 8 : 4;  // accumulator bytes
   int slab_log2 = 10;
   while (slab_log2 < NUM_SLAB_LOG2_MAX && ((int64_t)1 << slab_log2) < (int64_t)in.mmax) ++slab_log2;
-  const size_t sf = bitmap_smem_bytes(slab_log2, umax, VS), sc = compact_smem_bytes(slab_log2, umax, VS);
-  // Small bitmaps leave room for several blocks per SM: 256 threads each
-  // (measured best, with 8 entries per lane and round); a bitmap that fills
-  // the SM gets one 1024-thread block.
-  const bool small = sf <= (size_t)dev.smem_per_sm / 2 - 2048;
-  const void* kf = small ? (const void*)k_num_bitmap<DT, ACC, 256, 8> : (const void*)k_num_bitmap<DT, ACC, 1024, 4>;
-  const void* kc = (const void*)k_num_compact<DT, ACC, 256, 8>;
-  int bf = 0, bc = 0;
-  if (accumulator != 2 && sf <= (size_t)dev.smem_optin) bf = resident_blocks(kf, small ? 256 : 1024, sf);
-  if (accumulator != 1 && sc <= (size_t)dev.smem_optin) bc = resident_blocks(kc, 256, sc);
-  const bool compact = accumulator == 2 || (accumulator == 0 && bc > bf);
-  if (compact)
-    return launch_items(k_num_compact<DT, ACC, 256, 8>, 256, bc, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sc,
-                        only_dtype, ctr_w, dev, st);
-  if (small)
-    return launch_items(k_num_bitmap<DT, ACC, 256, 8>, 256, bf, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sf,
-                        only_dtype, ctr_w, dev, st);
-  return launch_items(k_num_bitmap<DT, ACC, 1024, 4>, 1024, bf, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sf,
-                      only_dtype, ctr_w, dev, st);
+  if (accumulator == 1 && slab_log2 > FLAT_LOG2) {
+    const size_t sf = bitmap_smem_bytes(slab_log2, umax, VS);
+    auto kern = k_num_bitmap<DT, ACC, 1024, 4>;
+    const int bf = sf <= (size_t)dev.smem_optin ? resident_blocks((const void*)kern, 1024, sf) : 0;
+    return launch_items(kern, 1024, bf, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sf, only_dtype, ctr_w,
+                        dev, st);
+  }
+  const bool wide = accumulator == 2 || slab_log2 > FLAT_LOG2;
+  const int flat_rows = accumulator == 2 ? 0 : FLAT_ROWS;
+  auto launch = heavy ? (wide ? launch_reg_items<DT, ACC, true, HEAVY_ITEM_BLOCK>
+                              : launch_reg_items<DT, ACC, false, HEAVY_ITEM_BLOCK>)
+                      : (wide ? launch_reg_items<DT, ACC, true, CTA_ITEM_BLOCK>
+                              : launch_reg_items<DT, ACC, false, CTA_ITEM_BLOCK>);
+  return launch(in, win, n_win, offs, col_ptr, out, slab_log2, umax, flat_rows, only_dtype, ctr_w, dev, st);
 }
 
 // Batches of several problem kinds: after the symbolic phase the
-// thread-block items' records are copied, grouped by kind (count, then place
-// with warp-aggregated appends; order inside a kind is arbitrary), so that
-// each kind's numeric launch reads only its own items.  The windows counted
-// by the symbolic kernels are read from the counters (at most `cap`).
+// thread-block items' records are copied, grouped by class (CTA, then heavy)
+// and kind (count, then place with warp-aggregated appends; order inside a
+// group is arbitrary), so that each numeric launch reads only its own items.
+// The numbers of records are read from the counters (at most `cap` in all).
+__device__ __forceinline__ int record_group(const Inputs& in, const Window* win, int cap, int n_cta, int x,
+                                            Window* W) {
+  *W = x < n_cta ? win[x] : win[cap - 1 - (x - n_cta)];
+  return item_kind(in.inst + inst_of(in, W->col)) + (x < n_cta ? 0 : 4);
+}
+
 __global__ void k_kind_count(Inputs in, const Window* __restrict__ win, int cap, Counters* ctr_w) {
-  const int nwin = min(ctr_w->n_windows, cap);
-  int c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-  for (int wi = blockIdx.x * blockDim.x + threadIdx.x; wi < nwin; wi += gridDim.x * blockDim.x) {
-    const int kd = item_kind(in.inst + inst_of(in, win[wi].col));
-    c0 += kd == 0;
-    c1 += kd == 1;
-    c2 += kd == 2;
-    c3 += kd == 3;
-  }
-  c0 = warp_sum(c0);
-  c1 = warp_sum(c1);
-  c2 = warp_sum(c2);
-  c3 = warp_sum(c3);
-  if ((threadIdx.x & 31) == 0) {
-    if (c0) atomicAdd(&ctr_w->kind_n[0], c0);
-    if (c1) atomicAdd(&ctr_w->kind_n[1], c1);
-    if (c2) atomicAdd(&ctr_w->kind_n[2], c2);
-    if (c3) atomicAdd(&ctr_w->kind_n[3], c3);
+  const int n_cta = min(ctr_w->n_windows, cap), nwin = min(n_cta + ctr_w->n_hwin, cap);
+  const int stride = gridDim.x * blockDim.x;
+  for (int w0 = blockIdx.x * blockDim.x; w0 < nwin; w0 += stride) {  // (block-uniform)
+    const int x = w0 + (int)threadIdx.x;
+    Window W;
+    const int grp = x < nwin ? record_group(in, win, cap, n_cta, x, &W) : -1;
+    for (int q = 0; q < 8; ++q) {
+      const unsigned m = __ballot_sync(SPK_FULL, grp == q);
+      if (m && (threadIdx.x & 31) == 0) atomicAdd(&ctr_w->kind_n[q], __popc(m));
+    }
   }
 }
 
 __global__ void k_kind_place(Inputs in, const Window* __restrict__ win, int cap, Window* __restrict__ wsort,
                              Counters* ctr_w) {
-  __shared__ int base[4];
+  __shared__ int base[8];
   if (threadIdx.x == 0) {
     int b = 0;
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 8; ++q) {
       base[q] = b;
       b += ctr_w->kind_n[q];
     }
   }
   __syncthreads();
-  const int nwin = min(ctr_w->n_windows, cap);
+  const int n_cta = min(ctr_w->n_windows, cap), nwin = min(n_cta + ctr_w->n_hwin, cap);
   const int lane = threadIdx.x & 31;
   const int stride = gridDim.x * blockDim.x;
   for (int w0 = blockIdx.x * blockDim.x; w0 < nwin; w0 += stride) {  // (block-uniform)
-    const int wi = w0 + (int)threadIdx.x;
+    const int x = w0 + (int)threadIdx.x;
     Window W{};
-    int kd = -1;
-    if (wi < nwin) {
-      W = win[wi];
-      kd = item_kind(in.inst + inst_of(in, W.col));
-    }
-    for (int q = 0; q < 4; ++q) {
-      const unsigned m = __ballot_sync(SPK_FULL, kd == q);
+    const int grp = x < nwin ? record_group(in, win, cap, n_cta, x, &W) : -1;
+    for (int q = 0; q < 8; ++q) {
+      const unsigned m = __ballot_sync(SPK_FULL, grp == q);
       if (!m) continue;
       const int leader = __ffs(m) - 1;
       int pos = 0;
       if (lane == leader) pos = atomicAdd(&ctr_w->kind_fill[q], __popc(m));
       pos = __shfl_sync(SPK_FULL, pos, leader);
-      if (kd == q) wsort[base[q] + pos + __popc(m & ((1u << lane) - 1u))] = W;
+      if (grp == q) wsort[base[q] + pos + __popc(m & ((1u << lane) - 1u))] = W;
     }
   }
 }
@@ -700,7 +968,7 @@ int num_cta_kinds(int dt, int f32_kinds) { return (dt != 1 ? (f32_kinds & 7) : 0
 cudaError_t launch_kind_sort(const Inputs& in, const Window* win, int cap, Window* wsort, Counters* ctr_w,
                              const DeviceInfo& dev, cudaStream_t st) {
   if (cap <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(&ctr_w->kind_n[0], 0, 8 * sizeof(int32_t), st);  // kind_n, kind_fill
+  cudaError_t e = cudaMemsetAsync(&ctr_w->kind_n[0], 0, 16 * sizeof(int32_t), st);  // kind_n, kind_fill
   if (e != cudaSuccess) return e;
   int blocks = (cap + 255) / 256;
   if (blocks > dev.sms * 8) blocks = dev.sms * 8;
@@ -709,35 +977,36 @@ cudaError_t launch_kind_sort(const Inputs& in, const Window* win, int cap, Windo
   return cudaGetLastError();
 }
 
-cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int n_win,
-                           const Window* wsort, const int32_t* kind_n, const int32_t* offs, const int64_t* col_ptr,
-                           const Outs& out, int window_max, int accumulator, Counters* ctr_w, const DeviceInfo& dev,
-                           cudaStream_t st, int* launches) {
+cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int64_t win_cap, int n_cta,
+                           int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
+                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
+                           const DeviceInfo& dev, cudaStream_t st, int* launches) {
   *launches = 0;
-  if (n_win <= 0) return cudaSuccess;
+  if (n_cta + n_heavy <= 0) return cudaSuccess;
   // Float problems: k <= FP32_ACC_TERMS sum in float, up to
   // FP32_PHASED_MAX_K in float by phases, beyond in double; each kind that
-  // the batch holds gets its own launch, over its own group of the records
+  // the batch holds gets its own launches, over its own groups of the records
   // (the item filter of kind q, sel[q], only checks that).
   const int kinds = num_cta_kinds(dt, f32_kinds);
   const bool alone = __builtin_popcount(kinds) == 1;
   constexpr int sel[4] = {2, 3, 4, 1};
   int base = 0;
   cudaError_t e = cudaSuccess;
-  for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+  for (int g = 0; g < 8 && e == cudaSuccess; ++g) {
+    const int q = g & 3;
+    const bool heavy = g >= 4;
     if (!((kinds >> q) & 1)) continue;
-    const Window* w = alone ? win : wsort + base;
-    const int n = alone ? n_win : kind_n[q];
-    base += alone ? 0 : kind_n[q];
+    // A batch of one kind: its records where the symbolic phase left them
+    // (CTA-class from the array's start, heavy at its end).
+    const Window* w = alone ? (heavy ? win + (win_cap - n_heavy) : win) : wsort + base;
+    const int n = alone ? (heavy ? n_heavy : n_cta) : kind_n[g];
+    base += alone ? 0 : n;
     if (n <= 0) continue;
     ++*launches;
     const int f = alone ? -1 : sel[q];
-    switch (q) {
-      case 0: e = launch_num_cta_t<0, 0>(in, w, n, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st); break;
-      case 1: e = launch_num_cta_t<0, 1>(in, w, n, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st); break;
-      case 2: e = launch_num_cta_t<0, 2>(in, w, n, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st); break;
-      default: e = launch_num_cta_t<1, 0>(in, w, n, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st);
-    }
+    auto launch = q == 0 ? launch_num_cta_t<0, 0> : q == 1 ? launch_num_cta_t<0, 1>
+                  : q == 2 ? launch_num_cta_t<0, 2> : launch_num_cta_t<1, 0>;
+    e = launch(in, w, n, heavy, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st);
   }
   return e;
 }

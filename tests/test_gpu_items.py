@@ -1,0 +1,74 @@
+"""Thread-block items in registers: the sizes where their chunks, slots, segment tables and layouts end.
+
+Small-integer values: indices and sums must match the oracle exactly in either type.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2112_10223_gb300 as spk
+from spk_testlib import check_full
+
+pytestmark = pytest.mark.gpu
+
+
+def _columns(k, m, lengths, seed, dtype, pool=None):
+    """k inputs; column j has lengths[j] entries dealt to the inputs at random (some inputs get none),
+    from the first pool[j] rows of a random row order when given (repeats across inputs)."""
+    r = np.random.default_rng(seed)
+    n = len(lengths)
+    cols = [[] for _ in range(k)]
+    for j, s in enumerate(lengths):
+        owner = np.sort(r.integers(0, k, s))
+        rows = np.empty(s, dtype=np.int64)
+        cand = None if pool is None else r.choice(m, pool[j], replace=False)
+        for i in np.unique(owner):
+            at = owner == i
+            c = int(at.sum())
+            src = m if cand is None else cand
+            rows[at] = np.sort(r.choice(src, c, replace=False))
+        for i in range(k):
+            cols[i].append(rows[owner == i])
+    out = []
+    for i in range(k):
+        cp = np.zeros(n + 1, dtype=np.int32)
+        cp[1:] = np.cumsum([len(c) for c in cols[i]])
+        ri = np.concatenate(cols[i]).astype(np.int32) if cp[-1] else np.zeros(0, np.int32)
+        va = r.integers(-8, 9, ri.size)
+        out.append((torch.from_numpy(cp), torch.from_numpy(ri), torch.from_numpy(va).to(dtype)))
+    return out
+
+
+# 256 threads of 16 slots hold 4096 entries, 384 hold 6144; slots come in pairs.
+LENGTHS = [1, 255, 256, 257, 511, 513, 1023, 1025, 4095, 4096, 4097, 6143, 6144, 6145, 8193, 12289]
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("m", [5000, 1 << 17, (1 << 17) + 1, 1 << 20, (1 << 20) + 77])
+def test_chunk_and_slot_edges(m, dtype):
+    pool = [min(m, max(s // 3, 40)) for s in LENGTHS]
+    A = _columns(37, m, LENGTHS, 1, dtype, pool) if m == 5000 else _columns(37, m, LENGTHS, 1, dtype)
+    for opt in (None, spk.default_options(warp_max=32, block_accumulator=2),
+                spk.default_options(warp_max=32, input_order=1)):
+        check_full(A, m, dtype, exact=True, options=opt)
+
+
+@pytest.mark.parametrize("k", [1, 2, 63, 64, 65, 255, 256, 257, 511, 512, 513, 1100])
+def test_segment_table_edges(k):
+    """Tables hold 512 inputs; sums of more than 167 inputs go in phases of 128 (float)."""
+    lengths = [600, 1500, 3000, 5000, 9000]
+    lengths = [min(s, 400 * k) for s in lengths]
+    for dtype in (torch.float32, torch.float64):
+        A = _columns(k, 3001, lengths, k, dtype, [min(3001, max(500, s // 2)) for s in lengths])
+        check_full(A, 3001, dtype, exact=True, options=spk.default_options(warp_max=64, cta_max=2048))
+
+
+def test_few_distinct_rows_many_terms():
+    """Items whose entries meet on a handful of rows, and whole columns of 4096 distinct rows."""
+    A = _columns(300, 4096, [1000, 4000, 20000], 3, torch.float32, [40, 90, 400])
+    check_full(A, 4096, torch.float32, exact=True)
+    r = torch.arange(4096, dtype=torch.int32)
+    full = [(torch.tensor([0, 4096], dtype=torch.int32), r + 7, torch.ones(4096, dtype=torch.float64))]
+    check_full(full, 5000, torch.float64, exact=True)
+    check_full([(full[0][0], r, full[0][2])], 4096, torch.float64, exact=True)
+    check_full([(full[0][0], r + ((1 << 20) - 4096), full[0][2])], 1 << 20, torch.float64, exact=True)
