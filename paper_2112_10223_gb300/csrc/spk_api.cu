@@ -377,6 +377,12 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   h->in.kmax = kmax;
   h->in.mmax = (int32_t)mmax;
   h->in.sorted = o.input_order == 0 ? 1 : 0;
+  // Uniform rows repeat about s^2 / 2m times in a column of s entries: few
+  // enough for the warp columns' filter while s^2 <= m / 2 (s: the mean; columns
+  // of more than 256 entries are not to be expected far above a mean below 64).
+  const double mean_s = ncols > 0 ? (double)nnz_in / (double)ncols : 0.0;
+  h->in.mean_s = (int32_t)(mean_s < 2e9 ? mean_s : 2e9);
+  h->in.split_warp = mean_s >= 64.0 && mean_s * mean_s <= 0.5 * (double)mmax;
   if (multi) {
     ce = spk::launch_col_inst(h->in, h->d_col_inst, h->dev.sms, h->st);
     h->launches += 1;
@@ -434,6 +440,7 @@ SPK_API spkadd_status spkadd_batch_plan(spkadd_handle** hp, int count, const int
 // h->nnz_each.
 static spkadd_status run_symbolic(spkadd_handle* h) {
   cudaError_t ce = cudaSuccess;
+  int warp_launches = 0;
   if (h->ncols > 0) {
     ce = spk::launch_sym_heavy(h->in, h->d_hl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->d_search, h->win_cap, h->d_ctr,
                                h->opt.window_max, h->opt.block_accumulator, h->dev, h->st);
@@ -441,9 +448,9 @@ static spkadd_status run_symbolic(spkadd_handle* h) {
       ce = spk::launch_sym_cta(h->in, h->d_cl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->win_cap, h->d_ctr,
                                h->opt.cta_max, h->dev, h->st);
     if (ce == cudaSuccess)
-      ce = spk::launch_sym_warp(h->in, h->d_wl, h->d_s, h->d_ctr, h->d_u, h->opt.warp_max, h->d_ctr, h->dev,
-                                h->st);
-    h->launches += 3;
+      ce = spk::launch_sym_warp(h->in, h->d_wl, h->d_s, h->d_ctr, h->d_u, h->opt.warp_max, h->d_ctr, h->dev, h->st,
+                                &warp_launches);
+    h->launches += 2 + warp_launches;
     // Several problem kinds: the thread-block items grouped by kind for the numeric launches.
     if (ce == cudaSuccess && h->d_wsort) {
       ce = spk::launch_kind_sort(h->in, h->d_win, (int)h->win_cap, h->d_wsort, h->d_ctr, h->dev, h->st);
@@ -518,7 +525,7 @@ SPK_API spkadd_status spkadd_batch_symbolic(spkadd_handle* h, int64_t* nnz_B) {
 // The numeric kernels of every problem, writing through `out`.
 static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
   cudaError_t ce = cudaSuccess;
-  int item_launches = 0;
+  int item_launches = 0, warp_launches = 0;
   if (h->h_ctr.n_windows + h->h_ctr.n_hwin > 0)
     ce = spk::launch_num_cta(h->in, h->dt_mode, h->f32_kinds, h->d_win, h->win_cap, h->h_ctr.n_windows,
                              h->h_ctr.n_hwin, h->d_wsort, h->h_ctr.kind_n,
@@ -526,10 +533,11 @@ static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
                              h->opt.window_max > h->opt.cta_max ? h->opt.window_max : h->opt.cta_max,
                              h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
   h->launches += item_launches;
-  if (ce == cudaSuccess && h->h_ctr.n_warp > 0)
-    ce = spk::launch_num_warp(h->in, h->dt_mode, h->d_wl, h->d_ctr, h->h_ctr.n_warp, h->d_s, h->d_u, h->d_colptr,
-                              out, h->opt.warp_max, h->opt.sort_mode, h->d_ctr, h->dev, h->st);
-  h->launches += (h->h_ctr.n_warp > 0) * (h->dt_mode == 2 ? 2 : 1);
+  if (ce == cudaSuccess && h->h_ctr.n_warp + h->h_ctr.n_wbig > 0)
+    ce = spk::launch_num_warp(h->in, h->dt_mode, h->d_wl, h->d_ctr, h->h_ctr.n_warp, h->h_ctr.n_wbig,
+                              h->h_ctr.n_bucket, h->d_s, h->d_u, h->d_colptr, out, h->opt.warp_max, h->opt.sort_mode, h->d_ctr, h->dev, h->st,
+                              &warp_launches);
+  h->launches += warp_launches;
   return from_cuda(ce);
 }
 
@@ -583,7 +591,7 @@ SPK_API spkadd_status spkadd_onepass(spkadd_handle* h, int64_t* B_col_ptr, int32
   int grid = 0;
   ce = cudaMemsetAsync(&h->d_ctr->n_unique, 0, sizeof(int32_t), h->st);
   if (ce != cudaSuccess) return from_cuda(ce);
-  ce = spk::launch_onepass(h->in, h->dt_mode, h->d_s, (int)h->ncols, h->opt.warp_max, B_col_ptr,
+  ce = spk::launch_onepass(h->in, h->dt_mode, h->d_s, (int)h->ncols, h->opt.warp_max, c.max_warp_s, B_col_ptr,
                            B_row_idx, B_val, capacity, h->d_op, h->opt.sort_mode == 1, h->opt.test_stall,
                            (unsigned long long)h->opt.wait_timeout_ms * 1000000ull, h->d_ctr, h->dev, h->st, &grid);
   if (ce != cudaSuccess) return from_cuda(ce);
@@ -653,7 +661,7 @@ SPK_API spkadd_status spkadd_get_info(spkadd_handle* h, spkadd_info* info) {
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->st);
   if (ce != cudaSuccess) return from_cuda(ce);
   const Counters c = pb->ctr;
-  info->cols_warp = c.n_warp;
+  info->cols_warp = (int64_t)c.n_warp + c.n_wbig;
   info->cols_cta = c.n_cta;
   info->cols_heavy = (int64_t)c.n_heavy + c.n_big;
   info->windows = (int64_t)c.n_windows + c.n_hwin;

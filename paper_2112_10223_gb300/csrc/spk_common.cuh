@@ -34,7 +34,7 @@ struct Window {
 };
 
 struct Counters {
-  int32_t n_warp, n_cta, n_heavy;
+  int32_t n_warp, n_cta, n_heavy;  // (n_warp: columns of at most WARP_SMALL entries)
   int32_t n_windows;    // Window records of CTA-class columns, from the record array's start
   int32_t n_search;     // of those, split windows needing per-input offsets
   int32_t n_unique;     // warp columns whose input rows are all distinct (u_j == s_j)
@@ -44,7 +44,9 @@ struct Counters {
   int32_t n_hwin;       // Window records of heavy columns, from the record array's end
   int32_t kind_n[8];    // batches of several problem kinds: thread-block items per kind (CTA-class, then heavy)
   int32_t kind_fill[8]; //   and their placement counters
-  int32_t pad[2];
+  int32_t n_wbig;       // warp columns above WARP_SMALL entries, listed from the list's end
+  int32_t n_bucket;     // split warp columns whose values k_warp_col sums
+  int32_t max_warp_s;   // largest s_j of a warp column
 };
 
 // Float sums.  A float sum of t terms, in any order, errs by at most
@@ -67,6 +69,10 @@ static_assert((FP32_PHASE_INPUTS - 1) + (FP32_PHASED_MAX_K / FP32_PHASE_INPUTS -
               "phased float sums must stay within the float error bound");
 static_assert(FP32_PHASE_INPUTS % 32 == 0, "phases are whole 32-input chunks");
 
+
+// Warp columns above this summed input count are listed apart (from the list's
+// end): their 512 sort keys are other code, and k_warp_col may take them.
+constexpr int32_t WARP_SMALL = 256;
 
 // Heavy columns above this summed input count are listed apart and handed out
 // first (largest work first keeps one huge R-MAT column from finishing last).
@@ -94,6 +100,8 @@ struct Inputs {
   int32_t kmax;
   int32_t mmax;
   int32_t sorted;           // rows strictly increasing inside every input column
+  int32_t split_warp;       // warp columns above WARP_SMALL entries: few repeated rows expected
+  int32_t mean_s;           // entries per column, on average
 };
 
 __device__ __forceinline__ int inst_of(const Inputs& in, int g) { return in.col_inst ? __ldg(in.col_inst + g) : 0; }

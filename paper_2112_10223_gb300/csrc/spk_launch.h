@@ -44,7 +44,8 @@ cudaError_t launch_window_search(const Inputs& in, const Window* win, const int3
                                  int32_t* offs, int sms, cudaStream_t st);
 
 cudaError_t launch_sym_warp(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr,
-                            int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st);
+                            int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
+                            int* launches);
 cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
                            Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, const DeviceInfo& dev,
                            cudaStream_t st);
@@ -54,9 +55,12 @@ cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_
                              int accumulator, const DeviceInfo& dev, cudaStream_t st);
 
 // dt: 0 = every problem float, 1 = every problem double, 2 = mixed batch.
-cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const Counters* ctr, int n_cols,
+// Counters after the symbolic phase: n_small and n_big warp columns, n_bucket of these k_warp_col's where they are split.
+cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const Counters* ctr, int n_small, int n_big,
+                            int n_bucket,
                             const int32_t* s, const int32_t* u, const int64_t* col_ptr, const Outs& out,
-                            int warp_max, int sort_mode, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st);
+                            int warp_max, int sort_mode, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
+                            int* launches);
 // Problem kinds of the thread-block numeric launches present in a batch
 // (bit 0 float k <= FP32_ACC_TERMS, bit 1 float up to FP32_PHASED_MAX_K, bit 2
 // larger float, bit 3 double); f32_kinds holds bits 0-2 of the float problems.
@@ -85,7 +89,7 @@ cudaError_t launch_inst_nnz(const Inputs& in, const int64_t* col_ptr, int64_t* n
 // bytes (ticket counter and look-back words).
 int onepass_tile_cols();
 size_t onepass_scratch_bytes(int64_t ncols);
-cudaError_t launch_onepass(const Inputs& in, int dt, const int32_t* s, int n, int warp_max, int64_t* col_ptr,
+cudaError_t launch_onepass(const Inputs& in, int dt, const int32_t* s, int n, int warp_max, int max_s, int64_t* col_ptr,
                            int32_t* out_row, void* out_val, long long capacity, void* scratch, int force_dedup,
                            int debug_stall, unsigned long long wait_ns, Counters* ctr, const DeviceInfo& dev,
                            cudaStream_t st, int* grid_out);

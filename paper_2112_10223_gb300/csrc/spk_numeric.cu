@@ -828,7 +828,7 @@ int resident_blocks(const void* fn, int block, size_t smem) {
     int blocks;
   };
   static std::mutex mu;
-  static Entry cache[64];
+  static Entry cache[256];
   static int ncache = 0;
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < ncache; ++i)
@@ -839,7 +839,7 @@ int resident_blocks(const void* fn, int block, size_t smem) {
     (void)cudaGetLastError();  // not sticky: leave no stale error for the next check
     return 0;
   }
-  if (b > 0 && ncache < 64) cache[ncache++] = Entry{fn, block, smem, b};
+  if (b > 0 && ncache < 256) cache[ncache++] = Entry{fn, block, smem, b};
   return b;
 }
 

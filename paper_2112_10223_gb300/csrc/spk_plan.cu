@@ -18,10 +18,22 @@ __device__ __forceinline__ void warp_append(bool pred, int32_t* __restrict__ lis
   if (pred) list[base + __popc(m & ((1u << lane) - 1u))] = value;
 }
 
+// The same, from the end of a list: entry x at end[-1 - x].
+__device__ __forceinline__ void warp_append_back(bool pred, int32_t* __restrict__ end, int32_t* counter, int32_t value,
+                                                 int lane) {
+  const unsigned m = __ballot_sync(SPK_FULL, pred);
+  if (!m) return;
+  const int leader = __ffs(m) - 1;
+  int base = 0;
+  if (lane == leader) base = atomicAdd(counter, __popc(m));
+  base = __shfl_sync(SPK_FULL, base, leader);
+  if (pred) end[-1 - (base + __popc(m & ((1u << lane) - 1u)))] = value;
+}
+
 // a1 of the hot path: s_j = sum_i nnz(A_i(:,j)) and the column's class
 // (Sec. III-A: the symbolic phase balances load on the summed input count),
 // for every global column of every problem of the batch.
-__global__ void __launch_bounds__(256) k_bin(Inputs in, int warp_max, int cta_max, int32_t* __restrict__ s_out,
+__global__ void __launch_bounds__(256) k_bin(Inputs in, int warp_lim, int cta_max, int32_t* __restrict__ s_out,
                                              int32_t* __restrict__ u_out, int32_t* __restrict__ warp_list,
                                              int32_t* __restrict__ cta_list, int32_t* __restrict__ heavy_list,
                                              int32_t* __restrict__ big_list,
@@ -48,13 +60,16 @@ __global__ void __launch_bounds__(256) k_bin(Inputs in, int warp_max, int cta_ma
         s = INT32_MAX;
       }
       if (s <= 0) cls = CLS_EMPTY;
-      else if (s <= warp_max) cls = CLS_WARP;
+      else if (s <= warp_lim) cls = CLS_WARP;
       else if (s <= cta_max) cls = CLS_CTA;
       else cls = CLS_HEAVY;
       s_out[g] = (int32_t)s;
       if (cls == CLS_EMPTY) u_out[g] = 0;
     }
-    warp_append(cls == CLS_WARP, warp_list, &ctr->n_warp, g, lane);
+    warp_append(cls == CLS_WARP && s <= WARP_SMALL, warp_list, &ctr->n_warp, g, lane);
+    warp_append_back(cls == CLS_WARP && s > WARP_SMALL, warp_list + in.ncols, &ctr->n_wbig, g, lane);
+    const int mx = warp_max(cls == CLS_WARP ? (int)s : 0);
+    if (lane == 0 && mx > 0 && mx > ctr->max_warp_s) atomicMax(&ctr->max_warp_s, mx);
     warp_append(cls == CLS_CTA, cta_list, &ctr->n_cta, g, lane);
     // Heavy columns: the largest go to their own list, handed out first.
     warp_append(cls == CLS_HEAVY && s <= BIG_S, heavy_list, &ctr->n_heavy, g, lane);

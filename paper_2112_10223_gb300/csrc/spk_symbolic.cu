@@ -735,7 +735,7 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
                            cudaStream_t st) {
   if (in.mmax <= (1 << SLAB_BITS)) {
     const bool wide = in.mmax > (1 << SYM_FLAT_LOG2);
-    const int words = (in.mmax + 31) / 32;
+    const int words = pow2_at_least((in.mmax + 31) / 32);  // (few sizes: their occupancy is looked up once)
     const size_t smem = sizeof(ItemMap<SYM_BLOCK>) + (wide ? (1024 + CTA_MAX_LIMIT) * 4 + 1024 * 2 : (size_t)words * 4);
     auto kern = wide ? k_sym_items<true> : k_sym_items<false>;
     const int bps = resident_blocks((const void*)kern, SYM_BLOCK, smem);

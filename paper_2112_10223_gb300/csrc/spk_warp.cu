@@ -2,6 +2,11 @@
 // one warp per column, for both the symbolic count (Alg. 6's role) and the
 // numeric sum (Alg. 5's role).
 //
+// k_warp_sort (below) sorts a column's entries in registers (spk_wsort.cuh) and
+// takes most columns.  k_warp_col, described next, takes problems of more than
+// 2^23 rows, and the long columns of problems whose rows hardly repeat
+// (bucket_column).
+//
 // The table is a bucketed hash whose hash is order-preserving,
 // b(r) = floor(r * NB / m) with NB = 2^q >= s_j buckets: a bucket holds about
 // one entry and every row of bucket b is smaller than every row of a later
@@ -31,6 +36,7 @@
 #include "spk_common.cuh"
 #include "spk_launch.h"
 #include "spk_lookback.cuh"
+#include "spk_wsort.cuh"
 
 
 namespace spk {
@@ -62,6 +68,9 @@ struct WarpColArgs {
   int smax;
   int force_dedup;         // numeric: sort_mode 1
   int unsorted_out;        // numeric: sort_mode 2
+  int split;               // k_warp_col takes the columns of bucket_column, k_warp_sort the others
+  int big_only;            // k_warp_col: the columns above WARP_SMALL entries only
+  int small_only;          // k_warp_sort: the others only
   int only_dtype;          // numeric, mixed batch: process only this dtype's columns (-1: all)
 };
 
@@ -219,12 +228,23 @@ struct ColState {
   int64_t out;  // numeric: global col_ptr_B[g]
 };
 
+// Where the problem's sizes say that rows hardly repeat (Inputs::split_warp),
+// k_warp_col counts the columns of more than 256 entries with its hashed filter
+// and sums those of them that proved to be at least seven eighths distinct rows
+// with its buckets; k_warp_sort takes all other columns.  (32 ER inputs of 2^20
+// rows, 512 entries a column, double: symbolic 1.48 ms against 2.6 ms sorted,
+// numeric 4.3 against 5.3 ms.)
+__device__ __forceinline__ bool bucket_column(int s, int u, bool numeric) {
+  return s > WARP_SMALL && (!numeric || (s - u) * 8 <= s);
+}
+
 template <bool NUMERIC, bool BATCH>
 __device__ __forceinline__ ColState load_col(const Inputs& in, const WarpColArgs& a, int cc, int ncols,
-                                             bool resident, const int32_t* my_cp, int lane, int k0) {
+                                             bool resident, const int32_t* my_cp, int lane, int k0, int nbig) {
   ColState st{-1, 0, 0, 0, 0, 0, 0};
   if (cc >= ncols) return st;
-  st.g = a.list[cc];
+  // The columns above WARP_SMALL entries first, from the list's end.
+  st.g = cc < nbig ? a.list[in.ncols - 1 - cc] : a.list[cc - nbig];
   if (BATCH) st.q = __ldg(in.col_inst + st.g);
   st.s = a.s_arr[st.g];
   if (NUMERIC) {
@@ -581,7 +601,8 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
   if (!BATCH && threadIdx.x < 16) s_mul[threadIdx.x] = in.inst[0].bucket_mul[threadIdx.x];
   if (!BATCH && threadIdx.x == 0) s_m0 = in.inst[0].m;
   __syncthreads();
-  const int ncols = a.ctr->n_warp;
+  const int nbig = a.ctr->n_wbig;
+  const int ncols = (a.big_only ? 0 : a.ctr->n_warp) + nbig;
   const int k0 = in.inst[0].k;
   const bool resident = RES;
   if (RES && (BATCH || k0 > 32)) {  // the host never launches this; never index lanes past k
@@ -599,9 +620,9 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
   const int stride = gridDim.x * WARPS;
   int c = blockIdx.x * WARPS + wid;
   // Scalars of the current column and of the next one (loaded a column ahead).
-  ColState cur = load_col<NUMERIC, BATCH>(in, a, c, ncols, resident, my_cp, lane, k0);
-  ColState nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, resident, my_cp, lane, k0);
-  int n_unique = 0;
+  ColState cur = load_col<NUMERIC, BATCH>(in, a, c, ncols, resident, my_cp, lane, k0, nbig);
+  ColState nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, resident, my_cp, lane, k0, nbig);
+  int n_unique = 0, n_bucket = 0;
   while (cur.g >= 0) {
     // One problem: its scalars were hoisted; a batch looks them up per column.
     const Inst* I = in.inst + cur.q;
@@ -610,7 +631,8 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
     const int j = BATCH ? cur.g - I->colbase : cur.g;
     const int qb = max(5, ceil_log2(cur.s));
     const int NB = 1 << qb;
-    if (NUMERIC && BATCH && a.only_dtype >= 0 && I->dtype != a.only_dtype) {
+    if ((a.split && !bucket_column(cur.s, cur.u, NUMERIC)) ||
+        (NUMERIC && BATCH && a.only_dtype >= 0 && I->dtype != a.only_dtype)) {
       // another launch handles this column
     } else if (NB > smax) {  // not reachable for a warp-class column
       if (lane == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
@@ -633,6 +655,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
         if (lane == 0) {
           a.u_out[cur.g] = cur.s - dups;
           n_unique += (dups == 0);
+          n_bucket += bucket_column(cur.s, cur.s - dups, true);
         }
       } else {
         // B(:,j) starts at col_ptr_B[g] - col_ptr_B[colbase] in its problem's buffers.
@@ -646,7 +669,97 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
     __syncwarp();
     c += stride;
     cur = nxt;
-    nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, resident, my_cp, lane, k0);
+    nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, resident, my_cp, lane, k0, nbig);
+  }
+  if (!NUMERIC && lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
+  if (!NUMERIC && lane == 0 && n_bucket) atomicAdd(&a.ctr_w->n_bucket, n_bucket);
+}
+
+// The same columns through the register sort (spk_wsort.cuh), for problems of
+// at most 2^WSORT_ROW_BITS rows.  What bounds it: the ALU pipe in the network of
+// 512 keys (80% busy), waits for the column's loads in the smaller ones.
+// Against the buckets (symbolic + numeric): 65536 columns of 256 to 384 entries
+// on 128 rows, float, four adds 3.40 -> 1.67 ms; R-MAT scale 14 k = 16 double
+// 0.182 -> 0.080 ms.
+template <int DT, bool NUMERIC, bool BATCH, bool RES, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24) / WARPS) k_warp_sort(Inputs in, WarpColArgs a) {
+  using VB = typename std::conditional<DT == 1, double, float>::type;
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const WsortSmem sm = wsort_carve<VB, NUMERIC>(sm_raw + (size_t)wid * wsort_bytes<VB, NUMERIC>(a.smax), a.smax);
+  if (lane < a.smax / 32) sm.blk[lane].x = 0u;
+  __syncwarp();
+  const int nbig = a.ctr->n_wbig;
+  const int c0 = a.small_only ? nbig : 0;
+  const int ncols = a.ctr->n_warp + nbig;
+  const int k0 = in.inst[0].k;
+  if (RES && (BATCH || k0 > 32)) {  // the host never launches this; never index lanes past k
+    if (threadIdx.x == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+    return;
+  }
+  const int32_t* my_cp = nullptr;
+  const int32_t* my_ri = nullptr;
+  const VB* my_va = nullptr;
+  if (RES && lane < k0) {
+    my_cp = in.cp[lane];
+    my_ri = in.ri[lane];
+    if constexpr (NUMERIC) my_va = static_cast<const VB*>(in.val[lane]);
+  }
+  const int m0 = in.inst[0].m;
+  const int stride = gridDim.x * WARPS;
+  int c = c0 + blockIdx.x * WARPS + wid;
+  // Scalars of the current column and of the next one (loaded a column ahead).
+  ColState cur = load_col<NUMERIC, BATCH>(in, a, c, ncols, RES, my_cp, lane, k0, nbig);
+  ColState nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig);
+  int n_unique = 0;
+  while (cur.g >= 0) {
+    const Inst* I = in.inst + cur.q;
+    const int k = BATCH ? I->k : k0;
+    const int off = BATCH ? I->ptr_off : 0;
+    const int j = BATCH ? cur.g - I->colbase : cur.g;
+    auto bounds = [&](int i, WsortIn<VB>& x) {
+      if (RES) {
+        x = WsortIn<VB>{cur.beg, cur.len, my_ri, my_va};
+      } else {
+        const int32_t* cp = in.cp[off + i];
+        x.beg = __ldg(cp + j);
+        x.len = __ldg(cp + j + 1) - x.beg;
+        x.rp = in.ri[off + i];
+        if constexpr (NUMERIC) x.vp = static_cast<const VB*>(in.val[off + i]);
+      }
+    };
+    if ((a.split && bucket_column(cur.s, cur.u, NUMERIC)) ||
+        (NUMERIC && BATCH && a.only_dtype >= 0 && I->dtype != a.only_dtype)) {
+      // another launch handles this column
+    } else if (cur.s > a.smax) {  // not reachable for a warp-class column
+      if (lane == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+    } else {
+      const uint32_t m = (uint32_t)(BATCH ? I->m : m0);
+      // B(:,j) starts at col_ptr_B[g] - col_ptr_B[colbase] in its problem's buffers.
+      int32_t* orow = nullptr;
+      VB* oval = nullptr;
+      if constexpr (NUMERIC) {
+        const int64_t out = cur.out - (BATCH ? a.col_ptr[I->colbase] : 0);
+        orow = (BATCH ? out_row_of(a.out, cur.q) : a.out.row0) + out;
+        oval = static_cast<VB*>(BATCH ? out_val_of(a.out, cur.q) : a.out.val0) + out;
+      }
+      const int u = wsort_any<VB, NUMERIC>(sm, k, cur.s, m, NUMERIC && a.unsorted_out && cur.u == cur.s, bounds, lane);
+      if constexpr (NUMERIC) {
+        if (u == cur.u) wsort_write<VB>(sm, wsort_eb(cur.s), cur.s, u, orow, oval, lane);
+        else if (lane == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);  // symbolic and numeric disagree
+      }
+      if constexpr (!NUMERIC) {
+        if (lane == 0) {
+          if (u < 0) atomicOr(&a.ctr_w->err, ERR_RANGE);  // a row outside [0, m): reported; B is never computed
+          a.u_out[cur.g] = u < 0 ? cur.s : u;
+          n_unique += u == cur.s;
+        }
+      }
+    }
+    __syncwarp();
+    c += stride;
+    cur = nxt;
+    nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig);
   }
   if (!NUMERIC && lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
 }
@@ -674,6 +787,7 @@ struct OnepassArgs {
   int n;
   int ntiles;
   int smax;
+  int cols;                    // k_sort_onepass: columns per warp and tile, of at most smax entries
   int force_dedup;
   int debug_stall;             // test switch: tile 1's look-back also waits on a word nothing writes
   unsigned long long wait_ns;  // bound of every device-side wait
@@ -809,6 +923,146 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_onepass(Inputs in, Onepa
   }
 }
 
+// The one-pass kernel over the register sort.  What bounds it for short columns
+// is the chain of a tile (ticket, column pointers, entries, look-back, write),
+// not the sorting, so a tile holds several columns per warp (a.cols, as many of
+// a.smax entries as fit 512): 300007 columns of 77 entries, float, 1.02 ms with
+// one column per warp in buckets, 0.92 ms in sorted keys, 0.41 ms with four.
+constexpr int ONEPASS_COLS_MAX = 16;
+
+template <int WARPS>
+struct SortTile {
+  int ticket;
+  int bad;                               // the look-back gave up
+  long long off;                         // the tile's first entry in B
+  int u[WARPS * ONEPASS_COLS_MAX];       // nnz(B(:,j)) of the tile's columns
+  int pre[WARPS * ONEPASS_COLS_MAX];     // and their exclusive prefix
+  int uq[WARPS];                         // columns without repeated rows
+};
+
+template <int DT, bool RES, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 3) k_sort_onepass(Inputs in, OnepassArgs a) {
+  using VB = typename std::conditional<DT == 1, double, float>::type;
+  static_assert(WARPS * ONEPASS_COLS_MAX <= 128, "four columns a lane in the tile's scan");
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ SortTile<WARPS> T;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int cap = a.smax, C = a.cols, per_tile = WARPS * C;
+  unsigned char* base = sm_raw + (size_t)wid * wsort_slots_bytes<VB>(cap, C);
+  if (lane < 16) wsort_carve_slot<VB>(base, cap, 0).blk[lane].x = 0u;
+  __syncwarp();
+  const int k = in.inst[0].k;
+  const uint32_t m = (uint32_t)in.inst[0].m;
+  if (RES && k > 32) {  // the host never launches this; never index lanes past k
+    if (threadIdx.x == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+    return;
+  }
+  const int32_t* my_cp = nullptr;
+  const int32_t* my_ri = nullptr;
+  const VB* my_va = nullptr;
+  if (RES && lane < k) {
+    my_cp = in.cp[lane];
+    my_ri = in.ri[lane];
+    my_va = static_cast<const VB*>(in.val[lane]);
+  }
+  for (;;) {
+    if (threadIdx.x == 0) T.ticket = (int)atomicAdd(a.queue, 1u);
+    __syncthreads();
+    const int tile = T.ticket;
+    if (tile >= a.ntiles) break;
+    const int64_t j0 = (int64_t)tile * per_tile + wid * C;
+    const int nc = (int)max((int64_t)0, min((int64_t)C, a.n - j0));  // this warp's columns
+    int beg = 0, end = 0, unique = 0;
+    if (RES && nc > 0 && lane < k) {
+      beg = __ldg(my_cp + j0);
+      end = __ldg(my_cp + j0 + 1);
+    }
+    for (int c = 0; c < C; ++c) {
+      int u = 0;
+      if (c < nc) {
+        const int64_t j = j0 + c;
+        int next = 0;
+        if (RES && c + 1 < nc && lane < k) next = __ldg(my_cp + j + 2);  // a column ahead
+        const int len = end - beg;
+        const int s = RES ? __reduce_add_sync(SPK_FULL, len) : __ldg(a.s_arr + j);
+        if (s > cap) {  // not reachable: the host sizes cap to the largest column
+          if (lane == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+        } else if (s > 0) {
+          auto bounds = [&](int i, WsortIn<VB>& x) {
+            if (RES) {
+              x = WsortIn<VB>{beg, len, my_ri, my_va};
+            } else {
+              const int32_t* cp = in.cp[i];
+              x.beg = __ldg(cp + j);
+              x.len = __ldg(cp + j + 1) - x.beg;
+              x.rp = in.ri[i];
+              x.vp = static_cast<const VB*>(in.val[i]);
+            }
+          };
+          u = wsort_any<VB, true>(wsort_carve_slot<VB>(base, cap, c), k, s, m, false, bounds, lane);
+          __syncwarp();
+          if (u < 0) {  // a row outside [0, m): reported; B is not computed for the column
+            if (lane == 0) atomicOr(&a.ctr_w->err, ERR_RANGE);
+            u = 0;
+          } else {
+            unique += u == s;
+          }
+        }
+        beg = end;
+        end = next;
+      }
+      if (lane == 0) T.u[wid * C + c] = u;
+    }
+    if (lane == 0) T.uq[wid] = unique;
+    __syncthreads();
+    if (wid == 0) {
+      int v[4], sum = 0;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        v[x] = 4 * lane + x < per_tile ? T.u[4 * lane + x] : 0;
+        sum += v[x];
+      }
+      int run = warp_incl_scan(sum, lane) - sum;
+      const long long agg = lb_warp_sum64(sum);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        if (4 * lane + x < per_tile) T.pre[4 * lane + x] = run;
+        run += v[x];
+      }
+      bool pois = false;
+      const long long excl = tile_lookback(a.status, tile, agg, a.wait_ns, a.debug_stall && tile == 1, &pois, lane);
+      const int uq = __reduce_add_sync(SPK_FULL, lane < WARPS ? T.uq[lane < WARPS ? lane : 0] : 0);
+      if (lane == 0) {
+        if (uq) atomicAdd(&a.ctr_w->n_unique, uq);
+        T.off = excl;
+        T.bad = pois ? 1 : 0;
+        if (pois) atomicOr(&a.ctr_w->err, ERR_TIMEOUT);
+      }
+    }
+    __syncthreads();
+    if (!T.bad) {
+      for (int c = 0; c < nc; ++c) {
+        const int64_t j = j0 + c;
+        const int u = T.u[wid * C + c];
+        const long long o = T.off + T.pre[wid * C + c];
+        if (lane == 0) {
+          a.col_ptr[j] = o;
+          if (j == a.n - 1) a.col_ptr[a.n] = o + u;
+        }
+        if (u > 0) {
+          const int s = __ldg(a.s_arr + j);
+          if (o + u <= a.capacity)
+            wsort_write<VB>(wsort_carve_slot<VB>(base, cap, c), wsort_eb(s), s, u, a.out_row + o,
+                            static_cast<VB*>(a.out_val) + o, lane);
+          else if (lane == 0)
+            atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
@@ -818,40 +1072,55 @@ static int pow2_at_least(int x) {
   return p;
 }
 
-static int blocks_per_sm(const DeviceInfo& dev, size_t smem_per_block, int threads_per_block) {
-  const size_t reserve = 1024;
-  int b = (int)(dev.smem_per_sm / (smem_per_block + reserve));
-  int bt = 2048 / threads_per_block;
-  if (b > bt) b = bt;
-  if (b > 32) b = 32;
-  return b < 1 ? 1 : b;
-}
-
 template <int DT, bool NUMERIC>
-static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max, int n_cols_hint,
-                                   const DeviceInfo& dev, cudaStream_t st) {
+static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max, int n_small, int n_big, int n_bucket,
+                                   const DeviceInfo& dev, cudaStream_t st, int* launches) {
   using VB = typename std::conditional<DT == 1, double, float>::type;
-  constexpr int WARPS = 8;
   a.smax = pow2_at_least(warp_max) < 32 ? 32 : pow2_at_least(warp_max);
-  const size_t smem = (size_t)WARPS * warp_col_bytes<VB, NUMERIC>(a.smax);
-  constexpr int U = NUMERIC ? 8 : 16;
-  auto kern = in.col_inst ? k_warp_col<DT, NUMERIC, true, false, WARPS, U>
-              : in.kmax <= 32 ? k_warp_col<DT, NUMERIC, false, true, WARPS, U>
-                              : k_warp_col<DT, NUMERIC, false, false, WARPS, U>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int grid = dev.sms * blocks_per_sm(dev, smem + 128, WARPS * 32);
-  if (n_cols_hint >= 0) {
-    const int need = (n_cols_hint + WARPS - 1) / WARPS;
-    if (grid > need) grid = need;
-    if (grid < 1) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto kern, int warps, size_t smem, int n_cols) {
+    const int bps = resident_blocks((const void*)kern, warps * 32, smem);
+    if (bps < 1) {
+      e = cudaErrorInvalidConfiguration;
+      return;
+    }
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return;
+    int grid = dev.sms * bps;
+    if (n_cols >= 0 && grid > (n_cols + warps - 1) / warps) grid = (n_cols + warps - 1) / warps;
+    if (grid < 1) return;
+    kern<<<grid, warps * 32, smem, st>>>(in, a);
+    e = cudaGetLastError();
+    ++*launches;
+  };
+  const bool sort = in.mmax <= (1 << WSORT_ROW_BITS);
+  // (Only k_warp_sort leaves every column without repeats as it is when B may be unsorted.)
+  a.split = sort && in.split_warp && a.smax > WARP_SMALL && !a.unsorted_out;
+  if (NUMERIC && n_bucket <= 0) a.split = 0;
+  a.big_only = a.split;
+  a.small_only = a.split && (!NUMERIC || n_bucket == n_big);  // no column above WARP_SMALL is left to sort
+  const int n_sort = NUMERIC ? n_small + (a.small_only ? 0 : n_big) : -1;
+  if (sort && n_sort != 0) {
+    constexpr int SW = 4;
+    go(in.col_inst ? k_warp_sort<DT, NUMERIC, true, false, SW>
+       : in.kmax <= 32 ? k_warp_sort<DT, NUMERIC, false, true, SW>
+                       : k_warp_sort<DT, NUMERIC, false, false, SW>,
+       SW, SW * wsort_bytes<VB, NUMERIC>(a.smax), n_sort);
   }
-  kern<<<grid, WARPS * 32, smem, st>>>(in, a);
-  return cudaGetLastError();
+  if (e == cudaSuccess && (!sort || a.split)) {
+    constexpr int WARPS = 8;
+    constexpr int U = NUMERIC ? 8 : 16;
+    go(in.col_inst ? k_warp_col<DT, NUMERIC, true, false, WARPS, U>
+       : in.kmax <= 32 ? k_warp_col<DT, NUMERIC, false, true, WARPS, U>
+                       : k_warp_col<DT, NUMERIC, false, false, WARPS, U>,
+       WARPS, WARPS * warp_col_bytes<VB, NUMERIC>(a.smax), !NUMERIC ? -1 : n_big + (a.split ? 0 : n_small));
+  }
+  return e;
 }
 
 cudaError_t launch_sym_warp(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr,
-                            int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
+                            int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
+                            int* launches) {
   WarpColArgs a{};
   a.list = list;
   a.ctr = ctr;
@@ -859,14 +1128,17 @@ cudaError_t launch_sym_warp(const Inputs& in, const int32_t* list, const int32_t
   a.u_out = u;
   a.ctr_w = ctr_w;
   a.only_dtype = -1;
-  return launch_warp_col<0, false>(in, a, warp_max, -1, dev, st);
+  *launches = 0;
+  return launch_warp_col<0, false>(in, a, warp_max, 0, 0, 0, dev, st, launches);
 }
 
-cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const Counters* ctr, int n_cols,
+cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const Counters* ctr, int n_small, int n_big,
+                            int n_bucket,
                             const int32_t* s, const int32_t* u, const int64_t* col_ptr, const Outs& out,
                             int warp_max, int sort_mode, Counters* ctr_w, const DeviceInfo& dev,
-                            cudaStream_t st) {
-  if (n_cols <= 0) return cudaSuccess;
+                            cudaStream_t st, int* launches) {
+  *launches = 0;
+  if (n_small + n_big <= 0) return cudaSuccess;
   WarpColArgs a{};
   a.list = list;
   a.ctr = ctr;
@@ -878,31 +1150,44 @@ cudaError_t launch_num_warp(const Inputs& in, int dt, const int32_t* list, const
   a.force_dedup = sort_mode == 1;
   a.unsorted_out = sort_mode == 2;
   a.only_dtype = -1;
-  if (dt == 0) return launch_warp_col<0, true>(in, a, warp_max, n_cols, dev, st);
-  if (dt == 1) return launch_warp_col<1, true>(in, a, warp_max, n_cols, dev, st);
+  if (dt == 0) return launch_warp_col<0, true>(in, a, warp_max, n_small, n_big, n_bucket, dev, st, launches);
+  if (dt == 1) return launch_warp_col<1, true>(in, a, warp_max, n_small, n_big, n_bucket, dev, st, launches);
   // Mixed batch: one launch per dtype, each skipping the other dtype's columns.
   a.only_dtype = 0;
-  cudaError_t e = launch_warp_col<0, true>(in, a, warp_max, n_cols, dev, st);
+  cudaError_t e = launch_warp_col<0, true>(in, a, warp_max, n_small, n_big, n_bucket, dev, st, launches);
   a.only_dtype = 1;
-  if (e == cudaSuccess) e = launch_warp_col<1, true>(in, a, warp_max, n_cols, dev, st);
+  if (e == cudaSuccess) e = launch_warp_col<1, true>(in, a, warp_max, n_small, n_big, n_bucket, dev, st, launches);
   return e;
 }
 
+// max_s: largest s_j (from the plan's counters).
 template <int DT>
-static cudaError_t launch_onepass_t(const Inputs& in, OnepassArgs a, int warp_max, const DeviceInfo& dev,
+static cudaError_t launch_onepass_t(const Inputs& in, OnepassArgs a, int warp_max, int max_s, const DeviceInfo& dev,
                                     cudaStream_t st, int* grid_out) {
   using VB = typename std::conditional<DT == 1, double, float>::type;
-  constexpr int WARPS = 8;  // columns per tile (warps per block)
+  constexpr int WARPS = 8;  // warps per block
   constexpr int U = 8;
-  a.smax = pow2_at_least(warp_max) < 32 ? 32 : pow2_at_least(warp_max);
-  const size_t smem = (size_t)WARPS * warp_col_bytes<VB, true>(a.smax);
-  auto kern = in.kmax <= 32 ? k_warp_onepass<DT, true, WARPS, U> : k_warp_onepass<DT, false, WARPS, U>;
+  const bool sort = in.mmax <= (1 << WSORT_ROW_BITS) && !(in.split_warp && in.mean_s > WARP_SMALL);
+  size_t smem;
+  void (*kern)(Inputs, OnepassArgs);
+  if (sort) {
+    a.smax = pow2_at_least(max_s) < 32 ? 32 : pow2_at_least(max_s);
+    // Several short columns per warp, while the tiles still fill the GPU a few times.
+    a.cols = WSORT_MAX / a.smax < ONEPASS_COLS_MAX ? WSORT_MAX / a.smax : ONEPASS_COLS_MAX;
+    while (a.cols > 1 && (int64_t)a.n < (int64_t)WARPS * a.cols * dev.sms * 12) a.cols >>= 1;
+    a.ntiles = (a.n + WARPS * a.cols - 1) / (WARPS * a.cols);
+    smem = (size_t)WARPS * wsort_slots_bytes<VB>(a.smax, a.cols);
+    kern = in.kmax <= 32 ? k_sort_onepass<DT, true, WARPS> : k_sort_onepass<DT, false, WARPS>;
+  } else {
+    a.smax = pow2_at_least(warp_max) < 32 ? 32 : pow2_at_least(warp_max);
+    a.ntiles = (a.n + WARPS - 1) / WARPS;
+    smem = (size_t)WARPS * warp_col_bytes<VB, true>(a.smax);
+    kern = in.kmax <= 32 ? k_warp_onepass<DT, true, WARPS, U> : k_warp_onepass<DT, false, WARPS, U>;
+  }
+  const int occ = resident_blocks((const void*)kern, WARPS * 32, smem);
+  if (occ < 1) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, WARPS * 32, smem);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) return cudaErrorInvalidConfiguration;
   int grid = dev.sms * occ;
   if (grid > a.ntiles) grid = a.ntiles;
   *grid_out = grid;
@@ -914,7 +1199,7 @@ int onepass_tile_cols() { return 8; }
 
 size_t onepass_scratch_bytes(int64_t ncols) { return 8 + (size_t)((ncols + 7) / 8) * 8 + 8; }
 
-cudaError_t launch_onepass(const Inputs& in, int dt, const int32_t* s, int n, int warp_max, int64_t* col_ptr,
+cudaError_t launch_onepass(const Inputs& in, int dt, const int32_t* s, int n, int warp_max, int max_s, int64_t* col_ptr,
                            int32_t* out_row, void* out_val, long long capacity, void* scratch, int force_dedup,
                            int debug_stall, unsigned long long wait_ns, Counters* ctr, const DeviceInfo& dev,
                            cudaStream_t st, int* grid_out) {
@@ -936,8 +1221,8 @@ cudaError_t launch_onepass(const Inputs& in, int dt, const int32_t* s, int n, in
   a.status = reinterpret_cast<unsigned long long*>(static_cast<char*>(scratch) + 8);
   cudaError_t e = cudaMemsetAsync(scratch, 0, 8 + (size_t)a.ntiles * 8, st);
   if (e != cudaSuccess || a.ntiles == 0) return e;
-  return dt == 1 ? launch_onepass_t<1>(in, a, warp_max, dev, st, grid_out)
-                 : launch_onepass_t<0>(in, a, warp_max, dev, st, grid_out);
+  return dt == 1 ? launch_onepass_t<1>(in, a, warp_max, max_s, dev, st, grid_out)
+                 : launch_onepass_t<0>(in, a, warp_max, max_s, dev, st, grid_out);
 }
 
 }  // namespace spk

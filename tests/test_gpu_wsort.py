@@ -1,0 +1,79 @@
+"""Light columns sorted in registers: key counts, segment tables, row limits, and the one-pass tiles.
+
+Small-integer values: indices and sums must match the oracle exactly in either type.
+"""
+import pytest
+import torch
+
+import oracle
+import paper_2112_10223_gb300 as spk
+from spk_testlib import compare, run_gpu, to_np
+from test_gpu_items import _columns
+
+pytestmark = pytest.mark.gpu
+
+# 32 E keys hold a column, E a power of two up to 16.
+LENGTHS = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 300, 511, 512]
+
+
+def _check(A, m, dtype, **opt):
+    want = oracle.add(to_np(A))
+    for method in ("twopass", "onepass"):
+        out = run_gpu(A, m, dtype=dtype, options=spk.default_options(**opt), info=True, method=method)
+        compare(tuple(t.cpu().numpy() for t in out[:3]), want, dtype, exact=True)
+    assert out[3]["onepass"] == 1 and out[3]["cols_unique"] >= 0
+    outs = spk.spkadd_batch([([tuple(t.cuda() for t in a) for a in A], m)] * 2, options=spk.default_options(**opt))
+    for o in outs:
+        compare(tuple(t.cpu().numpy() for t in o), want, dtype, exact=True)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("m", [600, 65537, 1 << 23, (1 << 23) + 1])  # keys hold rows below 2^23
+def test_key_counts_and_row_limits(m, dtype):
+    A = _columns(29, m, LENGTHS, 4, dtype)
+    _check(A, m, dtype)
+
+
+@pytest.mark.parametrize("k", [1, 31, 32, 33, 63, 64, 65, 130])  # tables hold 64 inputs, two per lane
+def test_segment_tables(k):
+    lengths = [min(s, 40 * k) for s in LENGTHS]
+    A = _columns(k, 4000, lengths, 5, torch.float64, [max(120, s // 2) for s in lengths])
+    _check(A, 4000, torch.float64)
+    _check(A, 4000, torch.float64, input_order=1, sort_mode=1)
+
+
+def test_equal_runs_and_last_rows():
+    """Every input the same: runs of k equal rows; rows up to the last."""
+    m = (1 << 23) - 1
+    rows = torch.arange(m - 25, m, dtype=torch.int32)
+    cp = torch.tensor([0, 25, 25, 50], dtype=torch.int32)
+    A = [(cp, torch.cat([rows, rows - 70]), torch.arange(50, dtype=torch.float64) - i) for i in range(20)]
+    _check(A, m, torch.float64)
+
+
+@pytest.mark.parametrize("d", [2, 9, 20, 40])  # columns per warp and tile follow the longest column
+def test_onepass_columns_per_warp(d):
+    n = 8 * 16 * 152 * 12 + 77  # enough columns for the largest tiles, and a ragged last one
+    g = torch.Generator().manual_seed(d)
+    A = []
+    for _ in range(3):
+        keep = torch.rand(n, d, generator=g) < 0.5
+        col, at = keep.nonzero(as_tuple=True)
+        cp = torch.zeros(n + 1, dtype=torch.int32)
+        cp[1:] = torch.cumsum(keep.sum(1), 0)
+        va = torch.randint(-8, 9, (at.numel(),), generator=g).to(torch.float64)
+        A.append((cp, (at * 7).to(torch.int32), va))
+    want = oracle.add(to_np(A))
+    out = run_gpu(A, 7 * d, info=True, method="onepass")
+    assert out[3]["onepass"] == 1
+    compare(tuple(t.cpu().numpy() for t in out[:3]), want, torch.float64, exact=True)
+
+
+def test_columns_split_between_sort_and_buckets():
+    """Few repeats expected (large m): the long columns go to the buckets, those that repeat after all to the sort."""
+    m = 1 << 22
+    lengths = [300, 512, 257, 256, 100, 400] * 20
+    pool = [400 if j % 6 == 1 else m for j in range(len(lengths))]
+    A = _columns(16, m, lengths, 6, torch.float64, pool)
+    _check(A, m, torch.float64)
+    _check(A, m, torch.float64, sort_mode=1)
