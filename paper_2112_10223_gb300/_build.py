@@ -1,6 +1,6 @@
 """Builds libspkadd.so in-tree with nvcc for sm_103a (GB300).
 
-Four translation units compiled in parallel, linked against the shared CUDA
+Seven translation units compiled in parallel, linked against the shared CUDA
 runtime (the same libcudart PyTorch loads), symbols hidden except the C ABI.
 """
 from __future__ import annotations
@@ -16,7 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(BUILD_DIR, "libspkadd.so")
-SOURCES = ["spk_api.cu", "spk_plan.cu", "spk_symbolic.cu", "spk_numeric.cu", "spk_noalloc.cu", "spk_warp.cu"]
+SOURCES = ["spk_api.cu", "spk_plan.cu", "spk_symbolic.cu", "spk_numeric.cu", "spk_noalloc.cu", "spk_warp.cu",
+           "spk_dup.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -138,6 +138,7 @@ struct spkadd_handle {
   void** d_out_tab = nullptr;          // batch: B row / value / col_ptr pointer tables
   int32_t *d_s = nullptr, *d_u = nullptr;
   int32_t *d_wl = nullptr, *d_cl = nullptr, *d_hl = nullptr;
+  int32_t* d_dup = nullptr;   // columns for k_num_dup
   Window* d_win = nullptr;
   int32_t* d_search = nullptr;
   int64_t win_cap = 0;
@@ -305,12 +306,15 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   const size_t o_wl = cv.take<int32_t>(ncols);
   const size_t o_cl = cv.take<int32_t>(ncols);
   const size_t o_hl = cv.take<int32_t>(2 * ncols);
+  // Columns for k_num_dup (never more than nnz / (warp_max + 1) columns are above the warp class).
+  const bool dup = o.block_accumulator == 0 && mmax <= (1 << spk::DUP_ROW_BITS);
+  const size_t o_dup = cv.take<int32_t>(!dup ? 0 : ncols < nnz_in / (o.warp_max + 1) ? ncols : nnz_in / (o.warp_max + 1));
   const size_t o_win = cv.take<Window>(win_cap);
   const size_t o_srch = cv.take<int32_t>(win_cap);
   const int cta_kinds = spk::num_cta_kinds(any32 && any64 ? 2 : (any64 ? 1 : 0), f32_kinds);
   const size_t o_ws = cv.take<Window>(__builtin_popcount(cta_kinds) > 1 ? win_cap : 0);
   const size_t o_colp = cv.take<int64_t>(ncols + 1);
-  const size_t o_scan = cv.take<long long>(spk::scan_tiles(ncols));
+  const size_t o_scan = cv.take<long long>(spk::scan_tiles(ncols) + 1);
   const size_t o_op = cv.take<char>(batch ? 0 : spk::onepass_scratch_bytes(ncols));
   h->ws_bytes = align_up(cv.off, 256);
   h->ws = static_cast<char*>(h->dev_alloc(h->ws_bytes));
@@ -328,6 +332,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   h->d_wl = reinterpret_cast<int32_t*>(h->ws + o_wl);
   h->d_cl = reinterpret_cast<int32_t*>(h->ws + o_cl);
   h->d_hl = reinterpret_cast<int32_t*>(h->ws + o_hl);
+  h->d_dup = dup ? reinterpret_cast<int32_t*>(h->ws + o_dup) : nullptr;
   h->d_win = reinterpret_cast<Window*>(h->ws + o_win);
   h->d_search = reinterpret_cast<int32_t*>(h->ws + o_srch);
   h->d_wsort = __builtin_popcount(cta_kinds) > 1 ? reinterpret_cast<Window*>(h->ws + o_ws) : nullptr;
@@ -409,7 +414,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
       return vs;
     }
   }
-  ce = spk::launch_bin(h->in, o.warp_max, o.cta_max, h->d_s, h->d_u, h->d_wl, h->d_cl, h->d_hl, h->d_ctr,
+  ce = spk::launch_bin(h->in, o.warp_max, o.cta_max, h->d_s, h->d_u, h->d_wl, h->d_cl, h->d_hl, h->d_scan, h->d_ctr,
                        h->dev.sms, h->st);
   h->launches += ncols > 0;
   if (ce != cudaSuccess) {
@@ -443,22 +448,23 @@ static spkadd_status run_symbolic(spkadd_handle* h) {
   int warp_launches = 0;
   if (h->ncols > 0) {
     ce = spk::launch_sym_heavy(h->in, h->d_hl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->d_search, h->win_cap, h->d_ctr,
-                               h->opt.window_max, h->opt.block_accumulator, h->dev, h->st);
+                               h->opt.window_max, h->opt.block_accumulator, h->d_dup, h->dev, h->st);
     if (ce == cudaSuccess)
       ce = spk::launch_sym_cta(h->in, h->d_cl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->win_cap, h->d_ctr,
-                               h->opt.cta_max, h->dev, h->st);
+                               h->opt.cta_max, h->d_dup, h->dev, h->st);
     if (ce == cudaSuccess)
       ce = spk::launch_sym_warp(h->in, h->d_wl, h->d_s, h->d_ctr, h->d_u, h->opt.warp_max, h->d_ctr, h->dev, h->st,
                                 &warp_launches);
     h->launches += 2 + warp_launches;
-    // Several problem kinds: the thread-block items grouped by kind for the numeric launches.
-    if (ce == cudaSuccess && h->d_wsort) {
-      ce = spk::launch_kind_sort(h->in, h->d_win, (int)h->win_cap, h->d_wsort, h->d_ctr, h->dev, h->st);
-      h->launches += 2;
-    }
   }
-  if (ce == cudaSuccess) ce = spk::launch_scan(h->d_u, (int)h->ncols, h->d_scan, h->d_colptr, h->st);
-  h->launches += h->ncols > 0 ? 3 : 2;
+  if (ce == cudaSuccess) ce = spk::launch_scan_fused(h->in, h->d_u, h->d_scan, h->d_colptr, h->d_dup, h->d_win, h->win_cap,
+                                                     h->d_ctr, h->st);
+  h->launches += 1;
+  // Several problem kinds: the thread-block items grouped by kind for the numeric launches.
+  if (ce == cudaSuccess && h->ncols > 0 && h->d_wsort) {
+    ce = spk::launch_kind_sort(h->in, h->d_win, (int)h->win_cap, h->d_wsort, h->d_ctr, h->dev, h->st);
+    h->launches += 2;
+  }
   if (ce == cudaSuccess && h->batch) {
     ce = spk::launch_inst_nnz(h->in, h->d_colptr, h->d_inst_nnz, h->st);
     h->launches += 1;
@@ -533,6 +539,11 @@ static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
                              h->opt.window_max > h->opt.cta_max ? h->opt.window_max : h->opt.cta_max,
                              h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
   h->launches += item_launches;
+  if (ce == cudaSuccess && h->h_ctr.n_dup > 0) {
+    ce = spk::launch_num_dup(h->in, spk::num_cta_kinds(h->dt_mode, h->f32_kinds), h->d_dup, h->h_ctr.n_dup, h->d_s,
+                             h->d_u, h->d_colptr, out, h->d_ctr, h->dev, h->st, &item_launches);
+    h->launches += item_launches;
+  }
   if (ce == cudaSuccess && h->h_ctr.n_warp + h->h_ctr.n_wbig > 0)
     ce = spk::launch_num_warp(h->in, h->dt_mode, h->d_wl, h->d_ctr, h->h_ctr.n_warp, h->h_ctr.n_wbig,
                               h->h_ctr.n_bucket, h->d_s, h->d_u, h->d_colptr, out, h->opt.warp_max, h->opt.sort_mode, h->d_ctr, h->dev, h->st,
@@ -664,7 +675,7 @@ SPK_API spkadd_status spkadd_get_info(spkadd_handle* h, spkadd_info* info) {
   info->cols_warp = (int64_t)c.n_warp + c.n_wbig;
   info->cols_cta = c.n_cta;
   info->cols_heavy = (int64_t)c.n_heavy + c.n_big;
-  info->windows = (int64_t)c.n_windows + c.n_hwin;
+  info->windows = (int64_t)c.n_windows + c.n_hwin + c.n_dup;
   info->windows_split = c.n_search;
   info->cols_unique = c.n_unique;
   info->workspace_bytes = (int64_t)(h->ws_bytes + h->offs_bytes);

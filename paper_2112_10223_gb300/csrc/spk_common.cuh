@@ -47,7 +47,20 @@ struct Counters {
   int32_t n_wbig;       // warp columns above WARP_SMALL entries, listed from the list's end
   int32_t n_bucket;     // split warp columns whose values k_warp_col sums
   int32_t max_warp_s;   // largest s_j of a warp column
+  int32_t n_dup;        // thread-block columns given to k_num_dup
+  int32_t dup_next[4];  // its work counters, one per problem kind
 };
+
+// Columns above the warp class with at most DUP_MAX_U distinct rows and at
+// least DUP_RATIO entries a row are summed by one warp each (k_num_dup).
+constexpr int DUP_MAX_U = 256;
+constexpr int DUP_RATIO = 4;
+constexpr int DUP_ROW_BITS = 23;  // rows below 2^23: a row and its table slot share a 32-bit key
+// Fewer of them than this leave warps idle (a column of 4096 entries takes one
+// warp about 90 us): they go to the thread-block items instead (a batch with
+// 3728 of them: 117 us here, 64 us there).
+constexpr int DUP_MIN_COLS = 8192;
+__host__ __device__ constexpr bool dup_column(int64_t s, int u) { return u <= DUP_MAX_U && s >= (int64_t)DUP_RATIO * u; }
 
 // Float sums.  A float sum of t terms, in any order, errs by at most
 // (t - 1) 2^-24 sum|terms| (first order), within 1e-5 sum|terms| for

@@ -31,13 +31,19 @@ int resident_blocks(const void* fn, int block, size_t smem);
 
 // heavy_list holds 2 * ncols entries: heavy columns with s_j <= BIG_S from the
 // start, the larger ones from entry ncols (Counters::n_heavy, ::n_big).
+// (It also zeroes the scan_tiles(ncols) + 1 words of launch_scan_fused.)
 cudaError_t launch_bin(const Inputs& in, int warp_max, int cta_max, int32_t* s, int32_t* u, int32_t* warp_list,
-                       int32_t* cta_list, int32_t* heavy_list, Counters* ctr, int sms, cudaStream_t st);
+                       int32_t* cta_list, int32_t* heavy_list, long long* scan_buf, Counters* ctr, int sms,
+                       cudaStream_t st);
 // Batch: col_inst[colbase + j] = q for every column j of every problem q.
 cudaError_t launch_col_inst(const Inputs& in, int32_t* col_inst, int sms, cudaStream_t st);
 cudaError_t launch_validate(const Inputs& in, const int64_t* nnz, Counters* ctr, int sms, cudaStream_t st);
 size_t scan_tiles(int64_t n);
 cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* col_ptr, cudaStream_t st);
+// The same scan in one launch over words that launch_bin zeroed.  Columns of the
+// dup list (may be null) also become window records when they are few.
+cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
+                              const int32_t* dup_list, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st);
 // Loads the scan kernels onto the current device (module loading is lazy).
 cudaError_t load_scan_kernels();
 cudaError_t launch_window_search(const Inputs& in, const Window* win, const int32_t* search_list, int n_search,
@@ -47,12 +53,13 @@ cudaError_t launch_sym_warp(const Inputs& in, const int32_t* list, const int32_t
                             int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
                             int* launches);
 cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
-                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, const DeviceInfo& dev,
-                           cudaStream_t st);
+                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, int32_t* dup_list,
+                           const DeviceInfo& dev, cudaStream_t st);
 cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
                              Window* win,
                              int32_t* search_list, int64_t win_cap, Counters* ctr_w, int window_max,
-                             int accumulator, const DeviceInfo& dev, cudaStream_t st);
+                             int accumulator, int32_t* dup_list, const DeviceInfo& dev, cudaStream_t st);
+// (dup_list: where columns for launch_num_dup go, Counters::n_dup of them; null: none are set apart.)
 
 // dt: 0 = every problem float, 1 = every problem double, 2 = mixed batch.
 // Counters after the symbolic phase: n_small and n_big warp columns, n_bucket of these k_warp_col's where they are split.
@@ -76,6 +83,10 @@ cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window
                            int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
                            const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
                            const DeviceInfo& dev, cudaStream_t st, int* launches);
+// The n columns of the dup list; kinds as num_cta_kinds gives them.
+cudaError_t launch_num_dup(const Inputs& in, int kinds, const int32_t* list, int n, const int32_t* s, const int32_t* u,
+                           const int64_t* col_ptr, const Outs& out, Counters* ctr_w, const DeviceInfo& dev,
+                           cudaStream_t st, int* launches);
 // Per-problem column pointers of B (a batch): out_cp[q][j] = col_ptr[colbase + j] - col_ptr[colbase].
 cudaError_t launch_out_colptr(const Inputs& in, const Outs& o, const int64_t* col_ptr, int sms, cudaStream_t st);
 // Per-problem nnz(B): nnz[q] = col_ptr[colbase + n] - col_ptr[colbase].

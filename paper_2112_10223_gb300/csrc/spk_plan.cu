@@ -2,6 +2,7 @@
 // and the per-input offsets of heavy-column row windows.
 #include "spk_common.cuh"
 #include "spk_launch.h"
+#include "spk_lookback.cuh"
 
 namespace spk {
 
@@ -36,10 +37,11 @@ __device__ __forceinline__ void warp_append_back(bool pred, int32_t* __restrict_
 __global__ void __launch_bounds__(256) k_bin(Inputs in, int warp_lim, int cta_max, int32_t* __restrict__ s_out,
                                              int32_t* __restrict__ u_out, int32_t* __restrict__ warp_list,
                                              int32_t* __restrict__ cta_list, int32_t* __restrict__ heavy_list,
-                                             int32_t* __restrict__ big_list,
-                                             Counters* __restrict__ ctr) {
+                                             int32_t* __restrict__ big_list, long long* __restrict__ scan_buf,
+                                             int scan_words, Counters* __restrict__ ctr) {
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < scan_words; x += stride) scan_buf[x] = 0;
   for (int64_t g0 = (int64_t)blockIdx.x * blockDim.x; g0 < in.ncols; g0 += stride) {
     const int g = (int)(g0 + threadIdx.x);
     const bool live = g < in.ncols;
@@ -210,6 +212,80 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int32_t* __rest
   if (blockIdx.x == 0 && threadIdx.x == 0) col_ptr[n] = *grand_total;
 }
 
+// The same scan in one launch (three took 9 us of a small call's 105): tiles in
+// ticket order, each tile's offset from a decoupled look-back over the tiles
+// before it.  scan_buf: the ticket counter, then one look-back word per tile,
+// zero at launch.  The tile taken first also turns the columns of the dup list
+// into window records when there are too few of them for k_num_dup.
+constexpr unsigned long long SCAN_WAIT_NS = 2000000000ull;
+
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int32_t* __restrict__ u, int n, int tiles,
+                                                          unsigned long long* __restrict__ scan_buf,
+                                                          int64_t* __restrict__ col_ptr,
+                                                          const int32_t* __restrict__ dup_list,
+                                                          Window* __restrict__ win, int64_t win_cap,
+                                                          Counters* __restrict__ ctr) {
+  __shared__ long long tmp[33];
+  __shared__ long long s_off;
+  __shared__ int s_tile;
+  if (threadIdx.x == 0) s_tile = (int)atomicAdd(reinterpret_cast<unsigned int*>(scan_buf), 1u);
+  __syncthreads();
+  const int tile = s_tile;
+  if (tile >= tiles) return;
+  unsigned long long* status = scan_buf + 1;
+  // Each thread owns SCAN_ITEMS consecutive counts of the tile.
+  const int64_t base = (int64_t)tile * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
+  int32_t v[SCAN_ITEMS];
+  long long acc = 0;
+#pragma unroll
+  for (int t = 0; t < SCAN_ITEMS; ++t) {
+    const int64_t j = base + t;
+    v[t] = j < n ? u[j] : 0;
+    acc += v[t];
+  }
+  long long total;
+  long long run = block_excl_scan64(acc, tmp, &total);
+  if (threadIdx.x < 32) {
+    bool bad = false;
+    const long long excl = tile_lookback(status, tile, total, SCAN_WAIT_NS, false, &bad, threadIdx.x);
+    if (threadIdx.x == 0) {
+      s_off = excl;
+      if (bad) atomicOr(&ctr->err, ERR_TIMEOUT);
+      if (tile == tiles - 1) col_ptr[n] = excl + total;
+    }
+  }
+  __syncthreads();
+  run += s_off;
+#pragma unroll
+  for (int t = 0; t < SCAN_ITEMS; ++t) {
+    const int64_t j = base + t;
+    if (j < n) col_ptr[j] = run;
+    run += v[t];
+  }
+  if (tile == 0 && dup_list) {
+    const int nd = ctr->n_dup, nw = ctr->n_windows, cap = (int)(win_cap - ctr->n_hwin);
+    if (nd > 0 && nd < DUP_MIN_COLS) {
+      for (int x = threadIdx.x; x < nd; x += SCAN_BLOCK) {
+        const int g = dup_list[x];
+        Window w;
+        w.col = g;
+        w.r_lo = 0;
+        w.r_hi = in.inst[inst_of(in, g)].m;
+        w.u = u[g];
+        w.out_off = 0;
+        w.search = -1;
+        if (nw + x < cap) win[nw + x] = w;
+        else atomicOr(&ctr->err, ERR_WINDOW_CAP);
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        ctr->n_windows = nw + nd;
+        ctr->n_dup = 0;
+      }
+    }
+  }
+}
+
 // Per-input offsets of split row windows (Sec. III-B: "partition rows ...
 // using binary searches"): for window w and input i, the first entry of
 // A_i(:,col) with row >= r_lo and the first with row >= r_hi.  One thread per
@@ -291,11 +367,13 @@ __global__ void __launch_bounds__(256) k_inst_nnz(Inputs in, const int64_t* __re
 // Host launchers.
 // ---------------------------------------------------------------------------
 cudaError_t launch_bin(const Inputs& in, int warp_max, int cta_max, int32_t* s, int32_t* u, int32_t* wl, int32_t* cl,
-                       int32_t* hl, Counters* ctr, int sms, cudaStream_t st) {
-  if (in.ncols == 0) return cudaSuccess;
+                       int32_t* hl, long long* scan_buf, Counters* ctr, int sms, cudaStream_t st) {
+  const int scan_words = (int)scan_tiles(in.ncols) + 1;
+  if (in.ncols == 0) return cudaMemsetAsync(scan_buf, 0, scan_words * sizeof(long long), st);
   int64_t blocks = ((int64_t)in.ncols + 255) / 256;
   if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-  k_bin<<<(int)blocks, 256, 0, st>>>(in, warp_max, cta_max, s, u, wl, cl, hl, hl + in.ncols, ctr);
+  k_bin<<<(int)blocks, 256, 0, st>>>(in, warp_max, cta_max, s, u, wl, cl, hl, hl + in.ncols, scan_buf, scan_words,
+                                      ctr);
   return cudaGetLastError();
 }
 
@@ -334,6 +412,15 @@ cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* c
   if (tiles > 0) k_scan_tiles<<<tiles, SCAN_BLOCK, 0, st>>>(u, n, tile_buf);
   k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(tile_buf, tiles, grand);
   k_scan_apply<<<tiles > 0 ? tiles : 1, SCAN_BLOCK, 0, st>>>(u, n, tile_buf, grand, col_ptr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
+                              const int32_t* dup_list, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st) {
+  int tiles = (int)(((int64_t)in.ncols + SCAN_TILE - 1) / SCAN_TILE);
+  if (tiles < 1) tiles = 1;
+  k_scan_fused<<<tiles, SCAN_BLOCK, 0, st>>>(in, u, in.ncols, tiles, reinterpret_cast<unsigned long long*>(scan_buf),
+                                            col_ptr, dup_list, win, win_cap, ctr);
   return cudaGetLastError();
 }
 

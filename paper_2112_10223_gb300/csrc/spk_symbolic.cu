@@ -121,7 +121,8 @@ template <bool WIDE>
 __global__ void __launch_bounds__(SYM_BLOCK, 5) k_sym_items(Inputs in, const int32_t* __restrict__ list,
                                                              const Counters* __restrict__ ctr,
                                                              int32_t* __restrict__ u_out, Window* __restrict__ win,
-                                                             int64_t win_cap, int words, Counters* ctr_w) {
+                                                             int64_t win_cap, int words, const int32_t* __restrict__ s_arr,
+                                                             int32_t* __restrict__ dup_list, Counters* ctr_w) {
   constexpr int B = SYM_BLOCK;
   using Map = ItemMap<B>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -265,7 +266,10 @@ __global__ void __launch_bounds__(SYM_BLOCK, 5) k_sym_items(Inputs in, const int
       for (int x = tid; x < ne; x += B) cw[x] = 0u;
     }
     item_unmap(M);
-    if (tid == 0) {
+    if (tid == 0 && dup_list && dup_column(s_arr[g], u)) {
+      u_out[g] = u;
+      dup_list[atomicAdd(&ctr_w->n_dup, 1)] = g;
+    } else if (tid == 0) {
       u_out[g] = u;
       const int wi = atomicAdd(&ctr_w->n_windows, 1);
       if (wi < win_cap - ctr->n_hwin) {
@@ -302,7 +306,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
                                                      const Counters* __restrict__ ctr, int32_t* __restrict__ u_out,
                                                      Window* __restrict__ win, int32_t* __restrict__ search_list,
                                                      int64_t win_cap, int win_target, int slab_log2,
-                                                     Counters* ctr_w) {
+                                                     int32_t* __restrict__ dup_list, Counters* ctr_w) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int red[BLOCK / 32 + 1];
   __shared__ int bnd[MAX_SLAB_WINDOWS + 1];
@@ -441,7 +445,9 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
       // than k binary searches per window.  Unordered inputs always do so.
       const bool searched = !whole && in.sorted &&
                             (nslabs > 1 || P > FILTER_WINDOWS || (int64_t)s_arr[g] > (int64_t)FILTER_SEG * k);
-      if (P > MAX_SLAB_WINDOWS) {  // win_target is validated on the host; guard anyway
+      if (whole && dup_list && dup_column(s_arr[g], slab_u)) {
+        if (threadIdx.x == 0) dup_list[atomicAdd(&ctr_w->n_dup, 1)] = g;
+      } else if (P > MAX_SLAB_WINDOWS) {  // win_target is validated on the host; guard anyway
         if (threadIdx.x == 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
       } else if (P > 0) {
         if (threadIdx.x == 0) {
@@ -731,8 +737,8 @@ static int pow2_at_least(int x) {
 }
 
 cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
-                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, const DeviceInfo& dev,
-                           cudaStream_t st) {
+                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, int32_t* dup_list,
+                           const DeviceInfo& dev, cudaStream_t st) {
   if (in.mmax <= (1 << SLAB_BITS)) {
     const bool wide = in.mmax > (1 << SYM_FLAT_LOG2);
     const int words = pow2_at_least((in.mmax + 31) / 32);  // (few sizes: their occupancy is looked up once)
@@ -742,7 +748,7 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
     if (bps < 1) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dev.sms * bps, SYM_BLOCK, smem, st>>>(in, list, ctr, u, win, win_cap, words, ctr_w);
+    kern<<<dev.sms * bps, SYM_BLOCK, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup_list, ctr_w);
     return cudaGetLastError();
   }
   constexpr int BLOCK = 512;
@@ -767,7 +773,7 @@ constexpr int HEAVY_CAP = 4096;  // non-empty 32-row words per sub-range of the 
 // symbolic 7.2 ms as a bitmap, about 13 ms compact).
 cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
                              Window* win, int32_t* search_list, int64_t win_cap, Counters* ctr_w, int window_max,
-                             int accumulator, const DeviceInfo& dev, cudaStream_t st) {
+                             int accumulator, int32_t* dup_list, const DeviceInfo& dev, cudaStream_t st) {
   int slab_log2 = 10;
   while (slab_log2 < SLAB_BITS && ((int64_t)1 << slab_log2) < (int64_t)in.mmax) ++slab_log2;
   const size_t w64 = (size_t)1 << (slab_log2 - 6);
@@ -797,7 +803,7 @@ cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_
   if (e != cudaSuccess) return e;
   // Windows end on 64-row words: a window holds at most win_target + 63 rows.
   kern<<<dev.sms * bf, block, smem, st>>>(in, list, s, ctr, u, win, search_list, win_cap, window_max - 64, slab_log2,
-                                          ctr_w);
+                                          dup_list, ctr_w);
   return cudaGetLastError();
 }
 

@@ -76,13 +76,14 @@ class Request:
     def workspace_bytes(self) -> int:
         """An estimate of the planner's workspace for the request: per-column and per-input tables, and the
         thread-block item records, bounded as the library bounds them for the default class limits (512 /
-        4096 / 4096), at 52 bytes each (record, search row and the copy grouped by problem kind).  After the
+        4096 / 4096), at 56 bytes each (record, search row, the copy grouped by problem kind and the list of
+        columns with few distinct rows).  After the
         symbolic phase the server charges the batch's actual workspace instead."""
         slabs = max(1, -(-self.m // (1 << 20)))
         heavy = min(self.n, self.nnz_in // 4097)
         cta = min(self.n, self.nnz_in // 513)
         items = self.nnz_in // 4032 + heavy * (slabs + 1) + cta + 16
-        return 48 * self.n + 64 * self.k + 52 * items + 4096
+        return 48 * self.n + 64 * self.k + 56 * items + 4096
 
     def output_bytes(self, nnz_out: int) -> int:
         """B's exact size once the symbolic phase has given nnz(B)."""

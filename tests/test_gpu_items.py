@@ -72,3 +72,22 @@ def test_few_distinct_rows_many_terms():
     check_full(full, 5000, torch.float64, exact=True)
     check_full([(full[0][0], r, full[0][2])], 4096, torch.float64, exact=True)
     check_full([(full[0][0], r + ((1 << 20) - 4096), full[0][2])], 1 << 20, torch.float64, exact=True)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("k,L,m", [(40, 16, 5000), (33, 32, 1 << 23), (200, 6, 9001), (70, 64, (1 << 23) + 1)])
+def test_many_columns_on_few_rows(k, L, m, dtype):
+    """Enough columns of 64 to 256 distinct rows for the warp-per-column table (rows below 2^23), one and
+    several segment tables, ragged and equal inputs, in and out of order."""
+    import synth
+    n = 8300
+    A = synth.spgemm_like(k, m, n, L, seed=9, dtype=dtype, value_kind="int8")
+    A[1] = (torch.zeros(n + 1, dtype=torch.int32), A[1][1][:0], A[1][2][:0])  # an empty input: lengths differ
+    check_full(A, m, dtype, exact=True)
+    flipped = []
+    for cp, ri, va in A:
+        e = torch.arange(ri.numel())
+        col = torch.repeat_interleave(torch.arange(n), (cp[1:] - cp[:-1]).long())
+        at = (cp[:-1].long()[col] + cp[1:].long()[col] - 1 - e)
+        flipped.append((cp, ri[at], va[at]))
+    check_full(flipped, m, dtype, exact=True, options=spk.default_options(input_order=1))
