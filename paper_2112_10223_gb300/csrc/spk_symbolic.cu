@@ -299,27 +299,32 @@ constexpr int FILTER_SEG = 64;
 // non-empty word), both kept zero between slabs, so the work per slab grows
 // with the rows present, not with the slab.  The popcount prefix over the
 // non-empty words gives nnz(B(:,j)) and cuts the column into windows of at
-// most win_target + 63 distinct rows (boundaries on 64-row words).
-template <int BLOCK, int U>
+// most win_target + 63 distinct rows (boundaries on 64-row words).  The rows
+// come through the entry map of spk_items.cuh, the next column's bounds while
+// this one is counted (15669 columns of 9000 entries, m = 20011: 0.81 -> 0.33 ms;
+// with the 128 KB bitmap of 2^20 rows one block holds the SM and the prefix and
+// its barriers decide: R-MAT scale 20 5.06 -> 4.94 ms).
+template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inputs in, const int32_t* __restrict__ list,
                                                      const int32_t* __restrict__ s_arr,
                                                      const Counters* __restrict__ ctr, int32_t* __restrict__ u_out,
                                                      Window* __restrict__ win, int32_t* __restrict__ search_list,
                                                      int64_t win_cap, int win_target, int slab_log2,
                                                      int32_t* __restrict__ dup_list, Counters* ctr_w) {
+  using Map = ItemMap<BLOCK>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int red[BLOCK / 32 + 1];
   __shared__ int bnd[MAX_SLAB_WINDOWS + 1];
   __shared__ int cval[MAX_SLAB_WINDOWS + 1];
   __shared__ int s_col_u, s_wbase, s_sbase;
-  constexpr int NW = BLOCK / 32;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int W64 = 1 << (slab_log2 - 6);
   const int NSW = (W64 + 31) >> 5;
-  unsigned long long* bm = reinterpret_cast<unsigned long long*>(sm_raw);
+  Map& M = *reinterpret_cast<Map*>(sm_raw);
+  unsigned long long* bm = reinterpret_cast<unsigned long long*>(sm_raw + sizeof(Map));
   uint32_t* summ = reinterpret_cast<uint32_t*>(bm + W64);
   for (int x = threadIdx.x; x < W64; x += BLOCK) bm[x] = 0ull;
   for (int x = threadIdx.x; x < NSW; x += BLOCK) summ[x] = 0u;
+  item_unmap(M);
   __syncthreads();
   const int n_big = ctr->n_big;
   const int ncols = n_big + ctr->n_heavy;
@@ -329,95 +334,119 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
   __shared__ int s_tk[2];
   if (threadIdx.x == 0) s_tk[0] = atomicAdd(&ctr_w->heavy_next, 1);
   __syncthreads();
+  // A column's bounds of its first segment table; those of a one-slab column
+  // are read while the column before it runs.
+  auto column = [&](int c) { return c < n_big ? list[in.ncols + c] : list[c - n_big]; };
+  auto bounds = [&](int g, const Inst* I, int k_lo) {
+    const int j = g - I->colbase, off = I->ptr_off;
+    auto seg = [&](int i, int* beg, int* end) {
+      const int32_t* cp = in.cp[off + i];
+      *beg = __ldg(cp + j);
+      *end = __ldg(cp + j + 1);
+    };
+    return item_bounds<BLOCK>(k_lo, min(Map::KT, I->k - k_lo), seg);
+  };
+  ItemBounds<BLOCK> F;
+  if (s_tk[0] < ncols) {
+    const int g = column(s_tk[0]);
+    F = bounds(g, in.inst + inst_of(in, g), 0);
+  }
   for (int it = 0;; ++it) {
     const int c = s_tk[it & 1];
     if (c >= ncols) break;
     if (threadIdx.x == 0) s_tk[(it + 1) & 1] = atomicAdd(&ctr_w->heavy_next, 1);
-    const int g = c < n_big ? list[in.ncols + c] : list[c - n_big];
+    const int g = column(c);
     const Inst* I = in.inst + inst_of(in, g);
-    const int k = I->k, off = I->ptr_off, m = I->m, j = g - I->colbase;
+    const int k = I->k, off = I->ptr_off, m = I->m;
     const int nslabs = (int)(((int64_t)m + slab_rows - 1) / slab_rows);
     if (threadIdx.x == 0) s_col_u = 0;
     for (int slab = 0; slab < nslabs; ++slab) {
       const int lo = slab * slab_rows;
       const int hi = (int)min((int64_t)m, (int64_t)lo + slab_rows);
       const uint32_t width = (uint32_t)(hi - lo);
-      // Chunks of 32 inputs side by side: `groups` of `wpg` warps.
-      const int nch = (k + 31) >> 5;
-      const int groups = min(nch, NW);
-      const int wpg = NW / groups;
-      const int gid = wid / wpg, lw = wid - gid * wpg;
-      for (int cb = gid * 32; gid < groups && cb < k; cb += groups * 32) {
-        const int i = cb + lane;
-        int beg = 0, len = 0;
-        const int32_t* rp = nullptr;  // this lane's input segment (its rows from beg)
-        if (i < k) {
-          const int32_t* cp = in.cp[off + i];
-          const int32_t* ri = in.ri[off + i];
-          int b = __ldg(cp + j), e = __ldg(cp + j + 1);
+      const int nib = (k + Map::KT - 1) / Map::KT;
+      for (int ib = 0; ib < nib; ++ib) {
+        const int k_lo = ib * Map::KT;
+        if (ib > 0 || nslabs > 1) {
+          F = bounds(g, I, k_lo);
           if (nslabs > 1 && in.sorted) {  // unordered inputs: the whole column, rows outside the slab skipped
-            b = lower_bound_i32(ri, b, e, lo);
-            e = lower_bound_i32(ri, b, e, hi);
-          }
-          beg = b;
-          len = e - b;
-          rp = ri + b;
-        }
-        ChunkMap cm;
-        const int nvalid = min(32, k - cb);
-        cm.init(beg, len, lane, nvalid);
-        // Sets the row bits of U rows (r < 0: none), then the summary marks they call for.
-        auto set_rows = [&](const int32_t (&r)[U]) {
-          bool fresh[U];
 #pragma unroll
-          for (int t = 0; t < U; ++t) {
-            const uint32_t rr = (uint32_t)(r[t] - lo);
-            fresh[t] = r[t] >= 0 && rr < width && set_row_bit(bm, rr);
-          }
-#pragma unroll
-          for (int t = 0; t < U; ++t)
-            if (fresh[t]) {
-              const uint32_t w = (uint32_t)(r[t] - lo) >> 6;
-              atomicOr(&summ[w >> 5], 1u << (w & 31));
-            }
-        };
-        if (!cm.equal && cm.total >= SEG_MAJOR_MIN * nvalid) {
-          // Long ragged segments: each warp walks whole segments (no per-entry search).
-          for (int sgi = lw; sgi < nvalid; sgi += wpg) {
-            const int ls = __shfl_sync(SPK_FULL, len, sgi);
-            const int32_t* p = reinterpret_cast<const int32_t*>(
-                __shfl_sync(SPK_FULL, reinterpret_cast<unsigned long long>(rp), sgi));
-            for (int e0 = 0; e0 < ls; e0 += 32 * U) {
-              int32_t r[U];
-#pragma unroll
-              for (int t = 0; t < U; ++t) {
-                const int o = e0 + t * 32 + lane;
-                r[t] = (e0 + t * 32 < ls && o < ls) ? __ldg(p + o) : -1;
+            for (int h = 0; h < Map::KPT; ++h)
+              if (F.beg[h] < F.end[h]) {
+                const int32_t* ri = in.ri[off + k_lo + Map::KPT * (int)threadIdx.x + h];
+                F.beg[h] = lower_bound_i32(ri, F.beg[h], F.end[h], lo);
+                F.end[h] = lower_bound_i32(ri, F.beg[h], F.end[h], hi);
               }
-              set_rows(r);
+          }
+          __syncthreads();
+        }
+        // Row bit, and the summary mark of the word whose half it is first in.
+        auto set_row = [&](uint32_t row) {
+          const uint32_t rr = row - (uint32_t)lo;
+          const uint32_t cl = min(rr, width - 1u);
+          uint32_t old = 1u;
+          if (rr < width) old = atomicOr(reinterpret_cast<uint32_t*>(bm) + (cl >> 5), 1u << (cl & 31));
+          if (old == 0u) atomicOr(&summ[cl >> 11], 1u << ((cl >> 6) & 31));
+        };
+        const int total = item_table<0, false, true>(M, in, off, k_lo, min(Map::KT, k - k_lo), F, M.red[0]);
+        __syncthreads();
+        if (total <= Map::CAP || total < 256 * M.ne) {  // chunk by chunk, all of a chunk's loads in flight
+          for (int c0 = 0; total > 0; c0 += Map::CAP) {
+            if (c0 > 0) {
+              item_map(M, c0);
+              __syncthreads();
             }
-          }
-          continue;
-        }
-        if (lw * 32 * U >= cm.total) continue;  // (warp-uniform) no entries for this warp
-        for (int e0 = lw * 32 * U; e0 < cm.total; e0 += wpg * 32 * U) {
-          int32_t r[U];
+            ItemSlots<BLOCK> L;
+            uint32_t r[ITEM_SLOTS];
+            L.init(c0, total);
+            item_rows(M, L, c0, r);
 #pragma unroll
-          for (int t = 0; t < U; ++t) {
-            r[t] = -1;
-            if (e0 + t * 32 >= cm.total) continue;  // (warp-uniform) slot wholly past the chunk's end
-            const int e = e0 + t * 32 + lane;
-            int o;
-            const int sg = cm.seg_off(e, &o);
-            const int32_t* p = reinterpret_cast<const int32_t*>(
-                __shfl_sync(SPK_FULL, reinterpret_cast<unsigned long long>(rp), sg & 31));
-            if (e < cm.total) r[t] = __ldg(p + o);
+            for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+              if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+              for (int q = q0; q < q0 + ITEM_GROUP; ++q) set_row(r[q]);
+            }
+            if (total - c0 <= Map::CAP) break;
+            __syncthreads();
+            item_unmap(M);
+            __syncthreads();
           }
-          // All bit sets of the round first, then the summary marks they call for.
-          set_rows(r);
+        } else {
+          // Long segments: each warp walks an equal run of the positions, segment
+          // by segment, without barriers (96 columns of 480,000 entries: 263 us
+          // in chunks, 232 us so; columns of 250 segments of 34: 0.33 and 1.08 ms).
+          const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+          const int run = (int)(((int64_t)total + Map::NW - 1) / Map::NW);
+          const int64_t p1 = min((int64_t)total, (int64_t)(wid + 1) * run);
+          int64_t p = (int64_t)wid * run;
+          int o = 0, oe = M.ne;  // the last segment that starts at or before p
+          while (oe - o > 1) {
+            const int mid = (o + oe) >> 1;
+            if (M.first[mid] <= p) o = mid;
+            else oe = mid;
+          }
+          for (; p < p1; ++o) {
+            const int32_t* rows = reinterpret_cast<const int32_t*>(M.seg[o].x);
+            const int64_t end = min(p1, (int64_t)M.first[o + 1]);
+            for (; p < end; p += 256) {
+              uint32_t r[8];
+#pragma unroll
+              for (int t = 0; t < 8; ++t) r[t] = (uint32_t)__ldg(rows + min(p + 32 * t + lane, end - 1));
+#pragma unroll
+              for (int t = 0; t < 8; ++t)
+                if (p + 32 * t < end) set_row(r[t]);  // (warp-uniform)
+            }
+            p = end;
+          }
         }
+        __syncthreads();
+        item_unmap(M);
       }
       __syncthreads();
+      if (slab == nslabs - 1 && s_tk[(it + 1) & 1] < ncols) {  // the next column's bounds, used when it starts
+        const int gn = column(s_tk[(it + 1) & 1]);
+        F = bounds(gn, in.inst + inst_of(in, gn), 0);
+      }
       // Popcount prefix over the non-empty words: thread t owns bitmap words
       // [t*per, t*per + per) (a power of two <= 32, inside one summary word);
       // `mine` holds which of them are non-empty.
@@ -777,13 +806,14 @@ cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_
   int slab_log2 = 10;
   while (slab_log2 < SLAB_BITS && ((int64_t)1 << slab_log2) < (int64_t)in.mmax) ++slab_log2;
   const size_t w64 = (size_t)1 << (slab_log2 - 6);
-  const size_t smem = w64 * 8 + ((w64 + 31) / 32) * 4 + 16;
+  const size_t bits = w64 * 8 + ((w64 + 31) / 32) * 4 + 16;
   const size_t nsw = (size_t)1 << (slab_log2 - 10);
   const size_t smem_c = nsw * 4 + (size_t)HEAVY_CAP * 4 + nsw * 8 + 16;
   // Small slabs: 256-thread blocks, several columns in flight per SM; a slab
   // bitmap that fills the SM: one 1024-thread block.
-  const bool small = smem * 2 + 4096 <= (size_t)dev.smem_per_sm / 2;
-  auto kern = small ? k_sym_heavy<256, 8> : k_sym_heavy<HEAVY_BLOCK, 8>;
+  const bool small = bits * 2 + 4096 <= (size_t)dev.smem_per_sm / 2;
+  const size_t smem = bits + (small ? sizeof(ItemMap<256>) : sizeof(ItemMap<HEAVY_BLOCK>));
+  auto kern = small ? k_sym_heavy<256> : k_sym_heavy<HEAVY_BLOCK>;
   auto kern_c = k_sym_heavy_compact<256, 8>;
   const int block = small ? 256 : HEAVY_BLOCK;
   int bf = 0, bc = 0;
