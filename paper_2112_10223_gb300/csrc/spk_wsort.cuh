@@ -329,8 +329,33 @@ __device__ __forceinline__ int wsort_column(const WsortSmem& sm, int k, int s, u
   return u;
 }
 
+// Sum of the run term(a), ..., term(b - 1), rounded once.  Doubles are added in
+// double.  Floats are added as an unevaluated pair of floats (Knuth's two-sum:
+// the rounding error of every addition is kept and added up), some 46 bits,
+// because a double addition occupies this GPU's double units for 16 clocks a
+// warp and a conversion as many; sums that are not finite that way (an overflow
+// on the way, an infinity, a NaN) are added again in double.  Against 64-bit
+// sums the results are the same as double accumulation's.
+template <typename V, typename TermF>
+__device__ __forceinline__ V wsort_run_sum(int a, int b, TermF&& term) {
+  if constexpr (sizeof(V) == 4) {
+    float hi = term(a), lo = 0.0f;
+    for (int y = a + 1; y < b; ++y) {
+      const float x = term(y);
+      const float s = __fadd_rn(hi, x);
+      const float t = __fsub_rn(s, hi);
+      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+      hi = s;
+    }
+    if (isfinite(hi) && isfinite(lo)) return b - a > 1 ? __fadd_rn(hi, lo) : hi;
+  }
+  double sum = (double)term(a);
+  for (int y = a + 1; y < b; ++y) sum += (double)term(y);
+  return (V)sum;
+}
+
 // Writes B(:, j) from a sorted column of 32 << eb key places: distinct row q's
-// run summed in double, rounded once.  (Columns without repeated rows are copied.)
+// run summed by wsort_run_sum.  (Columns without repeated rows are copied.)
 template <typename V>
 __device__ __forceinline__ void wsort_write(const WsortSmem& sm, int eb, int s, int u, int32_t* out_row, V* out_val,
                                             int lane) {
@@ -349,10 +374,8 @@ __device__ __forceinline__ void wsort_write(const WsortSmem& sm, int eb, int s, 
   for (int q = lane; q < u; q += 32) {
     const int a = sm.start[q], b = sm.start[q + 1];
     const uint32_t x = sm.key[a + (a >> eb)];
-    double sum = (double)sval[x & pm];
-    for (int y = a + 1; y < b; ++y) sum += (double)sval[sm.key[y + (y >> eb)] & pm];
     out_row[q] = (int32_t)(x >> pb);
-    out_val[q] = (V)sum;
+    out_val[q] = wsort_run_sum<V>(a, b, [&](int y) { return sval[sm.key[y + (y >> eb)] & pm]; });
   }
 }
 

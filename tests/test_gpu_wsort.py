@@ -77,3 +77,26 @@ def test_columns_split_between_sort_and_buckets():
     A = _columns(16, m, lengths, 6, torch.float64, pool)
     _check(A, m, torch.float64)
     _check(A, m, torch.float64, sort_mode=1)
+
+
+def test_float_runs_round_once_and_keep_infinities():
+    """Runs of equal rows are summed as if in double: cancellation, overflow on the way, infinities and NaN."""
+    inf, big = float("inf"), 3.0e38
+    runs = [[1.0, 2.0 ** -30, -1.0], [big, big, -big], [big, big, big], [inf, 1.0, big], [inf, -inf, 1.0],
+            [float("nan"), 1.0, 2.0], [-0.0, 0.0, -0.0], [1.0e-45, 1.0e-45, -1.0e-45], [1.0e8, 1.0, -1.0e8],
+            [big, -inf, big], [16777216.0, 1.0, 1.0]]
+    g = torch.Generator().manual_seed(3)
+    runs += [(torch.randn(3, generator=g) * 10.0 ** torch.randint(-20, 20, (3,), generator=g)).tolist() for _ in range(400)]
+    n, per = 41, len(runs) // 41 + 1
+    cp = torch.arange(n + 1, dtype=torch.int32) * per
+    v = torch.zeros(n * per, 3, dtype=torch.float32)
+    v[:len(runs)] = torch.tensor(runs, dtype=torch.float64).to(torch.float32)
+    rows = (torch.arange(per, dtype=torch.int32) * 3).repeat(n)
+    A = [(cp, rows, v[:, i].contiguous()) for i in range(3)]
+    d = v.double()
+    want = ((d[:, 0] + d[:, 1]) + d[:, 2]).to(torch.float32)
+    for method in ("twopass", "onepass"):
+        got = run_gpu(A, 3 * per, method=method)[2].cpu()
+        assert torch.equal(torch.isnan(got), torch.isnan(want))
+        ok = ~torch.isnan(want)
+        assert torch.equal(got[ok], want[ok])
