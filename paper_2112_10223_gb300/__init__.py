@@ -194,22 +194,35 @@ def _stream_ptr(stream):
     return stream, ctypes.c_void_p(stream.cuda_stream)
 
 
-def _csc_array(A, m: int, dtype):
-    """spkadd_csc descriptors of the inputs (and the tensors to keep alive)."""
-    arr = (CSC * len(A))()
-    keep = []
+def _check_inputs(A, dtype, where: str, dev: int | None, append) -> int:
+    """Checks the inputs' tensors, one pass, and appends every input's n, nnz and three addresses.
+
+    dev: index of the device they must be on (None: the first input's); returns it.  The attributes are read once
+    per tensor: a call with hundreds of inputs spends its host time here.
+    """
+    i32 = torch.int32
     for i, (cp, ri, va) in enumerate(A):
-        for t, dt in ((cp, torch.int32), (ri, torch.int32), (va, dtype)):
-            if t.dtype != dt or not t.is_cuda or not t.is_contiguous():
-                raise TypeError(f"input {i}: expected contiguous CUDA tensors (int32, int32, {dtype})")
-        arr[i].m = int(m)
-        arr[i].n = cp.numel() - 1
-        arr[i].nnz = ri.numel()
-        arr[i].col_ptr = cp.data_ptr()
-        arr[i].row_idx = ri.data_ptr() if ri.numel() else None
-        arr[i].val = va.data_ptr() if va.numel() else None
-        keep.append((cp, ri, va))
-    return arr, keep
+        d = cp.get_device()
+        if (d < 0 or ri.get_device() < 0 or va.get_device() < 0 or cp.dtype != i32 or ri.dtype != i32
+                or va.dtype != dtype or not (cp.is_contiguous() and ri.is_contiguous() and va.is_contiguous())):
+            raise TypeError(f"{where}input {i}: expected contiguous CUDA tensors (int32, int32, {dtype})")
+        if dev is None:
+            dev = d
+        if d != dev or ri.get_device() != dev or va.get_device() != dev:
+            raise TypeError("all inputs must be on one device")
+        nnz = ri.numel()
+        append((cp.numel() - 1, nnz, cp.data_ptr(), ri.data_ptr() if nnz else 0, va.data_ptr() if va.numel() else 0))
+    return dev
+
+
+def _csc_array(A, m: int, dtype, dev: int | None = None):
+    """spkadd_csc descriptors of the inputs, the tensors to keep alive, and the device they are on."""
+    rows = []
+    dev = _check_inputs(A, dtype, "", dev, rows.append)
+    m = int(m)
+    flat = [x for n, nnz, c, r, v in rows for x in (m, n, nnz, c, r, v)]
+    arr = (ctypes.c_int64 * len(flat))(*flat)
+    return ctypes.cast(arr, ctypes.POINTER(CSC)), [tuple(a) for a in A], dev
 
 
 def spkadd_plan(A, m: int, dtype=None, stream=None, options: Options | None = None) -> Handle:
@@ -221,10 +234,8 @@ def spkadd_plan(A, m: int, dtype=None, stream=None, options: Options | None = No
     dtype = dtype or A[0][2].dtype
     if dtype not in _DTYPE:
         raise TypeError("values must be float32 or float64")
-    arr, keep = _csc_array(A, m, dtype)
+    arr, keep, _ = _csc_array(A, m, dtype)
     dev = A[0][0].device
-    if any(t.device != dev for a in A for t in a):
-        raise TypeError("all inputs must be on one device")
     with torch.cuda.device(dev):
         stream, sp = _stream_ptr(stream)
         h = ctypes.c_void_p()
@@ -405,33 +416,27 @@ def spkadd_batch_plan_raw(k, m, n, nnz, col_ptr, row_idx, val, dtypes, stream=No
 
 def spkadd_batch_plan(problems, stream=None, options: Options | None = None) -> BatchHandle:
     """spkadd_batch_plan over [(A, m), ...], each A a list of (col_ptr, row_idx, val) CUDA tensors."""
-    ks, ms, ns, nnz, cps, ris, vas, dts, keep = [], [], [], [], [], [], [], [], []
+    ks, ms, ns, dts, keep, rows = [], [], [], [], [], []
+    dev = None
     for q, (A, m) in enumerate(problems):
         if len(A) == 0:
             _check(1, "spkadd_batch_plan")
         dtype = A[0][2].dtype
         if dtype not in _DTYPE:
             raise TypeError("values must be float32 or float64")
+        at = len(rows)
+        dev = _check_inputs(A, dtype, f"problem {q} ", dev, rows.append)
+        n = rows[at][0]
+        if any(r[0] != n for r in rows[at:]):
+            _check(2, "spkadd_batch_plan")
         ks.append(len(A))
         ms.append(int(m))
-        ns.append(A[0][0].numel() - 1)
+        ns.append(n)
         dts.append(dtype)
-        for i, (cp, ri, va) in enumerate(A):
-            for t, dt in ((cp, torch.int32), (ri, torch.int32), (va, dtype)):
-                if t.dtype != dt or not t.is_cuda or not t.is_contiguous():
-                    raise TypeError(f"problem {q} input {i}: expected contiguous CUDA tensors (int32, int32, {dtype})")
-            if cp.numel() - 1 != ns[-1]:
-                _check(2, "spkadd_batch_plan")
-            nnz.append(ri.numel())
-            cps.append(cp.data_ptr())
-            ris.append(ri.data_ptr() if ri.numel() else 0)
-            vas.append(va.data_ptr() if va.numel() else 0)
         keep.append(A)
-    dev = problems[0][0][0][0].device
-    if any(t.device != dev for A, _ in problems for a in A for t in a):
-        raise TypeError("all problems must be on one device")
+    _, nnz, cps, ris, vas = zip(*rows)
     return spkadd_batch_plan_raw(ks, ms, ns, nnz, cps, ris, vas, dts, stream=stream, options=options, keep=keep,
-                                 device=dev)
+                                 device=problems[0][0][0][0].device)
 
 
 def spkadd_batch_symbolic(h: BatchHandle) -> list:
@@ -527,8 +532,8 @@ class SpkaddStream:
         """B <- B + sum(A); returns nnz(B)."""
         if len(A) == 0:
             _check(1, "spkadd_stream_add")
-        arr, keep = _csc_array(A, self.m, self.dtype)
-        if any(t.device != self.device for a in A for t in a):
+        arr, keep, dev = _csc_array(A, self.m, self.dtype)
+        if torch.device("cuda", dev) != self.device:
             raise TypeError(f"inputs must be on {self.device}")
         with torch.cuda.device(self.device):
             _check(library().spkadd_stream_add(self.ptr, len(A), arr), "spkadd_stream_add")
