@@ -114,16 +114,20 @@ __global__ void __launch_bounds__(BLOCK) k_sym_cta(Inputs in, const int32_t* __r
 // Against the open-addressing table of k_sym_cta (a probe loop per entry, a
 // five-shuffle segment search): 131072 columns of 2048 entries 1.64 -> 0.80 ms,
 // R-MAT scale 20 1.11 -> 0.72 ms.  The table stays for more than 2^20 rows.
-constexpr int SYM_BLOCK = 256;
+// Threads per block of the flat form: what an item costs beyond its entries
+// (table, map, barriers: some 220 instructions a warp) is paid by fewer warps.
+// (256 threads: 65537 unordered columns 855 against 833 us, a batch of 20 1069
+// against 1042; 131072 columns of 2048 entries the same.)
+constexpr int SYM_BLOCK = 128;
 constexpr int SYM_FLAT_LOG2 = 18;  // 32 KB of bits
 
-template <bool WIDE>
-__global__ void __launch_bounds__(SYM_BLOCK, 5) k_sym_items(Inputs in, const int32_t* __restrict__ list,
+template <bool WIDE, int B>
+__global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int32_t* __restrict__ list,
                                                              const Counters* __restrict__ ctr,
                                                              int32_t* __restrict__ u_out, Window* __restrict__ win,
                                                              int64_t win_cap, int words, const int32_t* __restrict__ s_arr,
                                                              int32_t* __restrict__ dup_list, Counters* ctr_w) {
-  constexpr int B = SYM_BLOCK;
+  static_assert(!WIDE || B == 256, "four summary words a thread");
   using Map = ItemMap<B>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   Map& M = *reinterpret_cast<Map*>(sm_raw);
@@ -771,14 +775,16 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
   if (in.mmax <= (1 << SLAB_BITS)) {
     const bool wide = in.mmax > (1 << SYM_FLAT_LOG2);
     const int words = pow2_at_least((in.mmax + 31) / 32);  // (few sizes: their occupancy is looked up once)
-    const size_t smem = sizeof(ItemMap<SYM_BLOCK>) + (wide ? (1024 + CTA_MAX_LIMIT) * 4 + 1024 * 2 : (size_t)words * 4);
-    auto kern = wide ? k_sym_items<true> : k_sym_items<false>;
-    const int bps = resident_blocks((const void*)kern, SYM_BLOCK, smem);
-    if (bps < 1) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<dev.sms * bps, SYM_BLOCK, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup_list, ctr_w);
-    return cudaGetLastError();
+    auto go = [&](auto kern, int block, size_t smem) {
+      const int bps = resident_blocks((const void*)kern, block, smem);
+      if (bps < 1) return cudaErrorInvalidConfiguration;
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      kern<<<dev.sms * bps, block, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup_list, ctr_w);
+      return cudaGetLastError();
+    };
+    if (wide) return go(k_sym_items<true, 256>, 256, sizeof(ItemMap<256>) + (1024 + CTA_MAX_LIMIT) * 4 + 1024 * 2);
+    return go(k_sym_items<false, SYM_BLOCK>, SYM_BLOCK, sizeof(ItemMap<SYM_BLOCK>) + (size_t)words * 4);
   }
   constexpr int BLOCK = 512;
   const int tmax = pow2_at_least(2 * cta_max);
