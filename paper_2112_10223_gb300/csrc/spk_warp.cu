@@ -764,6 +764,113 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
   if (!NUMERIC && lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
 }
 
+// Symbolic count of light columns of few rows: one bit per row in a bitmap of the
+// warp's own, no sort; u_j is the number of bits its entries are first to set.
+// It waits for its loads; the bitmap's size costs warps and its clearing 64
+// wavefronts.  Against the sort: 65536 columns of 256 to 384 entries, m = 2^16,
+// four times, 0.62 -> 0.50 ms; a batch of 20 (m up to 2^14) 87 -> 55 us; m = 65537
+// (10 KB a warp) 44 -> 54 us, so 8 KB is the limit; R-MAT scale 14, whose columns
+// are mostly short, 18 -> 20 us, so short means are left to the sort.
+constexpr int WBITS_MAX_ROWS = 1 << 16;
+constexpr int WBITS_MIN_MEAN = 48;
+
+__host__ __device__ constexpr int wbits_words(int m) { return ((m + 31) / 32 + 127) / 128 * 128; }
+
+template <bool BATCH, bool RES, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_warp_bits(Inputs in, WarpColArgs a, int words) {
+  struct Head {
+    ulonglong2 seg[WSORT_KT];
+    uint2 blk[16];
+  };
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned char* base = sm_raw + (size_t)wid * (sizeof(Head) + (size_t)words * 4);
+  Head& H = *reinterpret_cast<Head*>(base);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(base + sizeof(Head));
+  for (int x = lane; x < words / 4; x += 32) reinterpret_cast<uint4*>(bits)[x] = make_uint4(0u, 0u, 0u, 0u);
+  if (lane < 16) H.blk[lane].x = 0u;
+  __syncwarp();
+  const int nbig = a.ctr->n_wbig;
+  const int ncols = a.ctr->n_warp + nbig;
+  const int k0 = in.inst[0].k, m0 = in.inst[0].m;
+  if (RES && (BATCH || k0 > 32)) {  // the host never launches this; never index lanes past k
+    if (threadIdx.x == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
+    return;
+  }
+  const int32_t* my_cp = nullptr;
+  const int32_t* my_ri = nullptr;
+  if (RES && lane < k0) {
+    my_cp = in.cp[lane];
+    my_ri = in.ri[lane];
+  }
+  const int stride = gridDim.x * WARPS;
+  int c = blockIdx.x * WARPS + wid;
+  ColState cur = load_col<false, BATCH>(in, a, c, ncols, RES, my_cp, lane, k0, nbig);
+  ColState nxt = load_col<false, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig);
+  int n_unique = 0, n_bucket = 0;
+  for (; cur.g >= 0; c += stride, cur = nxt,
+                     nxt = load_col<false, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig)) {
+    const Inst* I = in.inst + cur.q;
+    const int k = BATCH ? I->k : k0;
+    const int off = BATCH ? I->ptr_off : 0;
+    const int j = BATCH ? cur.g - I->colbase : cur.g;
+    const uint32_t m = (uint32_t)(BATCH ? I->m : m0);
+    auto bounds = [&](int i, WsortIn<float>& x) {
+      if (RES) {
+        x = WsortIn<float>{cur.beg, cur.len, my_ri, nullptr};
+      } else {
+        const int32_t* cp = in.cp[off + i];
+        x.beg = __ldg(cp + j);
+        x.len = __ldg(cp + j + 1) - x.beg;
+        x.rp = in.ri[off + i];
+      }
+    };
+    int fresh = 0;
+    bool bad = false;
+#pragma unroll 1
+    for (int cb = 0; cb < k; cb += WSORT_KT) {
+      const int nk = min(WSORT_KT, k - cb);
+      int total;
+      WsortIn<float> seg[2];
+      wsort_bounds<float>(seg, cb, nk, bounds, lane);
+      const uint32_t magic = wsort_table<float, false>(H.seg, H.blk, seg, nk, &total, lane);
+      __syncwarp();
+      constexpr int G = 8;
+#pragma unroll 1
+      for (int e0 = 0; e0 < total; e0 += 32 * G) {
+        uint32_t r[G];
+#pragma unroll
+        for (int t = 0; t < G; ++t) {  // (a lane past the end repeats the last entry)
+          const int e = min(e0 + 32 * t + lane, total - 1);
+          r[t] = (uint32_t)__ldg(reinterpret_cast<const int32_t*>(H.seg[wsort_seg(H.blk, magic, e)].x) + e);
+        }
+#pragma unroll
+        for (int t = 0; t < G; ++t) {
+          if (e0 + 32 * t >= total) break;  // (warp-uniform)
+          const uint32_t x = min(r[t], m - 1u), bit = 1u << (x & 31u);
+          bad = bad || r[t] >= m;
+          fresh += !(atomicOr(&bits[x >> 5], bit) & bit);
+        }
+      }
+      __syncwarp();
+      if (!magic && lane < 16) H.blk[lane].x = 0u;
+      __syncwarp();
+    }
+    const int used = wbits_words((int)m) / 4;
+    for (int x = lane; x < used; x += 32) reinterpret_cast<uint4*>(bits)[x] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    const int u = __reduce_add_sync(SPK_FULL, fresh);
+    if (__any_sync(SPK_FULL, bad) && lane == 0) atomicOr(&a.ctr_w->err, ERR_RANGE);  // B is never computed
+    if (lane == 0) {
+      a.u_out[cur.g] = u;
+      n_unique += u == cur.s;
+      n_bucket += bucket_column(cur.s, u, true);
+    }
+  }
+  if (lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
+  if (lane == 0 && n_bucket) atomicAdd(&a.ctr_w->n_bucket, n_bucket);
+}
+
 // ---------------------------------------------------------------------------
 // One pass over the inputs (spkadd_onepass).  Sec. II-D's symbolic phase exists
 // so that B can be allocated before the numeric phase; here B goes into
@@ -1093,6 +1200,23 @@ static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max
     e = cudaGetLastError();
     ++*launches;
   };
+  if constexpr (!NUMERIC) {
+    if (in.mmax <= WBITS_MAX_ROWS && in.mean_s >= WBITS_MIN_MEAN) {
+      constexpr int BW = 4;
+      const int words = wbits_words(pow2_at_least(in.mmax) < WBITS_MAX_ROWS ? pow2_at_least(in.mmax) : WBITS_MAX_ROWS);
+      const size_t smem = BW * (WSORT_KT * sizeof(ulonglong2) + 16 * sizeof(uint2) + (size_t)words * 4);
+      auto kern = in.col_inst ? k_warp_bits<true, false, BW>
+                  : in.kmax <= 32 ? k_warp_bits<false, true, BW>
+                                  : k_warp_bits<false, false, BW>;
+      const int bps = resident_blocks((const void*)kern, BW * 32, smem);
+      if (bps < 1) return cudaErrorInvalidConfiguration;
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      kern<<<dev.sms * bps, BW * 32, smem, st>>>(in, a, words);
+      ++*launches;
+      return cudaGetLastError();
+    }
+  }
   const bool sort = in.mmax <= (1 << WSORT_ROW_BITS);
   // (Only k_warp_sort leaves every column without repeats as it is when B may be unsorted.)
   a.split = sort && in.split_warp && a.smax > WARP_SMALL && !a.unsorted_out;

@@ -28,7 +28,7 @@ def _check(A, m, dtype, **opt):
 
 
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
-@pytest.mark.parametrize("m", [600, 65537, 1 << 23, (1 << 23) + 1])  # keys hold rows below 2^23
+@pytest.mark.parametrize("m", [600, 1 << 16, 65537, 1 << 23, (1 << 23) + 1])  # bitmaps 2^16 rows, keys below 2^23
 def test_key_counts_and_row_limits(m, dtype):
     A = _columns(29, m, LENGTHS, 4, dtype)
     _check(A, m, dtype)
