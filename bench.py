@@ -409,9 +409,10 @@ def kernel_label(info, method):
     if method == "onepass" and info.get("onepass"):
         return "k_warp_onepass (spkadd_onepass)"
     if info["cols_cta"] + info["cols_heavy"] == 0:
-        return "k_warp_col<numeric> (spkadd_numeric)"
-    return ("spkadd_numeric: k_warp_col<numeric> and the thread-block items' kernel "
-            "(k_num_compact or k_num_bitmap)")
+        mean = info["nnz_in"] / max(info["n"], 1)  # the library's rule (few repeats expected: buckets, else sorted)
+        return ("k_warp_col" if mean >= 64 and 2 * mean * mean <= info["m"] else "k_warp_sort") + \
+            "<numeric> (spkadd_numeric)"
+    return ("spkadd_numeric: k_warp_sort or k_warp_col, k_num_items and k_num_dup")
 
 
 def run_ours(args, world, rank, local):

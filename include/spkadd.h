@@ -62,7 +62,7 @@ typedef enum spkadd_status {
     SPKADD_ERR_OVERFLOW = 5,        /* m or n >= 2^31, or a column's input count >= 2^31 */
     SPKADD_ERR_NOMEM = 6,           /* the workspace allocation failed */
     SPKADD_ERR_CUDA = 7,            /* a CUDA runtime call or kernel launch failed */
-    SPKADD_ERR_TIMEOUT = 8,         /* a bounded device wait gave up */
+    SPKADD_ERR_TIMEOUT = 8,         /* a bounded device wait gave up (one pass: opt.wait_timeout_ms; scan: 60 s) */
     SPKADD_ERR_STATE = 9,           /* call out of order */
     SPKADD_ERR_UNSUPPORTED = 10,    /* valid request this library does not handle (e.g. k > SPKADD_MAX_K) */
     SPKADD_ERR_INTERNAL = 11        /* a device-side size invariant failed; the result is not valid */
@@ -121,8 +121,8 @@ typedef struct spkadd_options {
      * (range 1024..4096). */
     int32_t window_max;
     /* 0 = default: every column of B sorted by row.
-     * 1 = as 0, but warp-class columns always take the duplicate-merging
-     *     path of the numeric pass, even when the symbolic pass found no
+     * 1 = as 0, but warp-class columns summed in buckets take the
+     *     duplicate-merging path even when the symbolic pass found no
      *     repeated row (a test and diagnosis switch; results are the same).
      * 2 = rows of a column of B may come in any order (Alg. 5 sorts only
      *     when sorted output is wanted): warp-class columns without repeated
@@ -144,8 +144,9 @@ typedef struct spkadd_options {
      * per 32-row word plus a table of only the non-empty words, so shared
      * memory follows window_max (numeric) or a fixed table size
      * (symbolic: the slab is cut into sub-ranges that fit), not m.
-     * 0 = automatic: numeric items take the layout with more resident
-     * blocks per SM; the heavy symbolic count takes the flat bitmap. */
+     * 0 = automatic: numeric items take the flat bitmap for row ranges of at
+     * most 2^17 and the compact table above, or, with few distinct rows, a
+     * hash table; the heavy symbolic count takes the flat bitmap. */
     int32_t block_accumulator;
     /* Workspace allocator.  NULL alloc: cudaMallocAsync / cudaFreeAsync on
      * the plan's stream.  Otherwise alloc(bytes, stream, ctx) must return

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int32_t* __rest
 // before it.  scan_buf: the ticket counter, then one look-back word per tile,
 // zero at launch.  The tile taken first also turns the columns of the dup list
 // into window records when there are too few of them for k_num_dup.
-constexpr unsigned long long SCAN_WAIT_NS = 2000000000ull;
+constexpr unsigned long long SCAN_WAIT_NS = 60000000000ull;  // bound of a look-back wait (they last microseconds)
 
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int32_t* __restrict__ u, int n, int tiles,
                                                           unsigned long long* __restrict__ scan_buf,

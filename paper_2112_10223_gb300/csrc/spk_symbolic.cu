@@ -117,7 +117,9 @@ __global__ void __launch_bounds__(BLOCK) k_sym_cta(Inputs in, const int32_t* __r
 // Threads per block of the flat form: what an item costs beyond its entries
 // (table, map, barriers: some 220 instructions a warp) is paid by fewer warps.
 // (256 threads: 65537 unordered columns 855 against 833 us, a batch of 20 1069
-// against 1042; 131072 columns of 2048 entries the same.)
+// against 1042; 131072 columns of 2048 entries the same.)  Bitmaps of more than
+// 2^17 rows leave shared memory for five blocks: those have 256 threads (R-MAT
+// scale 18: 310 against 402 us).
 constexpr int SYM_BLOCK = 128;
 constexpr int SYM_FLAT_LOG2 = 18;  // 32 KB of bits
 
@@ -784,6 +786,7 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
       return cudaGetLastError();
     };
     if (wide) return go(k_sym_items<true, 256>, 256, sizeof(ItemMap<256>) + (1024 + CTA_MAX_LIMIT) * 4 + 1024 * 2);
+    if (words > (1 << 12)) return go(k_sym_items<false, 256>, 256, sizeof(ItemMap<256>) + (size_t)words * 4);
     return go(k_sym_items<false, SYM_BLOCK>, SYM_BLOCK, sizeof(ItemMap<SYM_BLOCK>) + (size_t)words * 4);
   }
   constexpr int BLOCK = 512;
