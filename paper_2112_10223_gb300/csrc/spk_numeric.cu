@@ -746,24 +746,37 @@ __global__ void __launch_bounds__(B, B == CTA_ITEM_BLOCK ? 4 : 2)
   if (threadIdx.x < sizeof(Window) / 4)
     reinterpret_cast<int32_t*>(sm.win)[threadIdx.x] = reinterpret_cast<const int32_t*>(win + wi)[threadIdx.x];
   __syncthreads();
-  ItemBounds<B> F;
-  {
-    const Window& W = sm.win[0];
+  auto bounds = [&](const Window& W) {
     const Inst* I = in.inst + inst_of(in, W.col);
     const int j = W.col - I->colbase, off = I->ptr_off;
     auto seg = [&](int i, int* beg, int* end) { window_seg(in, W, offs, off, j, i, beg, end); };
-    F = item_bounds<B>(0, min(I->k, ItemMap<B>::KT), seg);
-  }
+    return item_bounds<B>(0, min(I->k, ItemMap<B>::KT), seg);
+  };
+  ItemBounds<B> F = bounds(sm.win[0]);
   for (int turn = 0;; turn ^= 1) {
     const Window& W = sm.win[turn];
     const int q = inst_of(in, W.col);
     const Inst* I = in.inst + q;
-    if ((only_dtype >= 0 && !item_selected(only_dtype, I)) || W.r_hi <= W.r_lo) {  // (cannot happen)
+    if (only_dtype >= 0 && !item_selected(only_dtype, I)) {  // (cannot happen)
       if (threadIdx.x == 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
       return;
     }
-    const int64_t out = col_ptr[W.col] - (in.col_inst ? col_ptr[I->colbase] : 0) + W.out_off;
     const bool more = wi + step < nwin;
+    if (W.r_hi <= W.r_lo) {
+      // An empty window: the column's last cut fell into the slab's last word.
+      // It writes nothing, but the items after it are still this block's.
+      if (threadIdx.x == 0 && W.u != 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
+      if (!more) break;
+      wi += step;
+      __syncthreads();  // every thread is past the item before, whose record is replaced
+      if (threadIdx.x < sizeof(Window) / 4)
+        reinterpret_cast<int32_t*>(sm.win + (turn ^ 1))[threadIdx.x] =
+            reinterpret_cast<const int32_t*>(win + wi)[threadIdx.x];
+      __syncthreads();
+      F = bounds(sm.win[turn ^ 1]);
+      continue;
+    }
+    const int64_t out = col_ptr[W.col] - (in.col_inst ? col_ptr[I->colbase] : 0) + W.out_off;
     reg_item<V, A, ACC == 1, WIDE, B>(in, more ? win + wi + step : nullptr, turn, F, offs, out_row_of(o, q) + out,
                                       static_cast<V*>(out_val_of(o, q)) + out, sm, slab_log2, flat_rows, ctr_w);
     if (!more) break;

@@ -91,3 +91,18 @@ def test_many_columns_on_few_rows(k, L, m, dtype):
         at = (cp[:-1].long()[col] + cp[1:].long()[col] - 1 - e)
         flipped.append((cp, ri[at], va[at]))
     check_full(flipped, m, dtype, exact=True, options=spk.default_options(input_order=1))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n, parts", [(3, 1), (200, 4), (1400, 1)])
+def test_empty_last_window(n, parts, dtype):
+    """The last cut (a multiple of 4032 distinct rows) falls into the last 64-row word, which leaves an empty
+    window behind it; with more items than resident blocks, those that follow it must still be summed."""
+    m, u = 1 << 18, parts * 4032 + 2
+    rows = torch.cat([torch.arange(u - 10, dtype=torch.int64) * ((m - 64) // (u - 10)), torch.arange(m - 10, m)])
+    ri = rows.to(torch.int32).cuda().repeat(n)
+    cp = torch.arange(n + 1, dtype=torch.int32, device="cuda") * u
+    va = torch.arange(u * n, device="cuda").remainder(1000).to(dtype)
+    B_cp, B_ri, B_va = spk.spkadd([(cp, ri, va), (cp, ri, va)], m)
+    assert torch.equal(B_cp, cp.to(torch.int64)) and torch.equal(B_ri, ri)
+    assert torch.equal(B_va, 2 * va)
