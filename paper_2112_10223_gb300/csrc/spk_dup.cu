@@ -302,8 +302,6 @@ static cudaError_t launch_dup(const Inputs& in, const DupArgs& a, const DeviceIn
   const size_t smem = WARPS * sizeof(DupSmem<A>);
   const int bps = resident_blocks((const void*)kern, WARPS * 32, smem);
   if (bps < 1) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int grid = dev.sms * bps;
   if (grid > (a.n + WARPS - 1) / WARPS) grid = (a.n + WARPS - 1) / WARPS;
   kern<<<grid, WARPS * 32, smem, st>>>(in, a);

@@ -24,8 +24,11 @@ struct DeviceInfo {
   int smem_per_sm;
 };
 
+// Lets the launches of kernel `fn` on the current device take any amount of
+// dynamic shared memory up to the opt-in limit (set once, never lowered).
+cudaError_t allow_smem(const void* fn);
 // Resident blocks per SM of kernel `fn` at `block` threads and `smem` bytes of
-// dynamic shared memory (sets the kernel's shared-memory limit to smem; cached).
+// dynamic shared memory, which its launches may then take (cached).
 // 0 on error.
 int resident_blocks(const void* fn, int block, size_t smem);
 

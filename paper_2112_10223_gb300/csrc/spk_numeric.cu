@@ -829,12 +829,41 @@ __global__ void __launch_bounds__(BLOCK) k_num_bitmap(Inputs in, const Window* _
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
+// Lets a kernel's launches on the current device ask for all the dynamic shared
+// memory that a block can have there.  The limit belongs to the kernel and the
+// device, not to a launch: it is set once, to a number that depends on nothing
+// else, so host threads launching the same kernel with other sizes never lower
+// it under one another.
+cudaError_t allow_smem(const void* fn) {
+  struct Entry {
+    int dev;
+    const void* fn;
+  };
+  static std::mutex mu;
+  static Entry done[512];
+  static int ndone = 0;
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < ndone; ++i)
+    if (done[i].fn == fn && done[i].dev == dev) return cudaSuccess;
+  cudaFuncAttributes fa;
+  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess && ndone < 512) done[ndone++] = Entry{dev, fn};
+  return e;
+}
+
 // Resident blocks per SM of a kernel at a block size and dynamic shared
 // memory size (registers, shared memory and threads all counted), or 0 on
-// error.  Cached: the query is not free.  The launch sets the kernel's
-// shared-memory limit itself (another size may have been set since).
+// error; its launches may then ask for that size.  Cached per device: the
+// query is not free.
 int resident_blocks(const void* fn, int block, size_t smem) {
   struct Entry {
+    int dev;
     const void* fn;
     int block;
     size_t smem;
@@ -843,16 +872,21 @@ int resident_blocks(const void* fn, int block, size_t smem) {
   static std::mutex mu;
   static Entry cache[256];
   static int ncache = 0;
-  std::lock_guard<std::mutex> lock(mu);
-  for (int i = 0; i < ncache; ++i)
-    if (cache[i].fn == fn && cache[i].block == block && cache[i].smem == smem) return cache[i].blocks;
-  int b = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, block, smem) != cudaSuccess) {
+  int dev = 0, b = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
     (void)cudaGetLastError();  // not sticky: leave no stale error for the next check
     return 0;
   }
-  if (b > 0 && ncache < 256) cache[ncache++] = Entry{fn, block, smem, b};
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < ncache; ++i)
+    if (cache[i].fn == fn && cache[i].block == block && cache[i].smem == smem && cache[i].dev == dev)
+      return cache[i].blocks;
+  if (allow_smem(fn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, block, smem) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  if (b > 0 && ncache < 256) cache[ncache++] = Entry{dev, fn, block, smem, b};
   return b;
 }
 
@@ -869,8 +903,6 @@ static cudaError_t launch_items(K kern, int block, int blocks_per_sm, const Inpu
                                 const int32_t* offs, const int64_t* col_ptr, const Outs& out, int slab_log2, int umax,
                                 size_t smem, int only_dtype, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
   if (blocks_per_sm < 1) return cudaErrorInvalidConfiguration;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int grid = dev.sms * blocks_per_sm;
   if (grid > n_win) grid = n_win;
   if (grid < 1) return cudaSuccess;
@@ -886,8 +918,6 @@ static cudaError_t launch_reg_items(const Inputs& in, const Window* win, int n_w
   const size_t smem = ItemLayout<WIDE, B>(slab_log2, umax, (DT == 1 || ACC == 2) ? 8 : 4).bytes();
   const int bps = resident_blocks((const void*)kern, B, smem);
   if (bps < 1) return cudaErrorInvalidConfiguration;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int grid = dev.sms * bps;
   if (grid > n_win) grid = n_win;
   if (grid < 1) return cudaSuccess;

@@ -780,8 +780,6 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
     auto go = [&](auto kern, int block, size_t smem) {
       const int bps = resident_blocks((const void*)kern, block, smem);
       if (bps < 1) return cudaErrorInvalidConfiguration;
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
       kern<<<dev.sms * bps, block, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup_list, ctr_w);
       return cudaGetLastError();
     };
@@ -793,7 +791,7 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
   const int tmax = pow2_at_least(2 * cta_max);
   const size_t smem = (size_t)tmax * sizeof(int32_t);
   auto kern = k_sym_cta<BLOCK, 4>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem((const void*)kern);
   if (e != cudaSuccess) return e;
   const int grid = dev.sms * blocks_per_sm(dev, smem, BLOCK);
   kern<<<grid, BLOCK, smem, st>>>(in, list, s, ctr, u, win, win_cap, tmax, ctr_w);
@@ -830,16 +828,12 @@ cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_
   if (accumulator == 2) bc = resident_blocks((const void*)kern_c, 256, smem_c);
   if (accumulator == 2) {
     if (bc < 1) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(kern_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
-    if (e != cudaSuccess) return e;
     // Windows end on 32-row words: a window holds at most win_target + 31 rows.
     kern_c<<<dev.sms * bc, 256, smem_c, st>>>(in, list, s, ctr, u, win, search_list, win_cap, window_max - 64,
                                              slab_log2, HEAVY_CAP, ctr_w);
     return cudaGetLastError();
   }
   if (bf < 1) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   // Windows end on 64-row words: a window holds at most win_target + 63 rows.
   kern<<<dev.sms * bf, block, smem, st>>>(in, list, s, ctr, u, win, search_list, win_cap, window_max - 64, slab_log2,
                                           dup_list, ctr_w);

@@ -1191,8 +1191,6 @@ static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max
       e = cudaErrorInvalidConfiguration;
       return;
     }
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return;
     int grid = dev.sms * bps;
     if (n_cols >= 0 && grid > (n_cols + warps - 1) / warps) grid = (n_cols + warps - 1) / warps;
     if (grid < 1) return;
@@ -1210,8 +1208,6 @@ static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max
                                   : k_warp_bits<false, false, BW>;
       const int bps = resident_blocks((const void*)kern, BW * 32, smem);
       if (bps < 1) return cudaErrorInvalidConfiguration;
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
       kern<<<dev.sms * bps, BW * 32, smem, st>>>(in, a, words);
       ++*launches;
       return cudaGetLastError();
@@ -1310,8 +1306,6 @@ static cudaError_t launch_onepass_t(const Inputs& in, OnepassArgs a, int warp_ma
   }
   const int occ = resident_blocks((const void*)kern, WARPS * 32, smem);
   if (occ < 1) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   int grid = dev.sms * occ;
   if (grid > a.ntiles) grid = a.ntiles;
   *grid_out = grid;
