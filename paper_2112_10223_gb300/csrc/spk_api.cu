@@ -138,7 +138,7 @@ struct spkadd_handle {
   void** d_out_tab = nullptr;          // batch: B row / value / col_ptr pointer tables
   int32_t *d_s = nullptr, *d_u = nullptr;
   int32_t *d_wl = nullptr, *d_cl = nullptr, *d_hl = nullptr;
-  int32_t* d_dup = nullptr;   // columns for k_num_dup
+  spk::DupList dup{};         // columns for k_num_dup
   Window* d_win = nullptr;
   int32_t* d_search = nullptr;
   int64_t win_cap = 0;
@@ -308,7 +308,8 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   const size_t o_hl = cv.take<int32_t>(2 * ncols);
   // Columns for k_num_dup (never more than nnz / (warp_max + 1) columns are above the warp class).
   const bool dup = o.block_accumulator == 0 && mmax <= (1 << spk::DUP_ROW_BITS);
-  const size_t o_dup = cv.take<int32_t>(!dup ? 0 : ncols < nnz_in / (o.warp_max + 1) ? ncols : nnz_in / (o.warp_max + 1));
+  const int64_t dup_cap = !dup ? 0 : ncols < nnz_in / (o.warp_max + 1) ? ncols : nnz_in / (o.warp_max + 1);
+  const size_t o_dup = cv.take<int32_t>(dup_cap);
   const size_t o_win = cv.take<Window>(win_cap);
   const size_t o_srch = cv.take<int32_t>(win_cap);
   const int cta_kinds = spk::num_cta_kinds(any32 && any64 ? 2 : (any64 ? 1 : 0), f32_kinds);
@@ -332,7 +333,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   h->d_wl = reinterpret_cast<int32_t*>(h->ws + o_wl);
   h->d_cl = reinterpret_cast<int32_t*>(h->ws + o_cl);
   h->d_hl = reinterpret_cast<int32_t*>(h->ws + o_hl);
-  h->d_dup = dup ? reinterpret_cast<int32_t*>(h->ws + o_dup) : nullptr;
+  h->dup = spk::DupList{dup ? reinterpret_cast<int32_t*>(h->ws + o_dup) : nullptr, (int32_t)dup_cap};
   h->d_win = reinterpret_cast<Window*>(h->ws + o_win);
   h->d_search = reinterpret_cast<int32_t*>(h->ws + o_srch);
   h->d_wsort = __builtin_popcount(cta_kinds) > 1 ? reinterpret_cast<Window*>(h->ws + o_ws) : nullptr;
@@ -448,16 +449,16 @@ static spkadd_status run_symbolic(spkadd_handle* h) {
   int warp_launches = 0;
   if (h->ncols > 0) {
     ce = spk::launch_sym_heavy(h->in, h->d_hl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->d_search, h->win_cap, h->d_ctr,
-                               h->opt.window_max, h->opt.block_accumulator, h->d_dup, h->dev, h->st);
+                               h->opt.window_max, h->opt.block_accumulator, h->dup, h->dev, h->st);
     if (ce == cudaSuccess)
       ce = spk::launch_sym_cta(h->in, h->d_cl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->win_cap, h->d_ctr,
-                               h->opt.cta_max, h->d_dup, h->dev, h->st);
+                               h->opt.cta_max, h->dup, h->dev, h->st);
     if (ce == cudaSuccess)
       ce = spk::launch_sym_warp(h->in, h->d_wl, h->d_s, h->d_ctr, h->d_u, h->opt.warp_max, h->d_ctr, h->dev, h->st,
                                 &warp_launches);
     h->launches += 2 + warp_launches;
   }
-  if (ce == cudaSuccess) ce = spk::launch_scan_fused(h->in, h->d_u, h->d_scan, h->d_colptr, h->d_dup, h->d_win, h->win_cap,
+  if (ce == cudaSuccess) ce = spk::launch_scan_fused(h->in, h->d_u, h->d_scan, h->d_colptr, h->dup, h->d_win, h->win_cap,
                                                      h->d_ctr, h->st);
   h->launches += 1;
   // Several problem kinds: the thread-block items grouped by kind for the numeric launches.
@@ -540,7 +541,7 @@ static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
                              h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
   h->launches += item_launches;
   if (ce == cudaSuccess && h->h_ctr.n_dup > 0) {
-    ce = spk::launch_num_dup(h->in, spk::num_cta_kinds(h->dt_mode, h->f32_kinds), h->d_dup, h->h_ctr.n_dup, h->d_s,
+    ce = spk::launch_num_dup(h->in, spk::num_cta_kinds(h->dt_mode, h->f32_kinds), h->dup.cols, h->h_ctr.n_dup, h->d_s,
                              h->d_u, h->d_colptr, out, h->d_ctr, h->dev, h->st, &item_launches);
     h->launches += item_launches;
   }

@@ -62,6 +62,20 @@ constexpr int DUP_ROW_BITS = 23;  // rows below 2^23: a row and its table slot s
 constexpr int DUP_MIN_COLS = 8192;
 __host__ __device__ constexpr bool dup_column(int64_t s, int u) { return u <= DUP_MAX_U && s >= (int64_t)DUP_RATIO * u; }
 
+// The columns given to k_num_dup, Counters::n_dup of them.
+struct DupList {
+  int32_t* cols;  // null: none are set apart
+  int32_t cap;    // entries cols holds
+};
+
+// Lists column g (one thread).  The list is sized by the inputs' nnz: column
+// pointers that disagree with it leave an error, never a write past the list.
+__device__ __forceinline__ void dup_append(const DupList& d, int g, Counters* ctr_w) {
+  const int at = atomicAdd(&ctr_w->n_dup, 1);
+  if (at < d.cap) d.cols[at] = g;
+  else atomicOr(&ctr_w->err, ERR_WINDOW_CAP);
+}
+
 // Float sums.  A float sum of t terms, in any order, errs by at most
 // (t - 1) 2^-24 sum|terms| (first order), within 1e-5 sum|terms| for
 // t <= FP32_ACC_TERMS.  Thread-block accumulators of problems with k <= 167

@@ -9,6 +9,7 @@ namespace spk {
 
 struct Inputs;
 struct Outs;
+struct DupList;
 struct Counters;
 struct Window;
 
@@ -44,9 +45,9 @@ cudaError_t launch_validate(const Inputs& in, const int64_t* nnz, Counters* ctr,
 size_t scan_tiles(int64_t n);
 cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* col_ptr, cudaStream_t st);
 // The same scan in one launch over words that launch_bin zeroed.  Columns of the
-// dup list (may be null) also become window records when they are few.
+// dup list also become window records when they are few.
 cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
-                              const int32_t* dup_list, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st);
+                              const DupList& dup, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st);
 // Loads the scan kernels onto the current device (module loading is lazy).
 cudaError_t load_scan_kernels();
 cudaError_t launch_window_search(const Inputs& in, const Window* win, const int32_t* search_list, int n_search,
@@ -56,13 +57,13 @@ cudaError_t launch_sym_warp(const Inputs& in, const int32_t* list, const int32_t
                             int32_t* u, int warp_max, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
                             int* launches);
 cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
-                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, int32_t* dup_list,
+                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, const DupList& dup,
                            const DeviceInfo& dev, cudaStream_t st);
 cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
                              Window* win,
                              int32_t* search_list, int64_t win_cap, Counters* ctr_w, int window_max,
-                             int accumulator, int32_t* dup_list, const DeviceInfo& dev, cudaStream_t st);
-// (dup_list: where columns for launch_num_dup go, Counters::n_dup of them; null: none are set apart.)
+                             int accumulator, const DupList& dup, const DeviceInfo& dev, cudaStream_t st);
+// (dup: where columns for launch_num_dup go, Counters::n_dup of them.)
 
 // dt: 0 = every problem float, 1 = every problem double, 2 = mixed batch.
 // Counters after the symbolic phase: n_small and n_big warp columns, n_bucket of these k_warp_col's where they are split.

@@ -222,8 +222,7 @@ constexpr unsigned long long SCAN_WAIT_NS = 60000000000ull;  // bound of a look-
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int32_t* __restrict__ u, int n, int tiles,
                                                           unsigned long long* __restrict__ scan_buf,
                                                           int64_t* __restrict__ col_ptr,
-                                                          const int32_t* __restrict__ dup_list,
-                                                          Window* __restrict__ win, int64_t win_cap,
+                                                          DupList dup, Window* __restrict__ win, int64_t win_cap,
                                                           Counters* __restrict__ ctr) {
   __shared__ long long tmp[33];
   __shared__ long long s_off;
@@ -262,11 +261,11 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int3
     if (j < n) col_ptr[j] = run;
     run += v[t];
   }
-  if (tile == 0 && dup_list) {
+  if (tile == 0 && dup.cols) {
     const int nd = ctr->n_dup, nw = ctr->n_windows, cap = (int)(win_cap - ctr->n_hwin);
-    if (nd > 0 && nd < DUP_MIN_COLS) {
+    if (nd > 0 && nd < DUP_MIN_COLS && nd <= dup.cap) {  // (past cap: the error is set)
       for (int x = threadIdx.x; x < nd; x += SCAN_BLOCK) {
-        const int g = dup_list[x];
+        const int g = dup.cols[x];
         Window w;
         w.col = g;
         w.r_lo = 0;
@@ -416,11 +415,11 @@ cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* c
 }
 
 cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
-                              const int32_t* dup_list, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st) {
+                              const DupList& dup, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st) {
   int tiles = (int)(((int64_t)in.ncols + SCAN_TILE - 1) / SCAN_TILE);
   if (tiles < 1) tiles = 1;
   k_scan_fused<<<tiles, SCAN_BLOCK, 0, st>>>(in, u, in.ncols, tiles, reinterpret_cast<unsigned long long*>(scan_buf),
-                                            col_ptr, dup_list, win, win_cap, ctr);
+                                            col_ptr, dup, win, win_cap, ctr);
   return cudaGetLastError();
 }
 

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
                                                              const Counters* __restrict__ ctr,
                                                              int32_t* __restrict__ u_out, Window* __restrict__ win,
                                                              int64_t win_cap, int words, const int32_t* __restrict__ s_arr,
-                                                             int32_t* __restrict__ dup_list, Counters* ctr_w) {
+                                                             DupList dup, Counters* ctr_w) {
   static_assert(!WIDE || B == 256, "four summary words a thread");
   using Map = ItemMap<B>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -272,9 +272,9 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
       for (int x = tid; x < ne; x += B) cw[x] = 0u;
     }
     item_unmap(M);
-    if (tid == 0 && dup_list && dup_column(s_arr[g], u)) {
+    if (tid == 0 && dup.cols && dup_column(s_arr[g], u)) {
       u_out[g] = u;
-      dup_list[atomicAdd(&ctr_w->n_dup, 1)] = g;
+      dup_append(dup, g, ctr_w);
     } else if (tid == 0) {
       u_out[g] = u;
       const int wi = atomicAdd(&ctr_w->n_windows, 1);
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
                                                      const Counters* __restrict__ ctr, int32_t* __restrict__ u_out,
                                                      Window* __restrict__ win, int32_t* __restrict__ search_list,
                                                      int64_t win_cap, int win_target, int slab_log2,
-                                                     int32_t* __restrict__ dup_list, Counters* ctr_w) {
+                                                     DupList dup, Counters* ctr_w) {
   using Map = ItemMap<BLOCK>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ int red[BLOCK / 32 + 1];
@@ -480,8 +480,8 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
       // than k binary searches per window.  Unordered inputs always do so.
       const bool searched = !whole && in.sorted &&
                             (nslabs > 1 || P > FILTER_WINDOWS || (int64_t)s_arr[g] > (int64_t)FILTER_SEG * k);
-      if (whole && dup_list && dup_column(s_arr[g], slab_u)) {
-        if (threadIdx.x == 0) dup_list[atomicAdd(&ctr_w->n_dup, 1)] = g;
+      if (whole && dup.cols && dup_column(s_arr[g], slab_u)) {
+        if (threadIdx.x == 0) dup_append(dup, g, ctr_w);
       } else if (P > MAX_SLAB_WINDOWS) {  // win_target is validated on the host; guard anyway
         if (threadIdx.x == 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
       } else if (P > 0) {
@@ -772,7 +772,7 @@ static int pow2_at_least(int x) {
 }
 
 cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
-                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, int32_t* dup_list,
+                           Window* win, int64_t win_cap, Counters* ctr_w, int cta_max, const DupList& dup,
                            const DeviceInfo& dev, cudaStream_t st) {
   if (in.mmax <= (1 << SLAB_BITS)) {
     const bool wide = in.mmax > (1 << SYM_FLAT_LOG2);
@@ -780,7 +780,7 @@ cudaError_t launch_sym_cta(const Inputs& in, const int32_t* list, const int32_t*
     auto go = [&](auto kern, int block, size_t smem) {
       const int bps = resident_blocks((const void*)kern, block, smem);
       if (bps < 1) return cudaErrorInvalidConfiguration;
-      kern<<<dev.sms * bps, block, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup_list, ctr_w);
+      kern<<<dev.sms * bps, block, smem, st>>>(in, list, ctr, u, win, win_cap, words, s, dup, ctr_w);
       return cudaGetLastError();
     };
     if (wide) return go(k_sym_items<true, 256>, 256, sizeof(ItemMap<256>) + (1024 + CTA_MAX_LIMIT) * 4 + 1024 * 2);
@@ -809,7 +809,7 @@ constexpr int HEAVY_CAP = 4096;  // non-empty 32-row words per sub-range of the 
 // symbolic 7.2 ms as a bitmap, about 13 ms compact).
 cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_t* s, const Counters* ctr, int32_t* u,
                              Window* win, int32_t* search_list, int64_t win_cap, Counters* ctr_w, int window_max,
-                             int accumulator, int32_t* dup_list, const DeviceInfo& dev, cudaStream_t st) {
+                             int accumulator, const DupList& dup, const DeviceInfo& dev, cudaStream_t st) {
   int slab_log2 = 10;
   while (slab_log2 < SLAB_BITS && ((int64_t)1 << slab_log2) < (int64_t)in.mmax) ++slab_log2;
   const size_t w64 = (size_t)1 << (slab_log2 - 6);
@@ -836,7 +836,7 @@ cudaError_t launch_sym_heavy(const Inputs& in, const int32_t* list, const int32_
   if (bf < 1) return cudaErrorInvalidConfiguration;
   // Windows end on 64-row words: a window holds at most win_target + 63 rows.
   kern<<<dev.sms * bf, block, smem, st>>>(in, list, s, ctr, u, win, search_list, win_cap, window_max - 64, slab_log2,
-                                          dup_list, ctr_w);
+                                          dup, ctr_w);
   return cudaGetLastError();
 }
 

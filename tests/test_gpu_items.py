@@ -106,3 +106,18 @@ def test_empty_last_window(n, parts, dtype):
     B_cp, B_ri, B_va = spk.spkadd([(cp, ri, va), (cp, ri, va)], m)
     assert torch.equal(B_cp, cp.to(torch.int64)) and torch.equal(B_ri, ri)
     assert torch.equal(B_va, 2 * va)
+
+
+@pytest.mark.parametrize("n", [100, 8300])
+def test_columns_on_few_rows_beyond_the_stated_nnz(n):
+    """Column pointers that end past the stated nnz (the arrays behind are long enough here): more columns on few rows
+    than their list, sized by nnz, holds.  The call is refused and the next one is right."""
+    k, L, m = 40, 16, 64
+    rows = torch.arange(L, dtype=torch.int32, device="cuda").repeat(n)
+    cp = torch.arange(n + 1, dtype=torch.int32, device="cuda") * L
+    va = torch.ones(L * n, dtype=torch.float64, device="cuda")
+    with pytest.raises(spk.SpkaddError) as e:
+        spk.spkadd([(cp, rows[:L * 10], va[:L * 10])] * k, m)
+    assert e.value.name == "SPKADD_ERR_INTERNAL"
+    B_cp, B_ri, B_va = spk.spkadd([(cp, rows, va)] * k, m)
+    assert torch.equal(B_cp, cp.to(torch.int64)) and torch.equal(B_ri, rows) and bool((B_va == k).all())
