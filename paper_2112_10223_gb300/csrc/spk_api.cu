@@ -1,6 +1,7 @@
 // spk_api.cu -- the C ABI (include/spkadd.h): argument checks, workspace,
 // phase ordering and kernel launches.  No compute happens on the host.
 #include <climits>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -148,6 +149,7 @@ struct spkadd_handle {
   long long* d_scan = nullptr;
   char* d_op = nullptr;                // one-pass: ticket counter and look-back words
   bool onepass = false;                // B last computed by the one-pass kernel
+  bool sym_used = false;               // the symbolic phase's counters and scan words are not as the plan left them
   int32_t* d_offs = nullptr;
   Counters h_ctr{};
   int64_t nnz_out = -1;
@@ -447,7 +449,13 @@ SPK_API spkadd_status spkadd_batch_plan(spkadd_handle** hp, int count, const int
 static spkadd_status run_symbolic(spkadd_handle* h) {
   cudaError_t ce = cudaSuccess;
   int warp_launches = 0;
-  if (h->ncols > 0) {
+  if (h->sym_used) {  // the phase failed before: it starts over
+    ce = cudaMemsetAsync(&h->d_ctr->n_windows, 0, offsetof(Counters, kind_n) - offsetof(Counters, n_windows), h->st);
+    if (ce == cudaSuccess)
+      ce = cudaMemsetAsync(h->d_scan, 0, (spk::scan_tiles(h->ncols) + 1) * sizeof(long long), h->st);
+  }
+  h->sym_used = true;
+  if (ce == cudaSuccess && h->ncols > 0) {
     ce = spk::launch_sym_heavy(h->in, h->d_hl, h->d_s, h->d_ctr, h->d_u, h->d_win, h->d_search, h->win_cap, h->d_ctr,
                                h->opt.window_max, h->opt.block_accumulator, h->dup, h->dev, h->st);
     if (ce == cudaSuccess)

@@ -34,21 +34,24 @@ struct Window {
 };
 
 struct Counters {
+  // The plan's.
+  int32_t err;
   int32_t n_warp, n_cta, n_heavy;  // (n_warp: columns of at most WARP_SMALL entries)
+  int32_t n_big;        // heavy columns with s_j > BIG_S (listed apart, not counted in n_heavy)
+  int32_t n_wbig;       // warp columns above WARP_SMALL entries, listed from the list's end
+  int32_t max_warp_s;   // largest s_j of a warp column
+  // The symbolic phase's, from n_windows to n_dup: zero when it starts.
   int32_t n_windows;    // Window records of CTA-class columns, from the record array's start
+  int32_t n_hwin;       // Window records of heavy columns, from the record array's end
   int32_t n_search;     // of those, split windows needing per-input offsets
   int32_t n_unique;     // warp columns whose input rows are all distinct (u_j == s_j)
-  int32_t err;
-  int32_t n_big;        // heavy columns with s_j > BIG_S (listed apart, counted in n_heavy too)
   int32_t heavy_next;   // work counter of the heavy-column symbolic kernels
-  int32_t n_hwin;       // Window records of heavy columns, from the record array's end
+  int32_t n_bucket;     // split warp columns whose values k_warp_col sums
+  int32_t n_dup;        // thread-block columns given to k_num_dup
+  // Set to zero by the launches that use them.
   int32_t kind_n[8];    // batches of several problem kinds: thread-block items per kind (CTA-class, then heavy)
   int32_t kind_fill[8]; //   and their placement counters
-  int32_t n_wbig;       // warp columns above WARP_SMALL entries, listed from the list's end
-  int32_t n_bucket;     // split warp columns whose values k_warp_col sums
-  int32_t max_warp_s;   // largest s_j of a warp column
-  int32_t n_dup;        // thread-block columns given to k_num_dup
-  int32_t dup_next[4];  // its work counters, one per problem kind
+  int32_t dup_next[4];  // k_num_dup's work counters, one per problem kind
 };
 
 // Columns above the warp class with at most DUP_MAX_U distinct rows and at

@@ -121,3 +121,43 @@ def test_columns_on_few_rows_beyond_the_stated_nnz(n):
     assert e.value.name == "SPKADD_ERR_INTERNAL"
     B_cp, B_ri, B_va = spk.spkadd([(cp, rows, va)] * k, m)
     assert torch.equal(B_cp, cp.to(torch.int64)) and torch.equal(B_ri, rows) and bool((B_va == k).all())
+
+
+def test_symbolic_again_after_it_failed():
+    """A symbolic phase that found no memory for the windows' offsets starts over when it is called again."""
+    lengths = [600] * 3000 + [30000, 200, 5000]
+    A = _columns(20, 1 << 16, lengths, 11, torch.float64, [100] * 3000 + [1 << 16, 300, 700])
+    Ad = [tuple(t.cuda() for t in a) for a in A]
+    live, full = {}, []
+
+    @spk.ALLOC_FN
+    def alloc(nbytes, stream, ctx):
+        if live and not full:  # the workspace is the first; the second is refused once
+            full.append(nbytes)
+            return None
+        t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        live[t.data_ptr()] = t
+        return t.data_ptr()
+
+    @spk.FREE_FN
+    def free(ptr, stream, ctx):
+        live.pop(ptr, None)
+
+    o = spk.default_options()
+    o.alloc, o.free = alloc, free
+    want = [t.cpu() for t in spk.spkadd(Ad, 1 << 16)]
+    fresh = spk.spkadd(Ad, 1 << 16, info=True)[3]
+    h = spk.spkadd_plan(Ad, 1 << 16, options=o)
+    with pytest.raises(spk.SpkaddError) as e:
+        spk.spkadd_symbolic(h)
+    assert e.value.status == 6 and len(full) == 1
+    nnz = spk.spkadd_symbolic(h)
+    B = [torch.empty(len(lengths) + 1, dtype=torch.int64, device="cuda"), torch.empty(nnz, dtype=torch.int32, device="cuda"),
+         torch.empty(nnz, dtype=torch.float64, device="cuda")]
+    spk.spkadd_numeric(h, *B)
+    info = spk.spkadd_get_info(h)
+    spk.spkadd_destroy(h)
+    assert info["status"] == "SPKADD_OK"
+    for key in ("windows", "windows_split", "cols_unique"):
+        assert info[key] == fresh[key], key
+    assert all(torch.equal(x.cpu(), y) for x, y in zip(B, want))
