@@ -223,7 +223,9 @@ spkadd_status spkadd_symbolic(spkadd_handle* h, int64_t* nnz_B);
  *   B_row_idx[nnz_B] int32, sorted ascending inside every column
  *   B_val[nnz_B]     float or double per the plan's dtype
  * Enqueued on the plan's stream; returns without blocking.  May be called
- * again (with the same or other output buffers) to recompute B.
+ * again (with the same or other output buffers) to recompute B.  After
+ * spkadd_onepass it first runs the symbolic phase, if that has not run on the
+ * handle, and blocks as spkadd_symbolic does.
  */
 spkadd_status spkadd_numeric(spkadd_handle* h, int64_t* B_col_ptr, int32_t* B_row_idx, void* B_val);
 

@@ -150,6 +150,7 @@ struct spkadd_handle {
   char* d_op = nullptr;                // one-pass: ticket counter and look-back words
   bool onepass = false;                // B last computed by the one-pass kernel
   bool sym_used = false;               // the symbolic phase's counters and scan words are not as the plan left them
+  bool sym_done = false;               // its results are in the workspace
   int32_t* d_offs = nullptr;
   Counters h_ctr{};
   int64_t nnz_out = -1;
@@ -449,7 +450,7 @@ SPK_API spkadd_status spkadd_batch_plan(spkadd_handle** hp, int count, const int
 static spkadd_status run_symbolic(spkadd_handle* h) {
   cudaError_t ce = cudaSuccess;
   int warp_launches = 0;
-  if (h->sym_used) {  // the phase failed before: it starts over
+  if (h->sym_used) {  // the phase failed before, or one pass counted: it starts over
     ce = cudaMemsetAsync(&h->d_ctr->n_windows, 0, offsetof(Counters, kind_n) - offsetof(Counters, n_windows), h->st);
     if (ce == cudaSuccess)
       ce = cudaMemsetAsync(h->d_scan, 0, (spk::scan_tiles(h->ncols) + 1) * sizeof(long long), h->st);
@@ -510,6 +511,7 @@ static spkadd_status run_symbolic(spkadd_handle* h) {
     if (ce != cudaSuccess) return from_cuda(ce);
     h->launches += 2;
   }
+  h->sym_done = true;
   h->state = ST_SYMBOLIC;
   return SPKADD_OK;
 }
@@ -565,6 +567,10 @@ SPK_API spkadd_status spkadd_numeric(spkadd_handle* h, int64_t* B_col_ptr, int32
   if (!h || !B_col_ptr || h->batch) return SPKADD_ERR_INVALID_ARG;
   if (h->state < ST_SYMBOLIC) return SPKADD_ERR_STATE;
   if (h->nnz_out > 0 && (!B_row_idx || !B_val)) return SPKADD_ERR_INVALID_ARG;
+  if (!h->sym_done) {  // B so far came from the one-pass kernel, which leaves no column pointers or counts behind
+    const spkadd_status ss = run_symbolic(h);
+    if (ss != SPKADD_OK) return ss;
+  }
   cudaError_t ce = cudaMemcpyAsync(B_col_ptr, h->d_colptr, (size_t)(h->ncols + 1) * sizeof(int64_t),
                                    cudaMemcpyDeviceToDevice, h->st);
   if (ce != cudaSuccess) return from_cuda(ce);
@@ -608,6 +614,7 @@ SPK_API spkadd_status spkadd_onepass(spkadd_handle* h, int64_t* B_col_ptr, int32
     return SPKADD_OK;
   }
   h->h_ctr = c;
+  h->sym_used = true;
   int grid = 0;
   ce = cudaMemsetAsync(&h->d_ctr->n_unique, 0, sizeof(int32_t), h->st);
   if (ce != cudaSuccess) return from_cuda(ce);

@@ -213,3 +213,24 @@ def test_repeat_calls_same_handle():
     two = spk.spkadd(A, 1 << 16, method="twopass")
     assert torch.equal(outs[0][0], two[0]) and torch.equal(outs[0][1], two[1])
     assert torch.allclose(outs[0][2], two[2], rtol=0, atol=1e-5 * 16)
+
+
+def test_numeric_after_one_pass():
+    """The one-pass kernel leaves no column pointers in the workspace: spkadd_numeric on the same handle counts first."""
+    A = synth.to_device(synth.er(16, 1 << 14, 5000, 16, seed=8, dtype=F64, value_kind="int8"), torch.device(DEV))
+    cap = sum(a[1].numel() for a in A)
+    want = spk.spkadd(A, 1 << 14, method="twopass")
+    h = spk.spkadd_plan(A, 1 << 14)
+    out = [torch.empty(5001, dtype=torch.int64, device=DEV), torch.empty(cap, dtype=torch.int32, device=DEV),
+           torch.empty(cap, dtype=F64, device=DEV)]
+    for method in (spk.spkadd_onepass, spk.spkadd_numeric, spk.spkadd_onepass, spk.spkadd_numeric, spk.spkadd_numeric):
+        out[0].fill_(-1)
+        out[1].fill_(-1)
+        out[2].fill_(-1)
+        method(h, *out)
+        info = spk.spkadd_get_info(h)
+        assert info["status"] == "SPKADD_OK" and info["nnz_out"] == want[1].numel()
+        assert info["onepass"] == (method is spk.spkadd_onepass)
+        assert info["cols_unique"] == int((want[0].diff() == 256).sum())
+        assert all(torch.equal(x[:y.numel()], y) for x, y in zip(out, want))
+    spk.spkadd_destroy(h)
