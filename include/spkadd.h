@@ -14,8 +14,10 @@
  * entry can collect more than 167 terms (the float error bound
  * (t - 1) 2^-24 sum|terms| then holds), in float phases of 128 inputs whose
  * partial sums are added in float for k up to 4992, in double beyond;
- * runs of repeated rows in the one-warp columns are summed in double or in
- * pairs of floats (some 46 bits), and rounded once.
+ * runs of repeated rows in the one-warp columns (at most 512 terms) are summed
+ * in double, or in unevaluated sums of three floats that lose no more than a
+ * sum in double may (n^3 2^-72 against n 2^-53 of sum|terms| for n terms), and
+ * rounded once.
  *
  * The computation runs in phases, as the paper's k-way algorithms do:
  *   spkadd_plan      -- per-column input counts and load-balancing classes

@@ -91,7 +91,7 @@ __device__ __forceinline__ void dup_append(const DupList& d, int g, Counters* ct
 // ceil(k / 128) phase sums, and its error stays below
 // (127 + ceil(k / 128) - 1) 2^-24 sum|terms| <= 166 * 2^-24 sum|terms|.
 // Beyond FP32_PHASED_MAX_K the accumulators are double.  Warp columns
-// always sum a row's run in double.
+// sum a row's run in double or in three floats, with no larger error.
 constexpr int FP32_ACC_TERMS = 167;
 constexpr int FP32_PHASE_INPUTS = 128;  // whole 32-input chunks, one per warp group of a 256-thread block
 constexpr int FP32_PHASED_MAX_K = 4992;

@@ -329,25 +329,39 @@ __device__ __forceinline__ int wsort_column(const WsortSmem& sm, int k, int s, u
   return u;
 }
 
+// a + b = s + error, exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float* error) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  *error = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
+
 // Sum of the run term(a), ..., term(b - 1), rounded once.  Doubles are added in
-// double.  Floats are added as an unevaluated pair of floats (Knuth's two-sum:
-// the rounding error of every addition is kept and added up), some 46 bits,
-// because a double addition occupies this GPU's double units for 16 clocks a
-// warp and a conversion as many; sums that are not finite that way (an overflow
-// on the way, an infinity, a NaN) are added again in double.  Against 64-bit
-// sums the results are the same as double accumulation's.
+// double.  Floats are added as an unevaluated sum of three floats, because a
+// double addition occupies this GPU's double units for 16 clocks a warp and a
+// conversion as many: two-sum keeps the rounding error of every addition, a
+// second one those of adding the errors up (Ogita, Rump and Oishi, "Accurate sum
+// and dot product", 2005, their K = 3).  With u = 2^-24, what is left out is at
+// most n^3 u^3 sum|terms| for n terms, below the n 2^-53 sum|terms| of a sum in
+// double for n <= 724 (columns here have at most 512 entries), and nothing
+// where a sum in double is exact because the partial sums fit into 53 bits.
+// Sums that are not finite that way (an overflow on the way, an infinity, a NaN)
+// are added again in double.
 template <typename V, typename TermF>
 __device__ __forceinline__ V wsort_run_sum(int a, int b, TermF&& term) {
+  static_assert(WSORT_MAX <= 724, "the error bound above");
   if constexpr (sizeof(V) == 4) {
-    float hi = term(a), lo = 0.0f;
-    for (int y = a + 1; y < b; ++y) {
-      const float x = term(y);
-      const float s = __fadd_rn(hi, x);
-      const float t = __fsub_rn(s, hi);
-      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
-      hi = s;
+    float hi = term(a), mid = 0.0f, lo = 0.0f;
+    if (b - a > 1) hi = two_sum(hi, term(a + 1), &mid);
+    for (int y = a + 2; y < b; ++y) {
+      float e;
+      hi = two_sum(hi, term(y), &e);
+      mid = two_sum(mid, e, &e);
+      lo = __fadd_rn(lo, e);
     }
-    if (isfinite(hi) && isfinite(lo)) return b - a > 1 ? __fadd_rn(hi, lo) : hi;
+    float r = hi;  // (without errors as it is: minus zero stays)
+    if (mid != 0.0f || lo != 0.0f) r = lo != 0.0f ? (float)((double)hi + (double)mid + (double)lo) : __fadd_rn(hi, mid);
+    if (isfinite(r)) return r;
   }
   double sum = (double)term(a);
   for (int y = a + 1; y < b; ++y) sum += (double)term(y);

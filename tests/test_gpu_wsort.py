@@ -2,6 +2,9 @@
 
 Small-integer values: indices and sums must match the oracle exactly in either type.
 """
+import math
+
+import numpy as np
 import pytest
 import torch
 
@@ -100,3 +103,33 @@ def test_float_runs_round_once_and_keep_infinities():
         assert torch.equal(torch.isnan(got), torch.isnan(want))
         ok = ~torch.isnan(want)
         assert torch.equal(got[ok], want[ok])
+
+
+@pytest.mark.parametrize("n", [2, 3, 9, 64, 256, 512])
+def test_float_runs_are_as_exact_as_double_sums(n):
+    """Long runs that cancel: what a sum of n floats may lose is n^3 u^3 sum|terms| (u = 2^-24), at most 2^-45 of it,
+    besides its rounding to float; in all no more than a sum in double loses.  A run of minus zeros is minus zero."""
+    rng, cols = np.random.default_rng(n), 240
+    v = np.zeros((cols, n), dtype=np.float32)
+    for c in range(cols):
+        half = (rng.standard_normal(n // 2) * 2.0 ** rng.integers(-13, 13, n // 2)).astype(np.float32)
+        x = np.concatenate([half, -half, rng.standard_normal(n % 2).astype(np.float32)])
+        at = rng.integers(0, n, max(1, n // 8))
+        x[at] += (rng.standard_normal(at.size) * (0.0, 1e-10, 1e-6, 1e-3, 1.0)[c % 5]).astype(np.float32)
+        v[c] = x[rng.permutation(n)]
+    v[7::40] = -0.0
+    cp = torch.arange(cols + 1, dtype=torch.int32)
+    A = [(cp, torch.zeros(cols, dtype=torch.int32), torch.from_numpy(v[:, i].copy())) for i in range(n)]
+    exact = np.array([math.fsum(row) for row in v.astype(np.float64)])
+    size = np.abs(v.astype(np.float64)).sum(1)
+    acc = np.zeros(cols)
+    for i in range(n):
+        acc += v[:, i]
+    by_double = np.abs(acc.astype(np.float32).astype(np.float64) - exact)
+    for method in ("twopass", "onepass"):
+        got = run_gpu(A, 5, method=method)[2].cpu().numpy()
+        err = np.abs(got.astype(np.float64) - exact)
+        bound = 0.5 * np.spacing(np.abs(exact).astype(np.float32)).astype(np.float64) + n ** 3 * 2.0 ** -72 * size
+        assert (err <= bound).all(), (method, (err - bound).max())
+        assert err.sum() <= by_double.sum()
+        assert np.signbit(got[7::40]).all()
