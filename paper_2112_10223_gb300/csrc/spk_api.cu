@@ -467,8 +467,8 @@ static spkadd_status run_symbolic(spkadd_handle* h) {
                                 &warp_launches);
     h->launches += 2 + warp_launches;
   }
-  if (ce == cudaSuccess) ce = spk::launch_scan_fused(h->in, h->d_u, h->d_scan, h->d_colptr, h->dup, h->d_win, h->win_cap,
-                                                     h->d_ctr, h->st);
+  if (ce == cudaSuccess) ce = spk::launch_scan_fused(h->in, h->d_s, h->d_u, h->d_scan, h->d_colptr, h->dup, h->d_win,
+                                                     h->win_cap, h->d_ctr, h->st);
   h->launches += 1;
   // Several problem kinds: the thread-block items grouped by kind for the numeric launches.
   if (ce == cudaSuccess && h->ncols > 0 && h->d_wsort) {
@@ -551,8 +551,8 @@ static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
                              h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
   h->launches += item_launches;
   if (ce == cudaSuccess && h->h_ctr.n_dup > 0) {
-    ce = spk::launch_num_dup(h->in, spk::num_cta_kinds(h->dt_mode, h->f32_kinds), h->dup.cols, h->h_ctr.n_dup, h->d_s,
-                             h->d_u, h->d_colptr, out, h->d_ctr, h->dev, h->st, &item_launches);
+    ce = spk::launch_num_dup(h->in, h->dup.cols, h->h_ctr.n_dup, h->h_ctr.dup_n, h->d_u, h->d_colptr, out, h->d_ctr, h->dev,
+                             h->st, &item_launches);
     h->launches += item_launches;
   }
   if (ce == cudaSuccess && h->h_ctr.n_warp + h->h_ctr.n_wbig > 0)

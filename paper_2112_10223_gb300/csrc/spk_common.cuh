@@ -48,36 +48,14 @@ struct Counters {
   int32_t heavy_next;   // work counter of the heavy-column symbolic kernels
   int32_t n_bucket;     // split warp columns whose values k_warp_col sums
   int32_t n_dup;        // thread-block columns given to k_num_dup
+  int32_t dup_n[4];     //   how many of each problem kind,
+  int32_t dup_max[4];   //   the largest s_j of a kind's,
+  int64_t dup_sum[4];   //   and the sum of theirs
   // Set to zero by the launches that use them.
   int32_t kind_n[8];    // batches of several problem kinds: thread-block items per kind (CTA-class, then heavy)
   int32_t kind_fill[8]; //   and their placement counters
   int32_t dup_next[4];  // k_num_dup's work counters, one per problem kind
 };
-
-// Columns above the warp class with at most DUP_MAX_U distinct rows and at
-// least DUP_RATIO entries a row are summed by one warp each (k_num_dup).
-constexpr int DUP_MAX_U = 256;
-constexpr int DUP_RATIO = 4;
-constexpr int DUP_ROW_BITS = 23;  // rows below 2^23: a row and its table slot share a 32-bit key
-// Fewer of them than this leave warps idle (a column of 4096 entries takes one
-// warp about 90 us): they go to the thread-block items instead (a batch with
-// 3728 of them: 117 us here, 64 us there).
-constexpr int DUP_MIN_COLS = 8192;
-__host__ __device__ constexpr bool dup_column(int64_t s, int u) { return u <= DUP_MAX_U && s >= (int64_t)DUP_RATIO * u; }
-
-// The columns given to k_num_dup, Counters::n_dup of them.
-struct DupList {
-  int32_t* cols;  // null: none are set apart
-  int32_t cap;    // entries cols holds
-};
-
-// Lists column g (one thread).  The list is sized by the inputs' nnz: column
-// pointers that disagree with it leave an error, never a write past the list.
-__device__ __forceinline__ void dup_append(const DupList& d, int g, Counters* ctr_w) {
-  const int at = atomicAdd(&ctr_w->n_dup, 1);
-  if (at < d.cap) d.cols[at] = g;
-  else atomicOr(&ctr_w->err, ERR_WINDOW_CAP);
-}
 
 // Float sums.  A float sum of t terms, in any order, errs by at most
 // (t - 1) 2^-24 sum|terms| (first order), within 1e-5 sum|terms| for
@@ -135,6 +113,75 @@ struct Inputs {
 };
 
 __device__ __forceinline__ int inst_of(const Inputs& in, int g) { return in.col_inst ? __ldg(in.col_inst + g) : 0; }
+
+// Problem kinds of the thread-block numeric launches, one launch per kind
+// present: 0 float with k <= FP32_ACC_TERMS, 1 float with
+// FP32_ACC_TERMS < k <= FP32_PHASED_MAX_K (sums in phases), 2 float with
+// larger k (double accumulators), 3 double.
+__device__ __forceinline__ int item_kind(const Inst* I) {
+  if (I->dtype == 1) return 3;
+  return I->k <= FP32_ACC_TERMS ? 0 : (I->k <= FP32_PHASED_MAX_K ? 1 : 2);
+}
+
+// Columns above the warp class with at most DUP_MAX_U distinct rows and at
+// least DUP_RATIO entries a row are summed by one warp each (k_num_dup).
+constexpr int DUP_MAX_U = 256;
+constexpr int DUP_RATIO = 4;
+constexpr int DUP_ROW_BITS = 23;  // rows below 2^23: a row and its table slot share a 32-bit key
+// Fewer of them of one problem kind leave warps idle (a column of 4096 entries
+// takes one warp some 90 us): they go to the thread-block items instead.  Both
+// ways cross at 3500 (600 entries each), 6000 (4096) and 8000 (9000) float
+// columns and at 2500 to 4000 double ones; 16000 of 600, 4096 and 9000 entries:
+// 87 against 175, 251 against 371 and 836 against 978 us float, 105 against 203,
+// 318 against 615 and 720 against 1137 us double.
+constexpr int DUP_MIN_COLS = 8192;
+// And a column of more than one DUP_SHARE'th of its kind's entries, twice what a
+// warp gets on average, would still run when the others are done: it goes to the
+// thread-block items too.  16384 float columns of 1200 entries take 210 us; with
+// one more of 9600 entries 227 us here and 250 us with that column in the items,
+// of 19200 330 and 266 us, of 75000 936 and 371 us (all columns in the items:
+// 398, 398 and 498 us); double columns the same way.
+constexpr int DUP_SHARE = 2048;
+__host__ __device__ constexpr bool dup_column(int64_t s, int u) { return u <= DUP_MAX_U && s >= (int64_t)DUP_RATIO * u; }
+
+// The columns given to k_num_dup, Counters::n_dup of them.
+struct DupList {
+  int32_t* cols;  // null: none are set apart
+  int32_t cap;    // entries cols holds
+};
+
+// What one block has listed, in shared memory (Counters::dup_n, dup_max, dup_sum).
+struct DupTally {
+  int32_t n[4], max[4];
+  uint32_t sum[4];  // in units of 16 entries
+  __device__ __forceinline__ void clear() {
+    for (int q = 0; q < 4; ++q) {
+      n[q] = max[q] = 0;
+      sum[q] = 0u;
+    }
+  }
+  __device__ __forceinline__ void flush(Counters* ctr_w) const {
+    for (int q = 0; q < 4; ++q)
+      if (n[q] > 0) {
+        atomicAdd(&ctr_w->dup_n[q], n[q]);
+        atomicMax(&ctr_w->dup_max[q], max[q]);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&ctr_w->dup_sum[q]), (unsigned long long)sum[q] << 4);
+      }
+  }
+};
+
+// Lists column g of s entries.  The list is sized by the inputs' nnz: column
+// pointers that disagree with it leave an error, never a write past the list.
+// (The tally's atomics return nothing, so the one thread that lists a column
+// does not wait for them.)
+__device__ __forceinline__ void dup_append(const DupList& d, DupTally& tally, int g, int s, int kind, Counters* ctr_w) {
+  const int at = atomicAdd(&ctr_w->n_dup, 1);
+  if (at < d.cap) d.cols[at] = g;
+  else atomicOr(&ctr_w->err, ERR_WINDOW_CAP);
+  atomicAdd(&tally.n[kind], 1);
+  atomicAdd(&tally.sum[kind], (uint32_t)s >> 4);
+  atomicMax(&tally.max[kind], s);
+}
 
 // Where B goes: the caller's buffers, through per-problem pointer tables
 // (rows/vals/cps, a batch) or directly (row0/val0/cp0: a single problem, and

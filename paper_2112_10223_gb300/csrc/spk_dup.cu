@@ -9,9 +9,14 @@
 // compare-and-swap loops, which for doubles run at 0.9 lanes a clock per SM.
 // Here almost every entry finds its row at the first load, nothing but the
 // column's rows is touched, and since one input's rows are distinct, the lanes
-// of one input add with plain loads and stores, input after input, so a row's
-// terms are also summed in input order.  The distinct rows, listed as they are
-// inserted, are at the end sorted in registers (spk_wsort.cuh).
+// of one input add with plain loads and stores, input after input.  Where 32
+// entries come from more than DUP_ROUNDS inputs, that many turns take longer than
+// atomics: 16384 float columns of 1024 entries on 128 rows, one to an input,
+// 1178 us in turns, 439 us so (1363 us as block items), two to an input 636, 248
+// and 433, four 345, 187 and 277; double 1169, 477 and 826, 611, 279 and 334, 320,
+// 197 and 283.  At eight to an input (four inputs) both take the same time.  The
+// distinct rows, listed as they are inserted, are at the end sorted in registers
+// (spk_wsort.cuh).
 //
 // What bounds it: issue slots (65% busy at 32 warps per SM, 125 warp
 // instructions per 32 entries) and half of the shared-memory wavefronts.
@@ -31,6 +36,7 @@ constexpr int DUP_SLOT_BITS = 9;
 constexpr int DUP_SLOTS = 1 << DUP_SLOT_BITS;
 constexpr int DUP_BUCKETS = DUP_SLOTS / 2;
 constexpr int DUP_MAP = 2048;                    // positions of a start-bit map
+constexpr int DUP_ROUNDS = 4;                    // at most this many inputs' lanes add in turn
 constexpr uint32_t DUP_EMPTY = 0xffffffffu;
 static_assert(DUP_MAX_U * 2 <= DUP_SLOTS, "at most half of the slots are taken");
 static_assert(DUP_ROW_BITS + DUP_SLOT_BITS <= 32, "a row and its slot share a key");
@@ -47,7 +53,6 @@ struct DupSmem {
 
 struct DupArgs {
   const int32_t* list;     // global column ids
-  const int32_t* s_arr;
   const int32_t* u_arr;
   const int64_t* col_ptr;
   Outs out;
@@ -76,7 +81,8 @@ __device__ __noinline__ int dup_insert(DupSmem<A>& D, uint32_t row, uint32_t h) 
   return -1;  // more distinct rows than the symbolic pass counted
 }
 
-template <int DT, bool WIDE_ACC, int WARPS>
+// SORTED: rows strictly increasing inside every input column.
+template <int DT, bool WIDE_ACC, bool SORTED, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, (DT == 1 || WIDE_ACC ? 24 : 32) / WARPS)
     k_num_dup(Inputs in, DupArgs a) {
   using V = typename std::conditional<DT == 1, double, float>::type;
@@ -104,8 +110,7 @@ __global__ void __launch_bounds__(WARPS * 32, (DT == 1 || WIDE_ACC ? 24 : 32) / 
     const int q = inst_of(in, g);
     const Inst* I = in.inst + q;
     const int k = I->k, off = I->ptr_off, j = g - I->colbase;
-    const int kind = I->dtype == 1 ? 3 : I->k <= FP32_ACC_TERMS ? 0 : I->k <= FP32_PHASED_MAX_K ? 1 : 2;
-    if (a.kind >= 0 && kind != a.kind) {
+    if (a.kind >= 0 && item_kind(I) != a.kind) {
       c = __shfl_sync(SPK_FULL, coming, 0);
       continue;
     }
@@ -226,11 +231,12 @@ __global__ void __launch_bounds__(WARPS * 32, (DT == 1 || WIDE_ACC ? 24 : 32) / 
               }
             }
             const bool add = live && slot >= 0;
-            if (in.sorted) {
+            const int o0 = SORTED ? __shfl_sync(SPK_FULL, o[t], 0) : 0;
+            const int o1 = SORTED ? __shfl_sync(SPK_FULL, o[t], 31) : DUP_ROUNDS;
+            if (o1 - o0 < DUP_ROUNDS) {
               // One input's rows are distinct: its lanes add together.
-              const int o1 = __shfl_sync(SPK_FULL, o[t], 31);
 #pragma unroll 1
-              for (int x = __shfl_sync(SPK_FULL, o[t], 0); x <= o1; ++x) {
+              for (int x = o0; x <= o1; ++x) {
                 if (add && o[t] == x) D.acc[slot] += (A)v[t];
                 __syncwarp();
               }
@@ -295,20 +301,20 @@ __global__ void __launch_bounds__(WARPS * 32, (DT == 1 || WIDE_ACC ? 24 : 32) / 
 }
 
 template <int DT, bool WIDE_ACC>
-static cudaError_t launch_dup(const Inputs& in, const DupArgs& a, const DeviceInfo& dev, cudaStream_t st) {
+static cudaError_t launch_dup(const Inputs& in, const DupArgs& a, int n, const DeviceInfo& dev, cudaStream_t st) {
   constexpr int WARPS = 4;
   using A = typename std::conditional<DT == 1 || WIDE_ACC, double, float>::type;
-  auto kern = k_num_dup<DT, WIDE_ACC, WARPS>;
+  auto kern = in.sorted ? k_num_dup<DT, WIDE_ACC, true, WARPS> : k_num_dup<DT, WIDE_ACC, false, WARPS>;
   const size_t smem = WARPS * sizeof(DupSmem<A>);
   const int bps = resident_blocks((const void*)kern, WARPS * 32, smem);
   if (bps < 1) return cudaErrorInvalidConfiguration;
   int grid = dev.sms * bps;
-  if (grid > (a.n + WARPS - 1) / WARPS) grid = (a.n + WARPS - 1) / WARPS;
+  if (grid > (n + WARPS - 1) / WARPS) grid = (n + WARPS - 1) / WARPS;
   kern<<<grid, WARPS * 32, smem, st>>>(in, a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_num_dup(const Inputs& in, int kinds, const int32_t* list, int n, const int32_t* s, const int32_t* u,
+cudaError_t launch_num_dup(const Inputs& in, const int32_t* list, int n, const int32_t* n_kind, const int32_t* u,
                            const int64_t* col_ptr, const Outs& out, Counters* ctr_w, const DeviceInfo& dev,
                            cudaStream_t st, int* launches) {
   *launches = 0;
@@ -316,20 +322,18 @@ cudaError_t launch_num_dup(const Inputs& in, int kinds, const int32_t* list, int
   cudaError_t e = cudaMemsetAsync(&ctr_w->dup_next[0], 0, sizeof(ctr_w->dup_next), st);
   DupArgs a{};
   a.list = list;
-  a.s_arr = s;
   a.u_arr = u;
   a.col_ptr = col_ptr;
   a.out = out;
   a.ctr_w = ctr_w;
   a.n = n;
-  const bool alone = __builtin_popcount(kinds) == 1;
   for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
-    if (!((kinds >> q) & 1)) continue;
-    a.kind = alone ? -1 : q;
+    if (n_kind[q] <= 0) continue;
+    a.kind = n_kind[q] == n ? -1 : q;
     // Float sums of more than FP32_ACC_TERMS inputs in double.
-    e = q == 0 ? launch_dup<0, false>(in, a, dev, st)
-        : q == 3 ? launch_dup<1, false>(in, a, dev, st)
-                 : launch_dup<0, true>(in, a, dev, st);
+    e = q == 0 ? launch_dup<0, false>(in, a, n_kind[q], dev, st)
+        : q == 3 ? launch_dup<1, false>(in, a, n_kind[q], dev, st)
+                 : launch_dup<0, true>(in, a, n_kind[q], dev, st);
     ++*launches;
   }
   return e;

@@ -45,8 +45,8 @@ cudaError_t launch_validate(const Inputs& in, const int64_t* nnz, Counters* ctr,
 size_t scan_tiles(int64_t n);
 cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* col_ptr, cudaStream_t st);
 // The same scan in one launch over words that launch_bin zeroed.  Columns of the
-// dup list also become window records when they are few.
-cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
+// dup list that are not k_num_dup's after all become window records.
+cudaError_t launch_scan_fused(const Inputs& in, const int32_t* s, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
                               const DupList& dup, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st);
 // Loads the scan kernels onto the current device (module loading is lazy).
 cudaError_t load_scan_kernels();
@@ -87,8 +87,8 @@ cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window
                            int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
                            const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
                            const DeviceInfo& dev, cudaStream_t st, int* launches);
-// The n columns of the dup list; kinds as num_cta_kinds gives them.
-cudaError_t launch_num_dup(const Inputs& in, int kinds, const int32_t* list, int n, const int32_t* s, const int32_t* u,
+// The n columns of the dup list, n_kind of each problem kind (Counters::n_dup, dup_n).
+cudaError_t launch_num_dup(const Inputs& in, const int32_t* list, int n, const int32_t* n_kind, const int32_t* u,
                            const int64_t* col_ptr, const Outs& out, Counters* ctr_w, const DeviceInfo& dev,
                            cudaStream_t st, int* launches);
 // Per-problem column pointers of B (a batch): out_cp[q][j] = col_ptr[colbase + j] - col_ptr[colbase].

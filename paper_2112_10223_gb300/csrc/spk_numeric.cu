@@ -112,15 +112,6 @@ __device__ __forceinline__ bool item_selected(int sel, const Inst* I) {
   return true;
 }
 
-// Problem kinds of the thread-block numeric launches, one launch per kind
-// present: 0 float with k <= FP32_ACC_TERMS, 1 float with
-// FP32_ACC_TERMS < k <= FP32_PHASED_MAX_K (sums in phases), 2 float with
-// larger k (double accumulators), 3 double.
-__device__ __forceinline__ int item_kind(const Inst* I) {
-  if (I->dtype == 1) return 3;
-  return I->k <= FP32_ACC_TERMS ? 0 : (I->k <= FP32_PHASED_MAX_K ? 1 : 2);
-}
-
 // Pass B of an item's slab: every entry's value added at its rank.  Without
 // phases the sums stay in acc for the caller's write (returns false).
 // PHASED (float sums of problems with k > FP32_ACC_TERMS): a slab whose

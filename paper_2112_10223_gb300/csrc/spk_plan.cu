@@ -212,14 +212,88 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int32_t* __rest
   if (blockIdx.x == 0 && threadIdx.x == 0) col_ptr[n] = *grand_total;
 }
 
+// Turns the columns of the dup list that are not k_num_dup's after all (their
+// kind has too few, or they are larger than their share: DUP_MIN_COLS, DUP_SHARE)
+// into window records and closes the list's gaps.  One block of SCAN_BLOCK
+// threads; `tmp` holds 33 entries.
+__device__ __forceinline__ void dup_divide(const Inputs& in, const int32_t* __restrict__ s,
+                                           const int32_t* __restrict__ u, const DupList& dup,
+                                           Window* __restrict__ win, int64_t win_cap, Counters* __restrict__ ctr,
+                                           long long* tmp) {
+  const int nd = ctr->n_dup;
+  if (nd <= 0 || nd > dup.cap) return;  // (past cap: the error is set)
+  __shared__ int limit[4], left[4];
+  bool any = false;
+  for (int q = 0; q < 4; ++q) {
+    const int n = ctr->dup_n[q];
+    const int64_t share = ctr->dup_sum[q] / DUP_SHARE;
+    const int lim = n < DUP_MIN_COLS ? 0 : (int)(share < INT32_MAX ? share : INT32_MAX);
+    any = any || (n > 0 && ctr->dup_max[q] > lim);
+    if (threadIdx.x == 0) {
+      limit[q] = lim;
+      left[q] = 0;
+    }
+  }
+  if (!any) return;  // (block-uniform)
+  const int nw = ctr->n_windows, cap = (int)(win_cap - ctr->n_hwin);
+  __syncthreads();
+  constexpr int PER = 8;
+  int kept = 0, moved = 0;
+  for (int x0 = 0; x0 < nd; x0 += PER * SCAN_BLOCK) {
+    int g[PER], kind[PER];
+    unsigned keep = 0u, move = 0u;
+#pragma unroll
+    for (int t = 0; t < PER; ++t) {
+      const int x = x0 + t * SCAN_BLOCK + (int)threadIdx.x;
+      g[t] = x < nd ? dup.cols[x] : -1;
+    }
+#pragma unroll
+    for (int t = 0; t < PER; ++t)
+      if (g[t] >= 0) {
+        kind[t] = item_kind(in.inst + inst_of(in, g[t]));
+        (s[g[t]] <= limit[kind[t]] ? keep : move) |= 1u << t;
+      }
+    // Every read of this part of the list comes before the scan's barrier, every write after it and no further on.
+    long long total;
+    const long long ex = block_excl_scan64(__popc(keep) | ((long long)__popc(move) << 32), tmp, &total);
+    int at = kept + (int)(ex & 0xffffffff), wi = nw + moved + (int)(ex >> 32);
+#pragma unroll
+    for (int t = 0; t < PER; ++t) {
+      if ((keep >> t) & 1u) {
+        dup.cols[at++] = g[t];
+        atomicAdd(&left[kind[t]], 1);
+      } else if ((move >> t) & 1u) {
+        Window w;
+        w.col = g[t];
+        w.r_lo = 0;
+        w.r_hi = in.inst[inst_of(in, g[t])].m;
+        w.u = u[g[t]];
+        w.out_off = 0;
+        w.search = -1;
+        if (wi < cap) win[wi] = w;
+        else atomicOr(&ctr->err, ERR_WINDOW_CAP);
+        ++wi;
+      }
+    }
+    kept += (int)(total & 0xffffffff);
+    moved += (int)(total >> 32);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ctr->n_windows = nw + moved;
+    ctr->n_dup = kept;
+  }
+  if (threadIdx.x < 4) ctr->dup_n[threadIdx.x] = left[threadIdx.x];
+}
+
 // The same scan in one launch (three took 9 us of a small call's 105): tiles in
 // ticket order, each tile's offset from a decoupled look-back over the tiles
 // before it.  scan_buf: the ticket counter, then one look-back word per tile,
-// zero at launch.  The tile taken first also turns the columns of the dup list
-// into window records when there are too few of them for k_num_dup.
+// zero at launch.  The block of the tile taken first also divides the dup list.
 constexpr unsigned long long SCAN_WAIT_NS = 60000000000ull;  // bound of a look-back wait (they last microseconds)
 
-__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int32_t* __restrict__ u, int n, int tiles,
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int32_t* __restrict__ s,
+                                                          const int32_t* __restrict__ u, int n, int tiles,
                                                           unsigned long long* __restrict__ scan_buf,
                                                           int64_t* __restrict__ col_ptr,
                                                           DupList dup, Window* __restrict__ win, int64_t win_cap,
@@ -261,28 +335,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_fused(Inputs in, const int3
     if (j < n) col_ptr[j] = run;
     run += v[t];
   }
-  if (tile == 0 && dup.cols) {
-    const int nd = ctr->n_dup, nw = ctr->n_windows, cap = (int)(win_cap - ctr->n_hwin);
-    if (nd > 0 && nd < DUP_MIN_COLS && nd <= dup.cap) {  // (past cap: the error is set)
-      for (int x = threadIdx.x; x < nd; x += SCAN_BLOCK) {
-        const int g = dup.cols[x];
-        Window w;
-        w.col = g;
-        w.r_lo = 0;
-        w.r_hi = in.inst[inst_of(in, g)].m;
-        w.u = u[g];
-        w.out_off = 0;
-        w.search = -1;
-        if (nw + x < cap) win[nw + x] = w;
-        else atomicOr(&ctr->err, ERR_WINDOW_CAP);
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        ctr->n_windows = nw + nd;
-        ctr->n_dup = 0;
-      }
-    }
-  }
+  if (tile == 0 && dup.cols) dup_divide(in, s, u, dup, win, win_cap, ctr, tmp);
 }
 
 // Per-input offsets of split row windows (Sec. III-B: "partition rows ...
@@ -414,11 +467,11 @@ cudaError_t launch_scan(const int32_t* u, int n, long long* tile_buf, int64_t* c
   return cudaGetLastError();
 }
 
-cudaError_t launch_scan_fused(const Inputs& in, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
+cudaError_t launch_scan_fused(const Inputs& in, const int32_t* s, const int32_t* u, long long* scan_buf, int64_t* col_ptr,
                               const DupList& dup, Window* win, int64_t win_cap, Counters* ctr, cudaStream_t st) {
   int tiles = (int)(((int64_t)in.ncols + SCAN_TILE - 1) / SCAN_TILE);
   if (tiles < 1) tiles = 1;
-  k_scan_fused<<<tiles, SCAN_BLOCK, 0, st>>>(in, u, in.ncols, tiles, reinterpret_cast<unsigned long long*>(scan_buf),
+  k_scan_fused<<<tiles, SCAN_BLOCK, 0, st>>>(in, s, u, in.ncols, tiles, reinterpret_cast<unsigned long long*>(scan_buf),
                                             col_ptr, dup, win, win_cap, ctr);
   return cudaGetLastError();
 }

@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
   uint32_t* cw = bits + 1024;                                               //   CTA_MAX_LIMIT words, kept zero
   uint16_t* spre = reinterpret_cast<uint16_t*>(cw + CTA_MAX_LIMIT);         //   1024 prefixes
   const int tid = threadIdx.x;
+  __shared__ DupTally tally;
+  if (tid == 0) tally.clear();
   for (int x = tid; x < (WIDE ? 1024 + CTA_MAX_LIMIT : words); x += B) bits[x] = 0u;
   item_unmap(M);
   __syncthreads();
@@ -218,6 +220,7 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
       return sum;
     };
     int fresh = 0, ne = 0, u;
+    int s = 0, kind = 0;  // thread 0's, loaded while the rows are counted
     if (!WIDE) {
       rows_pass(true, [&]() {
         each_row([&](uint32_t x, bool in_m) {
@@ -230,6 +233,10 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
       if (c + (int)gridDim.x < ncols) {
         In = in.inst + inst_of(in, gn);
         Fn = bounds(gn, In, 0);
+      }
+      if (tid == 0 && dup.cols) {
+        s = s_arr[g];
+        kind = item_kind(I);
       }
       u = add_up(fresh);
       if (single) {
@@ -267,14 +274,18 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
           fresh += !(old & bit);
         });
       });
+      if (tid == 0 && dup.cols) {
+        s = s_arr[g];
+        kind = item_kind(I);
+      }
       u = add_up(fresh);  // (a barrier lies between the two uses of red[1])
       *reinterpret_cast<uint4*>(summ + 4 * tid) = make_uint4(0u, 0u, 0u, 0u);
       for (int x = tid; x < ne; x += B) cw[x] = 0u;
     }
     item_unmap(M);
-    if (tid == 0 && dup.cols && dup_column(s_arr[g], u)) {
+    if (tid == 0 && dup.cols && dup_column(s, u)) {
       u_out[g] = u;
-      dup_append(dup, g, ctr_w);
+      dup_append(dup, tally, g, s, kind, ctr_w);
     } else if (tid == 0) {
       u_out[g] = u;
       const int wi = atomicAdd(&ctr_w->n_windows, 1);
@@ -292,6 +303,7 @@ __global__ void __launch_bounds__(B, 1280 / B) k_sym_items(Inputs in, const int3
       }
     }
   }
+  if (tid == 0) tally.flush(ctr_w);
 }
 
 constexpr int HEAVY_BLOCK = 1024;
@@ -331,6 +343,8 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
   for (int x = threadIdx.x; x < W64; x += BLOCK) bm[x] = 0ull;
   for (int x = threadIdx.x; x < NSW; x += BLOCK) summ[x] = 0u;
   item_unmap(M);
+  __shared__ DupTally tally;
+  if (threadIdx.x == 0) tally.clear();
   __syncthreads();
   const int n_big = ctr->n_big;
   const int ncols = n_big + ctr->n_heavy;
@@ -481,7 +495,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
       const bool searched = !whole && in.sorted &&
                             (nslabs > 1 || P > FILTER_WINDOWS || (int64_t)s_arr[g] > (int64_t)FILTER_SEG * k);
       if (whole && dup.cols && dup_column(s_arr[g], slab_u)) {
-        if (threadIdx.x == 0) dup_append(dup, g, ctr_w);
+        if (threadIdx.x == 0) dup_append(dup, tally, g, s_arr[g], item_kind(I), ctr_w);
       } else if (P > MAX_SLAB_WINDOWS) {  // win_target is validated on the host; guard anyway
         if (threadIdx.x == 0) atomicOr(&ctr_w->err, ERR_INTERNAL);
       } else if (P > 0) {
@@ -537,6 +551,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK >= 1024 ? 1 : 4) k_sym_heavy(Inpu
     if (threadIdx.x == 0) u_out[g] = s_col_u;
     __syncthreads();
   }
+  if (threadIdx.x == 0) tally.flush(ctr_w);
 }
 
 // Heavy columns, compact form: the same count and window cuts from a summary

@@ -6,8 +6,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2112_10223_gb300 as spk
-from spk_testlib import check_full
+from spk_testlib import check_full, compare, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -161,3 +162,48 @@ def test_symbolic_again_after_it_failed():
     for key in ("windows", "windows_split", "cols_unique"):
         assert info[key] == fresh[key], key
     assert all(torch.equal(x.cpu(), y) for x, y in zip(B, want))
+
+
+def _few_rows(k, m, groups, seed, dtype):
+    """k inputs of the columns of groups [(n, P, L)]: n columns, L rows out of P in every input (on the GPU)."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    at = [torch.randint(0, m - 3 * P + 1, (n, 1), generator=g, device="cuda") for n, P, _ in groups]
+    cp = torch.zeros(sum(n for n, _, _ in groups) + 1, dtype=torch.int32, device="cuda")
+    cp[1:] = torch.cumsum(torch.cat([torch.full((n,), L, device="cuda") for n, _, L in groups]), 0)
+    out = []
+    for _ in range(k):
+        pick = [torch.rand(n, P, generator=g, device="cuda").topk(L, dim=1).indices.sort(dim=1).values for n, P, L in groups]
+        ri = torch.cat([(a + 3 * p).reshape(-1) for a, p in zip(at, pick)]).to(torch.int32)
+        out.append((cp, ri, torch.randint(-8, 9, (ri.numel(),), generator=g, device="cuda").to(dtype)))
+    return out
+
+
+def _launches(problems, **opt):
+    """Kernels launched for the problems, whose sums are checked."""
+    outs, info = spk.spkadd_batch(problems, info=True, options=spk.default_options(**opt))
+    for (A, _), B in zip(problems, outs):
+        compare(tuple(t.cpu().numpy() for t in B), oracle.add(to_np(A)), A[0][2].dtype, exact=True)
+    return info["kernel_launches"]
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("more, launches", [
+    ([], 0),               # all in the table: one launch, as when the block items (block_accumulator 1) take them all
+    ([(1, 1000, 40)], 1),  # beside them a column on many rows: the block items' launch as well
+    ([(1, 255, 55)], 0),   # 2200 entries, below the 2430 that one column may have
+    ([(1, 255, 100)], 1),  # 4000 entries: to the block items
+    ([(1, 255, 200)], 0),  # 8000 entries: to the block items, whose flat form launches once more, for the heavy class
+])
+def test_large_columns_on_few_rows_stay_out_of_the_table(more, launches, dtype):
+    """A column on few rows that has many times the entries of the others is not left to one warp."""
+    A = _few_rows(40, 4096, [(8300, 60, 15), *more], 5, dtype)
+    assert _launches([(A, 4096)]) - _launches([(A, 4096)], block_accumulator=1) == launches
+
+
+def test_few_columns_of_a_kind_stay_out_of_the_table():
+    """Columns on few rows are counted kind by kind: 8300 of one kind go to the table, 5000 of another do not."""
+    many = _few_rows(40, 4096, [(8300, 60, 15), (1, 1000, 40)], 6, torch.float64)
+    few = _few_rows(40, 4096, [(5000, 60, 15), (1, 1000, 40)], 7, torch.float32)
+    a, b = (many, 4096), (few, 4096)
+    flat = _launches([a, b], block_accumulator=1)
+    assert _launches([a, b]) == flat + 1  # k_num_items for either kind, and k_num_dup for one
