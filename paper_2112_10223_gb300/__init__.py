@@ -209,7 +209,7 @@ def _check_inputs(A, dtype, where: str, dev: int | None, append) -> int:
         if dev is None:
             dev = d
         if d != dev or ri.get_device() != dev or va.get_device() != dev:
-            raise TypeError("all inputs must be on one device")
+            raise TypeError(f"all {'problems' if where else 'inputs'} must be on one device")
         nnz = ri.numel()
         append((cp.numel() - 1, nnz, cp.data_ptr(), ri.data_ptr() if nnz else 0, va.data_ptr() if va.numel() else 0))
     return dev
@@ -434,9 +434,10 @@ def spkadd_batch_plan(problems, stream=None, options: Options | None = None) -> 
         ns.append(n)
         dts.append(dtype)
         keep.append(A)
+    device = problems[0][0][0][0].device  # (no problems: IndexError)
     _, nnz, cps, ris, vas = zip(*rows)
     return spkadd_batch_plan_raw(ks, ms, ns, nnz, cps, ris, vas, dts, stream=stream, options=options, keep=keep,
-                                 device=problems[0][0][0][0].device)
+                                 device=device)
 
 
 def spkadd_batch_symbolic(h: BatchHandle) -> list:

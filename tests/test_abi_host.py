@@ -186,6 +186,12 @@ def test_batch_plan_rejects_bad_arguments_without_cuda(lib, case, expect):
     assert not h.value
 
 
+def test_batch_of_no_problems_is_an_index_error():
+    for call in (spk.spkadd_batch_plan, spk.spkadd_batch):
+        with pytest.raises(IndexError):
+            call([])
+
+
 def test_batch_calls_on_null_handle(lib):
     n = (ctypes.c_int64 * 1)()
     assert lib.spkadd_batch_symbolic(None, ctypes.cast(n, ctypes.c_void_p)) == 1
