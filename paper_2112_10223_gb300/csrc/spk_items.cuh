@@ -107,6 +107,8 @@ __device__ __forceinline__ int item_table(ItemMap<B>& M, const Inputs& in, int o
 #pragma unroll
   for (int h = 0; h < KPT; ++h) {
     len[h] = F.end[h] - F.beg[h];
+    // Split windows of rows out of order: the end, the next window's start, may lie before the start.
+    if constexpr (VS > 0) len[h] = max(0, len[h]);
     ne += len[h] > 0;
     lsum += len[h];
   }

@@ -167,7 +167,7 @@ __device__ __forceinline__ void bitmap_item(const Inputs& in, const Window& W, c
       } else {
         const int32_t* o = offs + ((int64_t)W.search * in.kmax + i) * 2;
         b = o[0];
-        e = o[1];
+        e = max(b, o[1]);  // (rows out of order: the next window may start further down)
       }
       if (nsl > 1 && in.sorted) {  // unordered inputs: the whole segment, rows outside the slab skipped
         const int32_t* ri = in.ri[off + i];

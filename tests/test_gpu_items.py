@@ -207,3 +207,26 @@ def test_few_columns_of_a_kind_stay_out_of_the_table():
     a, b = (many, 4096), (few, 4096)
     flat = _launches([a, b], block_accumulator=1)
     assert _launches([a, b]) == flat + 1  # k_num_items for either kind, and k_num_dup for one
+
+
+@pytest.mark.parametrize("acc", [0, 1, 2])
+@pytest.mark.parametrize("m", [1 << 17, 1 << 20, (1 << 20) + 5000])
+def test_rows_out_of_order_stay_inside_the_inputs(m, acc):
+    """Unordered columns stated to be ordered: B is unspecified, but every segment of a split window stays inside its
+    input, and the next call is right.  (Starts of consecutive windows, found by binary search, may lie in either
+    order; segments of negative length would shift the other inputs' positions past their ends.)"""
+    k, L = 8, 20000
+    g = torch.Generator(device="cuda").manual_seed(m)
+    cp = torch.tensor([0, L, 2 * L], dtype=torch.int32, device="cuda")
+    A = [(cp, torch.cat([torch.randperm(m, generator=g, device="cuda")[:L] for _ in range(2)]).to(torch.int32),
+          torch.ones(2 * L, dtype=torch.float64, device="cuda")) for _ in range(k)]
+    h = spk.spkadd_plan(A, m, options=spk.default_options(block_accumulator=acc))
+    nnz = spk.spkadd_symbolic(h)
+    B = [torch.empty(3, dtype=torch.int64, device="cuda"), torch.full((nnz,), -1, dtype=torch.int32, device="cuda"),
+         torch.empty(nnz, dtype=torch.float64, device="cuda")]
+    spk.spkadd_numeric(h, *B)
+    info = spk.spkadd_get_info(h)
+    spk.spkadd_destroy(h)
+    assert info["windows_split"] > 8 and info["status"] in ("SPKADD_OK", "SPKADD_ERR_INTERNAL")
+    in_order = [(c, torch.cat([r[:L].sort().values, r[L:].sort().values]), v) for c, r, v in A]
+    assert check_full(in_order, m, torch.float64, exact=True)[0]["status"] == "SPKADD_OK"
