@@ -252,7 +252,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   else spkadd_default_options(&o);
   spkadd_status os = check_options(o);
   if (os != SPKADD_OK) return os;
-  int64_t nnz_in = 0, total_k = 0, ncols = 0, mmax = 0, win_cap = 0;
+  int64_t nnz_in = 0, total_k = 0, ncols = 0, mmax = 0, mmin = INT32_MAX, win_cap = 0;
   int kmax = 0, f32_kinds = 0;
   bool any32 = false, any64 = false;
   for (int q = 0; q < count; ++q) {
@@ -263,6 +263,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
     total_k += ks[q];
     ncols += As[q][0].n;
     if (As[q][0].m > mmax) mmax = As[q][0].m;
+    if (As[q][0].m < mmin) mmin = As[q][0].m;
     if (ks[q] > kmax) kmax = ks[q];
     (dts[q] == SPKADD_F64 ? any64 : any32) = true;
     if (dts[q] == SPKADD_F32)
@@ -310,7 +311,7 @@ static spkadd_status plan_problems(spkadd_handle** hp, bool batch, int count, co
   const size_t o_cl = cv.take<int32_t>(ncols);
   const size_t o_hl = cv.take<int32_t>(2 * ncols);
   // Columns for k_num_dup (never more than nnz / (warp_max + 1) columns are above the warp class).
-  const bool dup = o.block_accumulator == 0 && mmax <= (1 << spk::DUP_ROW_BITS);
+  const bool dup = o.block_accumulator == 0 && mmin <= (1 << spk::DUP_ROW_BITS);
   const int64_t dup_cap = !dup ? 0 : ncols < nnz_in / (o.warp_max + 1) ? ncols : nnz_in / (o.warp_max + 1);
   const size_t o_dup = cv.take<int32_t>(dup_cap);
   const size_t o_win = cv.take<Window>(win_cap);

@@ -127,7 +127,7 @@ __device__ __forceinline__ int item_kind(const Inst* I) {
 // least DUP_RATIO entries a row are summed by one warp each (k_num_dup).
 constexpr int DUP_MAX_U = 256;
 constexpr int DUP_RATIO = 4;
-constexpr int DUP_ROW_BITS = 23;  // rows below 2^23: a row and its table slot share a 32-bit key
+constexpr int DUP_ROW_BITS = 20;  // of problems of at most 2^20 rows: one slab of the symbolic kernels that list them
 // Fewer of them of one problem kind leave warps idle (a column of 4096 entries
 // takes one warp some 90 us): they go to the thread-block items instead.  Both
 // ways cross at 3500 (600 entries each), 6000 (4096) and 8000 (9000) float

@@ -40,6 +40,7 @@ constexpr int DUP_ROUNDS = 4;                    // at most this many inputs' la
 constexpr uint32_t DUP_EMPTY = 0xffffffffu;
 static_assert(DUP_MAX_U * 2 <= DUP_SLOTS, "at most half of the slots are taken");
 static_assert(DUP_ROW_BITS + DUP_SLOT_BITS <= 32, "a row and its slot share a key");
+static_assert(DUP_ROW_BITS == SLAB_BITS, "columns of one slab only");
 
 template <typename A>
 struct DupSmem {

@@ -78,8 +78,8 @@ def test_few_distinct_rows_many_terms():
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 @pytest.mark.parametrize("k,L,m", [(40, 16, 5000), (33, 32, 1 << 23), (200, 6, 9001), (70, 64, (1 << 23) + 1)])
 def test_many_columns_on_few_rows(k, L, m, dtype):
-    """Enough columns of 64 to 256 distinct rows for the warp-per-column table (rows below 2^23), one and
-    several segment tables, ragged and equal inputs, in and out of order."""
+    """Enough columns on few rows for the warp-per-column table where the problem has at most 2^20 rows (others stay
+    with the block items), one and several segment tables, ragged and equal inputs, in and out of order."""
     import synth
     n = 8300
     A = synth.spgemm_like(k, m, n, L, seed=9, dtype=dtype, value_kind="int8")
@@ -178,12 +178,63 @@ def _few_rows(k, m, groups, seed, dtype):
     return out
 
 
-def _launches(problems, **opt):
+def _launches(problems, wants=None, **opt):
     """Kernels launched for the problems, whose sums are checked."""
     outs, info = spk.spkadd_batch(problems, info=True, options=spk.default_options(**opt))
-    for (A, _), B in zip(problems, outs):
-        compare(tuple(t.cpu().numpy() for t in B), oracle.add(to_np(A)), A[0][2].dtype, exact=True)
+    for (A, _), B, want in zip(problems, outs, wants or [oracle.add(to_np(A)) for A, _ in problems]):
+        compare(tuple(t.cpu().numpy() for t in B), want, A[0][2].dtype, exact=True)
     return info["kernel_launches"]
+
+
+def _flipped(A):
+    """The inputs with every column's entries in the opposite order."""
+    out = []
+    for cp, ri, va in A:
+        col = torch.repeat_interleave(torch.arange(cp.numel() - 1, device=cp.device), (cp[1:] - cp[:-1]).long())
+        at = cp[:-1].long()[col] + cp[1:].long()[col] - 1 - torch.arange(ri.numel(), device=cp.device)
+        out.append((cp, ri[at], va[at]))
+    return out
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("k, m, P, L, beside, table", [
+    (40, 5000, 31, 15, 60, True),        # one key a lane in the final sort, entries of several inputs in a round
+    (600, 5000, 64, 1, 6, True),         # two keys; ten tables of 64 inputs, one entry to an input
+    (40, 1 << 20, 128, 32, 60, True),    # four keys; rows up to 2^20
+    (20, 9001, 255, 60, 100, True),      # eight keys
+    (5, 4096, 255, 255, 700, True),      # the most distinct rows a column may have, and one more
+    (5, 4096, 256, 256, 700, True),
+    (5, 4096, 257, 257, 700, False),
+    (130, 5000, 60, 30, 30, True),       # tables of 1920 positions: one start-bit map
+    (64, 5000, 80, 48, 60, True),        # of 3072: two
+    (100, 5000, 200, 50, 300, True),     # heavy columns (5000 entries), listed by k_sym_heavy
+])
+def test_table_of_few_rows_edges(k, m, P, L, beside, table, dtype):
+    """Columns that reach the warp-per-column table, of equal and of mixed segment lengths, in and out of order.  One
+    column on many rows, of the same class, goes to the block items in any case, so the table is one launch more than
+    the flat accumulator makes."""
+    groups = [(8300, P, L), (1, 1000, beside)]
+    A = _few_rows(k, m, groups, 3, dtype)
+    shorter = _few_rows(k, m, [(8300, P, max(1, L - 3)), groups[1]], 3, dtype)
+    empty = (torch.zeros_like(A[0][0]), A[0][1][:0], A[0][2][:0])
+    for inputs in (A, A[:k - k // 3] + shorter[:k // 3 - 1] + [empty] if P < 255 and L > 3 else A):
+        want = [oracle.add(to_np(inputs))]
+        for B, order in ((inputs, 0), (_flipped(inputs), 1)):
+            flat = _launches([(B, m)], want, block_accumulator=1, input_order=order)
+            assert _launches([(B, m)], want, input_order=order) - flat == table
+
+
+def test_table_of_few_rows_in_batches():
+    """One launch of the table for each problem kind; and in a batch with a problem of more than 2^20 rows, whose own
+    columns are never listed, the heavy columns of the others are."""
+    P = [(_few_rows(k, 4096, [(8300, 60, 15), (1, 1000, 3000 // k)], k, dt), 4096)
+         for k, dt in ((40, torch.float32), (200, torch.float32), (40, torch.float64))]
+    wants = [oracle.add(to_np(A)) for A, _ in P]
+    assert _launches(P, wants) - _launches(P, wants, block_accumulator=1) == 3
+    tall = _few_rows(30, 1 << 22, [(30, 200, 100), (10, 255, 200)], 4, torch.float64)
+    P = [(_few_rows(100, 5000, [(8300, 200, 50), (1, 1000, 300)], 5, torch.float64), 5000), (tall, 1 << 22)]
+    wants = [oracle.add(to_np(A)) for A, _ in P]
+    assert _launches(P, wants) - _launches(P, wants, block_accumulator=2) == 1
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
