@@ -21,13 +21,18 @@ LENGTHS = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 300, 5
 
 def _check(A, m, dtype, **opt):
     want = oracle.add(to_np(A))
+    s = sum(a[0].diff() for a in A).numpy()
+    unique = int(((np.diff(want["col_ptr"]) == s) & (s > 0)).sum())
+    launches = {}
     for method in ("twopass", "onepass"):
         out = run_gpu(A, m, dtype=dtype, options=spk.default_options(**opt), info=True, method=method)
         compare(tuple(t.cpu().numpy() for t in out[:3]), want, dtype, exact=True)
-    assert out[3]["onepass"] == 1 and out[3]["cols_unique"] >= 0
+        assert out[3]["onepass"] == (method == "onepass") and out[3]["cols_unique"] == unique
+        launches[method] = out[3]["kernel_launches"]
     outs = spk.spkadd_batch([([tuple(t.cuda() for t in a) for a in A], m)] * 2, options=spk.default_options(**opt))
     for o in outs:
         compare(tuple(t.cpu().numpy() for t in o), want, dtype, exact=True)
+    return launches
 
 
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
@@ -78,8 +83,12 @@ def test_columns_split_between_sort_and_buckets():
     lengths = [300, 512, 257, 256, 100, 400] * 20
     pool = [400 if j % 6 == 1 else m for j in range(len(lengths))]
     A = _columns(16, m, lengths, 6, torch.float64, pool)
-    _check(A, m, torch.float64)
-    _check(A, m, torch.float64, sort_mode=1)
+    for mode in (0, 1):  # bins, heavy and CTA counts, two light ones, scan, two light sums
+        assert _check(A, m, torch.float64, sort_mode=mode)["twopass"] == 8
+    far = _columns(16, m, lengths, 6, torch.float64)  # hardly a repeat: every long column stays in the buckets
+    assert _check(far, m, torch.float64)["twopass"] == 8
+    short = _columns(16, 1 << 17, lengths, 6, torch.float64)  # repeats expected: all to the sort
+    assert _check(short, 1 << 17, torch.float64)["twopass"] == 6
 
 
 def test_float_runs_round_once_and_keep_infinities():
