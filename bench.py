@@ -406,13 +406,21 @@ def time_pairwise_tree(A, m, ours, steps, warmup):
 
 
 def kernel_label(info, method):
+    """Numeric kernels of a step, by the library's rules for light columns (default warp_max): problems past 2^23 rows
+    and long columns of few expected repeats go through buckets, the others through the register sort."""
+    mean = info["nnz_in"] / max(info["n"], 1)
+    sort, few = info["m"] <= 1 << 23, mean >= 64 and 2 * mean * mean <= info["m"]
     if method == "onepass" and info.get("onepass"):
-        return "k_warp_onepass (spkadd_onepass)"
+        return ("k_sort_onepass" if sort and not (few and int(mean) > 256) else "k_warp_onepass") + " (spkadd_onepass)"
+    if not sort:
+        light = "k_warp_col"
+    elif not few:
+        light = "k_warp_sort"
+    else:  # (k_warp_col sums those above 256 entries)
+        light = "k_warp_col" if mean > 256 else "k_warp_sort and k_warp_col"
     if info["cols_cta"] + info["cols_heavy"] == 0:
-        mean = info["nnz_in"] / max(info["n"], 1)  # the library's rule (few repeats expected: buckets, else sorted)
-        return ("k_warp_col" if mean >= 64 and 2 * mean * mean <= info["m"] else "k_warp_sort") + \
-            "<numeric> (spkadd_numeric)"
-    return ("spkadd_numeric: k_warp_sort or k_warp_col, k_num_items and k_num_dup")
+        return light + "<numeric> (spkadd_numeric)"
+    return f"spkadd_numeric: {light}, k_num_items and k_num_dup"
 
 
 def run_ours(args, world, rank, local):

@@ -179,7 +179,8 @@ typedef struct spkadd_info {
     int64_t cols_warp;      /* columns per class (valid after spkadd_symbolic) */
     int64_t cols_cta;
     int64_t cols_heavy;
-    int64_t windows;        /* numeric thread-block work items (CTA columns + heavy windows) */
+    int64_t windows;        /* numeric work items above the warp class: CTA columns, heavy windows, and the columns
+                             * on few distinct rows that one warp each sums */
     int64_t windows_split;  /* of those, row windows that needed per-input binary searches */
     int64_t cols_unique;    /* warp columns in which no row repeats across the inputs */
     int64_t workspace_bytes;

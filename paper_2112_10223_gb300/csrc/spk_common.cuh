@@ -315,19 +315,6 @@ struct ChunkMap {
     *off = e - __shfl_sync(SPK_FULL, w.P, sg);
     return sg;
   }
-  // Element index (inside its input) of flattened position e; *seg = segment.
-  // Every lane must call it (it shuffles).
-  __device__ __forceinline__ int locate(int e, int* seg) const {
-    if (equal) {
-      const int sg = (int)__umulhi((uint32_t)e, magic32);
-      const int b = __shfl_sync(SPK_FULL, beg, sg & 31);
-      *seg = sg;
-      return b + (e - sg * L);
-    }
-    const int sg = w.find(e);
-    *seg = sg;
-    return w.index_in_input(e, sg);
-  }
 };
 
 // ---------------------------------------------------------------------------

@@ -123,21 +123,22 @@ template <typename V, typename A, bool PHASED, int BLOCK, int U, typename SegF, 
 __device__ __forceinline__ bool add_values(const Inputs& in, int k, int off, SegF& seg, FAdd& add, SegCache& sc,
                                            A* acc, V* oval, int slab_u, int lim, int s_ent) {
   auto none = [](uint32_t, int32_t, V) {};
-  if (!PHASED || s_ent - slab_u < FP32_ACC_TERMS) {
-    block_for_each_entry<true, V, BLOCK, U>(in, 0, k, off, seg, add, none, sc);
-    return false;
-  }
-  for (int p0 = 0; p0 < k; p0 += FP32_PHASE_INPUTS) {
-    SegCache fresh{0, 0, false};  // a phase's chunks differ from pass A's
-    block_for_each_entry<true, V, BLOCK, U>(in, p0, min(k, p0 + FP32_PHASE_INPUTS), off, seg, add, none, fresh);
-    __syncthreads();
-    for (int q = threadIdx.x; q < slab_u; q += BLOCK) {
-      if (q < lim) oval[q] = p0 == 0 ? (V)acc[q] : oval[q] + (V)acc[q];
-      acc[q] = A(0);
+  if constexpr (PHASED)
+    if (s_ent - slab_u >= FP32_ACC_TERMS) {
+      for (int p0 = 0; p0 < k; p0 += FP32_PHASE_INPUTS) {
+        SegCache fresh{0, 0, false};  // a phase's chunks differ from pass A's
+        block_for_each_entry<true, V, BLOCK, U>(in, p0, min(k, p0 + FP32_PHASE_INPUTS), off, seg, add, none, fresh);
+        __syncthreads();
+        for (int q = threadIdx.x; q < slab_u; q += BLOCK) {
+          if (q < lim) oval[q] = p0 == 0 ? (V)acc[q] : oval[q] + (V)acc[q];
+          acc[q] = A(0);
+        }
+        __syncthreads();
+      }
+      return true;
     }
-    __syncthreads();
-  }
-  return true;
+  block_for_each_entry<true, V, BLOCK, U>(in, 0, k, off, seg, add, none, sc);
+  return false;
 }
 
 // One item (a CTA-class column or a heavy column's row window [r_lo, r_hi),

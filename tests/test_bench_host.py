@@ -74,3 +74,19 @@ def test_wave_plan_respects_the_budget_and_order():
     for w in waves:
         used = sum(bench._instance_bytes(params[q]) for q in w)
         assert used <= budget or len(w) == 1
+
+
+@pytest.mark.parametrize("m, n, mean, onepass, above, want", [
+    (1 << 20, 1 << 20, 512, 0, 0, "k_warp_col<numeric>"),
+    (1 << 20, 1 << 20, 512, 1, 0, "k_warp_onepass"),
+    (1 << 20, 1 << 20, 100, 0, 0, "k_warp_sort and k_warp_col<numeric>"),
+    (1 << 20, 1 << 20, 100, 1, 0, "k_sort_onepass"),
+    (1024, 1024, 32, 0, 0, "k_warp_sort<numeric>"),
+    (1024, 1024, 32, 1, 0, "k_sort_onepass"),
+    ((1 << 23) + 1, 1000, 32, 0, 0, "k_warp_col<numeric>"),
+    ((1 << 23) + 1, 1000, 32, 1, 0, "k_warp_onepass"),
+    (1 << 20, 1 << 20, 1000, 0, 5, "spkadd_numeric: k_warp_sort, k_num_items"),
+])
+def test_kernel_label_follows_the_library_rules(m, n, mean, onepass, above, want):
+    info = {"m": m, "n": n, "nnz_in": mean * n, "cols_cta": above, "cols_heavy": 0, "onepass": onepass}
+    assert bench.kernel_label(info, "onepass" if onepass else "twopass").startswith(want)
