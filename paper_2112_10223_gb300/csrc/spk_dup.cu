@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(WARPS * 32, (DT == 1 || WIDE_ACC ? 24 : 32) / 
       for (int t = 0; t < E; ++t) D.list[lane * (E + 1) + t] = r[t];
       __syncwarp();
     };
-    const int eb = wsort_eb(rows);
+    const int eb = wsort_eb<WSORT_LOW>(rows);
     if (eb == 0) sort_rows(std::integral_constant<int, 1>());
     else if (eb == 1) sort_rows(std::integral_constant<int, 2>());
     else if (eb == 2) sort_rows(std::integral_constant<int, 4>());

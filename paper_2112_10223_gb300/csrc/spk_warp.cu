@@ -68,6 +68,7 @@ struct WarpColArgs {
   int smax;
   int force_dedup;         // numeric: sort_mode 1
   int unsorted_out;        // numeric: sort_mode 2
+  int bucket_max;          // numeric: longest column that may go to k_warp_col (bucket_column)
   int split;               // k_warp_col takes the columns of bucket_column, k_warp_sort the others
   int big_only;            // k_warp_col: the columns above WARP_SMALL entries only
   int small_only;          // k_warp_sort: the others only
@@ -233,9 +234,17 @@ struct ColState {
 // and sums those of them that proved to be at least seven eighths distinct rows
 // with its buckets; k_warp_sort takes all other columns.  (32 ER inputs of 2^20
 // rows, 512 entries a column, double: symbolic 1.48 ms against 2.6 ms sorted,
-// numeric 4.3 against 5.3 ms.)
-__device__ __forceinline__ bool bucket_column(int s, int u, bool numeric) {
-  return s > WARP_SMALL && (!numeric || (s - u) * 8 <= s);
+// numeric 4.3 against 5.3 ms.)  In other problems of at most 32 inputs the buckets
+// sum such columns up to BUCKET_NEAR entries, which fill the sort's 320 keys
+// badly (about 97000 columns of 258 entries in three inputs: float 215 against
+// 246 us, double 223 against 265; of 288: 212 and 227, 218 and 243; of 318: 208
+// and 211, 218 and 228), when there are enough of them for a launch of its own
+// (R-MAT scale 17, k = 4, float: 1300 of them 9 us among the other columns, 30 apart).
+constexpr int BUCKET_NEAR = 288;
+constexpr int BUCKET_NEAR_COLS = 1 << 15;
+
+__device__ __forceinline__ bool bucket_column(const WarpColArgs& a, int s, int u, bool numeric) {
+  return s > WARP_SMALL && (!numeric || (s <= a.bucket_max && (s - u) * 8 <= s));
 }
 
 template <bool NUMERIC, bool BATCH>
@@ -631,7 +640,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
     const int j = BATCH ? cur.g - I->colbase : cur.g;
     const int qb = max(5, ceil_log2(cur.s));
     const int NB = 1 << qb;
-    if ((a.split && !bucket_column(cur.s, cur.u, NUMERIC)) ||
+    if ((a.split && !bucket_column(a, cur.s, cur.u, NUMERIC)) ||
         (NUMERIC && BATCH && a.only_dtype >= 0 && I->dtype != a.only_dtype)) {
       // another launch handles this column
     } else if (NB > smax) {  // not reachable for a warp-class column
@@ -655,7 +664,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
         if (lane == 0) {
           a.u_out[cur.g] = cur.s - dups;
           n_unique += (dups == 0);
-          n_bucket += bucket_column(cur.s, cur.s - dups, true);
+          n_bucket += bucket_column(a, cur.s, cur.s - dups, true);
         }
       } else {
         // B(:,j) starts at col_ptr_B[g] - col_ptr_B[colbase] in its problem's buffers.
@@ -681,7 +690,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_warp_col(Inputs in, WarpColAr
 // Against the buckets (symbolic + numeric): 65536 columns of 256 to 384 entries
 // on 128 rows, float, four adds 3.40 -> 1.67 ms; R-MAT scale 14 k = 16 double
 // 0.182 -> 0.080 ms.
-template <int DT, bool NUMERIC, bool BATCH, bool RES, int WARPS>
+template <int DT, bool NUMERIC, bool BATCH, bool RES, int SIZES, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24) / WARPS) k_warp_sort(Inputs in, WarpColArgs a) {
   using VB = typename std::conditional<DT == 1, double, float>::type;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -690,8 +699,8 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
   if (lane < a.smax / 32) sm.blk[lane].x = 0u;
   __syncwarp();
   const int nbig = a.ctr->n_wbig;
-  const int c0 = a.small_only ? nbig : 0;
-  const int ncols = a.ctr->n_warp + nbig;
+  const int c0 = SIZES == WSORT_LOW || a.small_only ? nbig : 0;
+  const int ncols = ((SIZES & WSORT_LOW) ? a.ctr->n_warp : 0) + nbig;
   const int k0 = in.inst[0].k;
   if (RES && (BATCH || k0 > 32)) {  // the host never launches this; never index lanes past k
     if (threadIdx.x == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);
@@ -711,7 +720,7 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
   // Scalars of the current column and of the next one (loaded a column ahead).
   ColState cur = load_col<NUMERIC, BATCH>(in, a, c, ncols, RES, my_cp, lane, k0, nbig);
   ColState nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig);
-  int n_unique = 0;
+  int n_unique = 0, n_bucket = 0;
   while (cur.g >= 0) {
     const Inst* I = in.inst + cur.q;
     const int k = BATCH ? I->k : k0;
@@ -728,7 +737,7 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
         if constexpr (NUMERIC) x.vp = static_cast<const VB*>(in.val[off + i]);
       }
     };
-    if ((a.split && bucket_column(cur.s, cur.u, NUMERIC)) ||
+    if ((a.split && bucket_column(a, cur.s, cur.u, NUMERIC)) ||
         (NUMERIC && BATCH && a.only_dtype >= 0 && I->dtype != a.only_dtype)) {
       // another launch handles this column
     } else if (cur.s > a.smax) {  // not reachable for a warp-class column
@@ -743,9 +752,9 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
         orow = (BATCH ? out_row_of(a.out, cur.q) : a.out.row0) + out;
         oval = static_cast<VB*>(BATCH ? out_val_of(a.out, cur.q) : a.out.val0) + out;
       }
-      const int u = wsort_any<VB, NUMERIC>(sm, k, cur.s, m, NUMERIC && a.unsorted_out && cur.u == cur.s, bounds, lane);
+      const int u = wsort_any<VB, NUMERIC, SIZES>(sm, k, cur.s, m, NUMERIC && a.unsorted_out && cur.u == cur.s, bounds, lane);
       if constexpr (NUMERIC) {
-        if (u == cur.u) wsort_write<VB>(sm, wsort_eb(cur.s), cur.s, u, orow, oval, lane);
+        if (u == cur.u) wsort_write<VB, SIZES>(sm, cur.s, u, orow, oval, lane);
         else if (lane == 0) atomicOr(&a.ctr_w->err, ERR_INTERNAL);  // symbolic and numeric disagree
       }
       if constexpr (!NUMERIC) {
@@ -753,6 +762,7 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
           if (u < 0) atomicOr(&a.ctr_w->err, ERR_RANGE);  // a row outside [0, m): reported; B is never computed
           a.u_out[cur.g] = u < 0 ? cur.s : u;
           n_unique += u == cur.s;
+          n_bucket += bucket_column(a, cur.s, u, true);
         }
       }
     }
@@ -762,6 +772,7 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
     nxt = load_col<NUMERIC, BATCH>(in, a, c + stride, ncols, RES, my_cp, lane, k0, nbig);
   }
   if (!NUMERIC && lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
+  if (!NUMERIC && lane == 0 && n_bucket) atomicAdd(&a.ctr_w->n_bucket, n_bucket);
 }
 
 // Symbolic count of light columns of few rows: one bit per row in a bitmap of the
@@ -864,7 +875,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_warp_bits(Inputs in,
     if (lane == 0) {
       a.u_out[cur.g] = u;
       n_unique += u == cur.s;
-      n_bucket += bucket_column(cur.s, u, true);
+      n_bucket += bucket_column(a, cur.s, u, true);
     }
   }
   if (lane == 0 && n_unique) atomicAdd(&a.ctr_w->n_unique, n_unique);
@@ -1047,7 +1058,7 @@ struct SortTile {
   int uq[WARPS];                         // columns without repeated rows
 };
 
-template <int DT, bool RES, int WARPS>
+template <int DT, bool RES, int SIZES, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 3) k_sort_onepass(Inputs in, OnepassArgs a) {
   using VB = typename std::conditional<DT == 1, double, float>::type;
   static_assert(WARPS * ONEPASS_COLS_MAX <= 128, "four columns a lane in the tile's scan");
@@ -1106,7 +1117,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_sort_onepass(Inputs in, Onepa
               x.vp = static_cast<const VB*>(in.val[i]);
             }
           };
-          u = wsort_any<VB, true>(wsort_carve_slot<VB>(base, cap, c), k, s, m, false, bounds, lane);
+          u = wsort_any<VB, true, SIZES>(wsort_carve_slot<VB>(base, cap, c), k, s, m, false, bounds, lane);
           __syncwarp();
           if (u < 0) {  // a row outside [0, m): reported; B is not computed for the column
             if (lane == 0) atomicOr(&a.ctr_w->err, ERR_RANGE);
@@ -1159,7 +1170,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) k_sort_onepass(Inputs in, Onepa
         if (u > 0) {
           const int s = __ldg(a.s_arr + j);
           if (o + u <= a.capacity)
-            wsort_write<VB>(wsort_carve_slot<VB>(base, cap, c), wsort_eb(s), s, u, a.out_row + o,
+            wsort_write<VB, SIZES>(wsort_carve_slot<VB>(base, cap, c), s, u, a.out_row + o,
                             static_cast<VB*>(a.out_val) + o, lane);
           else if (lane == 0)
             atomicOr(&a.ctr_w->err, ERR_INTERNAL);
@@ -1179,11 +1190,19 @@ static int pow2_at_least(int x) {
   return p;
 }
 
+// Light columns of both lengths, together, below which one kernel sums them: R-MAT
+// scale 14, k = 16 (12000 of them) takes 233 us with one and 238 with two, scale
+// 20, k = 64 21.9 against 21.5 ms; in between (scale 15 to 17, k = 4, 16 and 64,
+// both types) they are within 2%, two the faster in double.
+constexpr int SORT_APART_COLS = 1 << 16;
+
 template <int DT, bool NUMERIC>
 static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max, int n_small, int n_big, int n_bucket,
                                    const DeviceInfo& dev, cudaStream_t st, int* launches) {
   using VB = typename std::conditional<DT == 1, double, float>::type;
   a.smax = pow2_at_least(warp_max) < 32 ? 32 : pow2_at_least(warp_max);
+  const bool sort = in.mmax <= (1 << WSORT_ROW_BITS);
+  a.bucket_max = in.split_warp ? WARP_MAX_LIMIT : !in.col_inst && in.kmax <= 32 ? BUCKET_NEAR : 0;
   cudaError_t e = cudaSuccess;
   auto go = [&](auto kern, int warps, size_t smem, int n_cols) {
     const int bps = resident_blocks((const void*)kern, warps * 32, smem);
@@ -1213,20 +1232,41 @@ static cudaError_t launch_warp_col(const Inputs& in, WarpColArgs a, int warp_max
       return cudaGetLastError();
     }
   }
-  const bool sort = in.mmax <= (1 << WSORT_ROW_BITS);
   // (Only k_warp_sort leaves every column without repeats as it is when B may be unsorted.)
-  a.split = sort && in.split_warp && a.smax > WARP_SMALL && !a.unsorted_out;
-  if (NUMERIC && n_bucket <= 0) a.split = 0;
+  const bool buckets = sort && a.bucket_max > 0 && a.smax > WARP_SMALL && !a.unsorted_out;
+  a.split = NUMERIC ? buckets && n_bucket >= (in.split_warp ? 1 : BUCKET_NEAR_COLS) : buckets && in.split_warp;
   a.big_only = a.split;
   a.small_only = a.split && (!NUMERIC || n_bucket == n_big);  // no column above WARP_SMALL is left to sort
-  const int n_sort = NUMERIC ? n_small + (a.small_only ? 0 : n_big) : -1;
-  if (sort && n_sort != 0) {
-    constexpr int SW = 4;
-    go(in.col_inst ? k_warp_sort<DT, NUMERIC, true, false, SW>
-       : in.kmax <= 32 ? k_warp_sort<DT, NUMERIC, false, true, SW>
-                       : k_warp_sort<DT, NUMERIC, false, false, SW>,
-       SW, SW * wsort_bytes<VB, NUMERIC>(a.smax), n_sort);
+  constexpr int SW = 4;
+  const int smax = a.smax;
+  auto go_sort = [&](auto sizes, int s, int n_cols) {
+    constexpr int S = decltype(sizes)::value;
+    a.smax = s;
+    // (Double sums of long columns run faster without the input pointers in registers:
+    // 62500 columns of 400 entries in 16 inputs 300 -> 271 us.)
+    constexpr bool RES = !(NUMERIC && DT == 1 && S == WSORT_LONG);
+    go(in.col_inst ? k_warp_sort<DT, NUMERIC, true, false, S, SW>
+       : in.kmax <= 32 ? k_warp_sort<DT, NUMERIC, false, RES, S, SW>
+                       : k_warp_sort<DT, NUMERIC, false, false, S, SW>,
+       SW, SW * wsort_bytes<VB, NUMERIC>(s), n_cols);
+  };
+  if constexpr (NUMERIC) {
+    // Short and long columns by kernels of their own, which keep more of their
+    // state in registers; few of both by one, since a launch takes longer.
+    const int n_long = a.small_only ? 0 : n_big;
+    if (sort && n_small > 0 && n_long > 0 && n_small + n_long < SORT_APART_COLS) {
+      go_sort(std::integral_constant<int, WSORT_LOW | WSORT_TOP>(), smax, n_small + n_long);
+    } else if (sort) {
+      if (n_long > 0) go_sort(std::integral_constant<int, WSORT_LONG>(), smax, n_long);
+      if (e == cudaSuccess && n_small > 0)
+        go_sort(std::integral_constant<int, WSORT_LOW>(), smax < WARP_SMALL ? smax : WARP_SMALL, n_small);
+    }
+  } else if (sort) {
+    // 10 and 12 keys a lane where such columns are likely.
+    if (in.mean_s >= 128 && in.mean_s <= 400) go_sort(std::integral_constant<int, WSORT_LOW | WSORT_LONG>(), smax, -1);
+    else go_sort(std::integral_constant<int, WSORT_LOW | WSORT_TOP>(), smax, -1);
   }
+  a.smax = smax;
   if (e == cudaSuccess && (!sort || a.split)) {
     constexpr int WARPS = 8;
     constexpr int U = NUMERIC ? 8 : 16;
@@ -1297,7 +1337,13 @@ static cudaError_t launch_onepass_t(const Inputs& in, OnepassArgs a, int warp_ma
     while (a.cols > 1 && (int64_t)a.n < (int64_t)WARPS * a.cols * dev.sms * 12) a.cols >>= 1;
     a.ntiles = (a.n + WARPS * a.cols - 1) / (WARPS * a.cols);
     smem = (size_t)WARPS * wsort_slots_bytes<VB>(a.smax, a.cols);
-    kern = in.kmax <= 32 ? k_sort_onepass<DT, true, WARPS> : k_sort_onepass<DT, false, WARPS>;
+    auto pick = [&](auto sizes) {
+      constexpr int S = decltype(sizes)::value;
+      kern = in.kmax <= 32 ? k_sort_onepass<DT, true, S, WARPS> : k_sort_onepass<DT, false, S, WARPS>;
+    };
+    if (max_s <= WARP_SMALL) pick(std::integral_constant<int, WSORT_LOW>());
+    else if (in.mean_s <= 384) pick(std::integral_constant<int, WSORT_LOW | WSORT_LONG>());
+    else pick(std::integral_constant<int, WSORT_LOW | WSORT_TOP>());
   } else {
     a.smax = pow2_at_least(warp_max) < 32 ? 32 : pow2_at_least(warp_max);
     a.ntiles = (a.n + WARPS - 1) / WARPS;

@@ -3,13 +3,16 @@
 // An entry's key is (row << pos_bits | position), 32 bits: the position is its
 // index in the flattened column (input after input), so keys are distinct,
 // equal rows end up adjacent in input order, and the value is found again
-// through the position.  A column of s entries takes N = 32 E >= s keys, E a
-// power of two up to 16, as a bitonic network over element index lane * E + i:
-// strides below E are compare-exchanges between a lane's own registers, the
-// others exchange one register with another lane.  No atomics, no counters and
-// no per-column table to clear, and the same work whatever the rows are: the
-// order-preserving buckets of k_warp_col need an insertion sort per bucket,
-// which is quadratic where rows repeat or crowd.
+// through the position.  A column of s entries takes N = 32 E >= s keys, E one
+// of 1, 2, 4, 8, 10, 12 and 16, as a bitonic network over element index
+// lane * E + i: strides below E are compare-exchanges between a lane's own
+// registers, the others exchange one register with another lane.  No atomics, no
+// counters and no per-column table to clear, and the same work whatever the rows
+// are: the order-preserving buckets of k_warp_col need an insertion sort per
+// bucket, which is quadratic where rows repeat or crowd.  10 and 12 keys a lane
+// are there because 16 do the work of 512 entries for 257 to 384 of them (float,
+// 16 inputs, numeric: 78125 columns of 320 entries 280 -> 212 us, buckets 234;
+// 65104 of 384 247 -> 205, buckets 252; symbolic 253 -> 219, filter 230).
 #pragma once
 
 #include "spk_common.cuh"
@@ -31,23 +34,70 @@ __device__ __forceinline__ uint32_t wsort_keep(uint32_t x, uint32_t y, bool up) 
   return (x < y) != up ? x : y;  // (keys differ, or are both past the end)
 }
 
+// Sorts a lane's E keys: Knuth's merge exchange (The Art of Computer Programming
+// 3, 5.2.2, algorithm M), for any E.
+template <int E, int P0, int P, int Q, int R, int D>
+__device__ __forceinline__ void wsort_lane(uint32_t (&r)[E]) {
+#pragma unroll
+  for (int i = 0; i + D < E; ++i)
+    if ((i & P) == R) wsort_ce(r[i], r[i + D]);
+  if constexpr (Q != P) wsort_lane<E, P0, P, Q / 2, P, Q - P>(r);
+  else if constexpr (P > 1) wsort_lane<E, P0, P / 2, P0, 0, P / 2>(r);
+}
+
+// Sorts a lane's E keys that form a bitonic sequence.  Comparing the halves
+// elementwise leaves two bitonic sequences (E even); what is left at an odd
+// length, 5 or 3, is sorted outright.
+template <int E>
+__device__ __forceinline__ void wsort_clean(uint32_t (&r)[E]) {
+  constexpr int ODD = E == 10 ? 5 : E == 12 ? 3 : 1;
+#pragma unroll
+  for (int st = E >> 1; st >= ODD; st >>= 1) {
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (i / st % 2 == 0 && i + st < E) wsort_ce(r[i], r[i + st]);
+  }
+#pragma unroll
+  for (int h = 0; ODD > 1 && h < E; h += ODD) {
+    if constexpr (ODD == 5) {
+      wsort_ce(r[h], r[h + 3]);
+      wsort_ce(r[h + 1], r[h + 4]);
+      wsort_ce(r[h], r[h + 2]);
+      wsort_ce(r[h + 1], r[h + 3]);
+      wsort_ce(r[h], r[h + 1]);
+      wsort_ce(r[h + 2], r[h + 4]);
+      wsort_ce(r[h + 1], r[h + 2]);
+      wsort_ce(r[h + 3], r[h + 4]);
+      wsort_ce(r[h + 2], r[h + 3]);
+    } else if constexpr (ODD == 3) {
+      wsort_ce(r[h], r[h + 1]);
+      wsort_ce(r[h + 1], r[h + 2]);
+      wsort_ce(r[h], r[h + 1]);
+    }
+  }
+}
+
 // Sorts the warp's 32 E keys ascending by element index lane * E + i.  The
 // merges across lanes are loops (lane masks at run time): unrolled, the
 // network of 16 keys a lane alone is 36 KB of code, and warps at different
 // places in it wait for instructions.
 template <int E>
 __device__ __forceinline__ void wsort_network(uint32_t (&r)[E], int lane) {
+  if constexpr (E == 10 || E == 12) {
+    wsort_lane<E, 8, 8, 8, 0, 8>(r);
+  } else {
 #pragma unroll
-  for (int size = 2; size <= E; size <<= 1) {
-    // First step of a merge: element x meets x ^ (size - 1); then strides size / 4, ..., 1.
-#pragma unroll
-    for (int i = 0; i < E; ++i)
-      if ((i ^ (size - 1)) > i) wsort_ce(r[i], r[i ^ (size - 1)]);
-#pragma unroll
-    for (int st = size >> 2; st >= 1; st >>= 1) {
+    for (int size = 2; size <= E; size <<= 1) {
+      // First step of a merge: element x meets x ^ (size - 1); then strides size / 4, ..., 1.
 #pragma unroll
       for (int i = 0; i < E; ++i)
-        if (!(i & st)) wsort_ce(r[i], r[i + st]);
+        if ((i ^ (size - 1)) > i) wsort_ce(r[i], r[i ^ (size - 1)]);
+#pragma unroll
+      for (int st = size >> 2; st >= 1; st >>= 1) {
+#pragma unroll
+        for (int i = 0; i < E; ++i)
+          if (!(i & st)) wsort_ce(r[i], r[i + st]);
+      }
     }
   }
 #pragma unroll 1
@@ -66,13 +116,26 @@ __device__ __forceinline__ void wsort_network(uint32_t (&r)[E], int lane) {
 #pragma unroll
       for (int i = 0; i < E; ++i) r[i] = wsort_keep(r[i], __shfl_xor_sync(SPK_FULL, r[i], lm), up);
     }
-#pragma unroll
-    for (int st = E >> 1; st >= 1; st >>= 1) {
-#pragma unroll
-      for (int i = 0; i < E; ++i)
-        if (!(i & st)) wsort_ce(r[i], r[i + st]);
-    }
+    wsort_clean<E>(r);
   }
+}
+
+// Networks a kernel holds: 1 to 8 keys a lane, 10 and 12, 16.  Without the
+// middle ones a column of more than 256 entries takes 16.
+enum : int { WSORT_LOW = 1, WSORT_MID = 2, WSORT_TOP = 4, WSORT_LONG = WSORT_MID | WSORT_TOP };
+
+// Sorted element x lies at x + (x >> eb): one pad word per E elements (an odd
+// stride between lanes) or, at 10 and 12 keys a lane, per 32 (of the shifts the
+// one with the fewest bank conflicts, storing and reading).
+template <int SIZES>
+__device__ __forceinline__ int wsort_eb(int s) {
+  if (!(SIZES & WSORT_LOW) || s > 256) return (SIZES & WSORT_MID) && s <= 384 ? 5 : 4;
+  return s <= 32 ? 0 : s <= 64 ? 1 : s <= 128 ? 2 : 3;
+}
+// Bits of a key's position, below the row.
+template <int SIZES>
+__device__ __forceinline__ int wsort_pb(int s) {
+  return (SIZES & WSORT_LOW) && s <= 256 ? 5 + wsort_eb<SIZES>(s) : 9;
 }
 
 constexpr int WSORT_KT = 64;  // inputs per segment table, two per lane
@@ -212,8 +275,8 @@ __device__ __forceinline__ void wsort_bounds(WsortIn<V>* s, int cb, int nk, Boun
 template <typename V, bool NUMERIC, int E, typename BoundsF>
 __device__ __forceinline__ int wsort_column(const WsortSmem& sm, int k, int s, uint32_t m, bool as_is,
                                             BoundsF& bounds, int lane) {
-  constexpr int EB = E == 1 ? 0 : E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4;
-  constexpr int PB = 5 + EB;  // position bits
+  constexpr int EB = E == 1 ? 0 : E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : E == 16 ? 4 : 5;  // wsort_eb
+  constexpr int PB = E > 8 ? 9 : 5 + EB;                                                    // wsort_pb
   V* sval = reinterpret_cast<V*>(sm.vals);
   uint32_t r[E];
   bool bad = false;
@@ -223,7 +286,7 @@ __device__ __forceinline__ int wsort_column(const WsortSmem& sm, int k, int s, u
     wsort_bounds<V>(in, 0, k, bounds, lane);
     const uint32_t magic = wsort_table<V, NUMERIC>(sm.seg, sm.blk, in, k, &total, lane);
     __syncwarp();
-    constexpr int G = E < 8 ? E : 8;
+    constexpr int G = E <= 8 ? E : E == 10 ? 5 : E == 12 ? 6 : 8;
 #pragma unroll
     for (int t0 = 0; t0 < E; t0 += G) {
       V v[G];
@@ -316,8 +379,10 @@ __device__ __forceinline__ int wsort_column(const WsortSmem& sm, int k, int s, u
   const int inc = warp_incl_scan(cnt, lane);
   const int u = __shfl_sync(SPK_FULL, inc, 31);
 #pragma unroll
-  for (int i = 0; i < E; ++i)
-    sm.key[lane * (E + 1) + i] = r[i];  // element x at x + (x >> EB): an odd stride between lanes
+  for (int i = 0; i < E; ++i) {
+    const int x = i0 + i;
+    sm.key[EB == 5 ? x + (x >> 5) : lane * (E + 1) + i] = r[i];  // x + (x >> EB)
+  }
   int q = inc - cnt;
   if (u < s) {
 #pragma unroll
@@ -368,12 +433,11 @@ __device__ __forceinline__ V wsort_run_sum(int a, int b, TermF&& term) {
   return (V)sum;
 }
 
-// Writes B(:, j) from a sorted column of 32 << eb key places: distinct row q's
-// run summed by wsort_run_sum.  (Columns without repeated rows are copied.)
-template <typename V>
-__device__ __forceinline__ void wsort_write(const WsortSmem& sm, int eb, int s, int u, int32_t* out_row, V* out_val,
-                                            int lane) {
-  const int pb = 5 + eb;
+// Writes B(:, j) from a sorted column: distinct row q's run summed by
+// wsort_run_sum.  (Columns without repeated rows are copied.)
+template <typename V, int SIZES>
+__device__ __forceinline__ void wsort_write(const WsortSmem& sm, int s, int u, int32_t* out_row, V* out_val, int lane) {
+  const int eb = wsort_eb<SIZES>(s), pb = wsort_pb<SIZES>(s);
   const uint32_t pm = (1u << pb) - 1u;
   const V* sval = reinterpret_cast<const V*>(sm.vals);
   if (u == s) {
@@ -393,20 +457,25 @@ __device__ __forceinline__ void wsort_write(const WsortSmem& sm, int eb, int s, 
   }
 }
 
-// log2 of the keys a lane holds for a column of s entries.
-__device__ __forceinline__ int wsort_eb(int s) { return s <= 32 ? 0 : s <= 64 ? 1 : s <= 128 ? 2 : s <= 256 ? 3 : 4; }
-
-// wsort_column for any s <= WSORT_MAX.
-template <typename V, bool NUMERIC, typename BoundsF>
+// wsort_column for any s <= WSORT_MAX that the kernel's networks hold.
+template <typename V, bool NUMERIC, int SIZES, typename BoundsF>
 __device__ __forceinline__ int wsort_any(const WsortSmem& sm, int k, int s, uint32_t m, bool as_is, BoundsF& bounds,
                                          int lane) {
-  switch (wsort_eb(s)) {
-    case 0: return wsort_column<V, NUMERIC, 1>(sm, k, s, m, as_is, bounds, lane);
-    case 1: return wsort_column<V, NUMERIC, 2>(sm, k, s, m, as_is, bounds, lane);
-    case 2: return wsort_column<V, NUMERIC, 4>(sm, k, s, m, as_is, bounds, lane);
-    case 3: return wsort_column<V, NUMERIC, 8>(sm, k, s, m, as_is, bounds, lane);
-    default: return wsort_column<V, NUMERIC, 16>(sm, k, s, m, as_is, bounds, lane);
+  if constexpr ((SIZES & WSORT_LOW) != 0) {
+    switch (wsort_eb<WSORT_LOW>(s)) {
+      case 0: return wsort_column<V, NUMERIC, 1>(sm, k, s, m, as_is, bounds, lane);
+      case 1: return wsort_column<V, NUMERIC, 2>(sm, k, s, m, as_is, bounds, lane);
+      case 2: return wsort_column<V, NUMERIC, 4>(sm, k, s, m, as_is, bounds, lane);
+      case 3: return wsort_column<V, NUMERIC, 8>(sm, k, s, m, as_is, bounds, lane);
+      default: break;
+    }
   }
+  if constexpr ((SIZES & WSORT_MID) != 0) {
+    if (s <= 320) return wsort_column<V, NUMERIC, 10>(sm, k, s, m, as_is, bounds, lane);
+    if (s <= 384) return wsort_column<V, NUMERIC, 12>(sm, k, s, m, as_is, bounds, lane);
+  }
+  if constexpr ((SIZES & WSORT_TOP) != 0) return wsort_column<V, NUMERIC, 16>(sm, k, s, m, as_is, bounds, lane);
+  return -1;  // (not reachable)
 }
 
 }  // namespace spk

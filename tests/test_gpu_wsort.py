@@ -15,13 +15,14 @@ from test_gpu_items import _columns
 
 pytestmark = pytest.mark.gpu
 
-# 32 E keys hold a column, E a power of two up to 16.
-LENGTHS = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 300, 511, 512]
+# 32 E keys hold a column, E = 1, 2, 4, 8, 10, 12 or 16.
+LENGTHS = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 288, 289, 300, 319, 320, 321, 383, 384, 385,
+           511, 512]
 
 
 def _check(A, m, dtype, **opt):
     want = oracle.add(to_np(A))
-    s = sum(a[0].diff() for a in A).numpy()
+    s = sum(a[0].cpu().diff() for a in A).numpy()
     unique = int(((np.diff(want["col_ptr"]) == s) & (s > 0)).sum())
     launches = {}
     for method in ("twopass", "onepass"):
@@ -75,6 +76,52 @@ def test_onepass_columns_per_warp(d):
     out = run_gpu(A, 7 * d, info=True, method="onepass")
     assert out[3]["onepass"] == 1
     compare(tuple(t.cpu().numpy() for t in out[:3]), want, torch.float64, exact=True)
+
+
+def _dealt(k, m, lengths, n, dtype, seed):
+    """k inputs; n columns of each length, dealt evenly to the inputs.  The rows of every other length lie close
+    together (many repeats across the inputs), those of the others anywhere."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    rows, counts = [[] for _ in range(k)], [[] for _ in range(k)]
+    for at, s in enumerate(lengths):
+        for i in range(k):
+            L = s // k + (i < s % k)
+            step = max(1, (m if at % 2 else 3 * max(1, s // k)) // max(L, 1))
+            r = torch.arange(L, device="cuda") * step + torch.randint(0, step, (n, L), generator=g, device="cuda")
+            rows[i].append(r.reshape(-1).to(torch.int32))
+            counts[i].append(torch.full((n,), L, device="cuda"))
+    out = []
+    for i in range(k):
+        cp = torch.zeros(n * len(lengths) + 1, dtype=torch.int32, device="cuda")
+        cp[1:] = torch.cumsum(torch.cat(counts[i]), 0)
+        ri = torch.cat(rows[i])
+        out.append((cp, ri, torch.randint(-8, 9, (ri.numel(),), generator=g, device="cuda").to(dtype)))
+    return out
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("k", [5, 32, 33, 70])  # inputs in registers, one chunk, two halves of a table, two tables
+def test_short_and_long_columns_in_kernels_of_their_own(k, dtype):
+    """Enough columns of both lengths that each is summed by its own kernel, at every network's edges; and by one."""
+    m = 60000
+    both = _dealt(k, m, [s for s in LENGTHS if s >= 31], 3200, dtype, k)
+    assert _check(both, m, dtype)["twopass"] == 7  # bins, three counts, scan, two light sums
+    few = _dealt(k, m, [s for s in LENGTHS if s >= 31], 50, dtype, k)
+    assert _check(few, m, dtype)["twopass"] == 6
+    long = _dealt(k, m, [s for s in LENGTHS if s > 288], 300, dtype, k)
+    assert _check(long, m, dtype)["twopass"] == 6
+    for rows in (m, 70000):  # a mean above 384: no networks of 320 and 384 keys
+        assert _check(_dealt(k, rows, [256, 385, 511, 512, 500], 60, dtype, k), rows, dtype)["twopass"] == 6
+
+
+def test_columns_just_above_the_short_ones():
+    """Columns of 257 to 288 entries of few repeats go to the buckets when there are many."""
+    m, n = 40000, 16400  # (mean 149: too many repeats expected for all long columns to go there)
+    near = _dealt(6, m, [20, 257, 20, 288, 20, 289], n, torch.float64, 1)
+    assert _check(near, m, torch.float64)["twopass"] == 8  # bins, three counts, scan, sort of short and long, buckets
+    repeats = _dealt(6, m, [257, 20, 288, 20, 289, 20], n, torch.float64, 1)
+    assert _check(repeats, m, torch.float64)["twopass"] == 7
+    assert _check(_dealt(6, m, [20, 257, 20, 288, 20, 289], 100, torch.float64, 1), m, torch.float64)["twopass"] == 6
 
 
 def test_columns_split_between_sort_and_buckets():
