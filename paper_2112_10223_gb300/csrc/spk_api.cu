@@ -1,5 +1,6 @@
 // spk_api.cu -- the C ABI (include/spkadd.h): argument checks, workspace,
 // phase ordering and kernel launches.  No compute happens on the host.
+#include <algorithm>
 #include <climits>
 #include <cstddef>
 #include <cstdlib>
@@ -549,7 +550,9 @@ static spkadd_status run_numeric(spkadd_handle* h, const spk::Outs& out) {
                              h->h_ctr.n_hwin, h->d_wsort, h->h_ctr.kind_n,
                              h->d_offs, h->d_colptr, out,
                              h->opt.window_max > h->opt.cta_max ? h->opt.window_max : h->opt.cta_max,
-                             h->opt.block_accumulator, h->d_ctr, h->dev, h->st, &item_launches);
+                             h->opt.block_accumulator,
+                             h->h_ctr.heavy_sum / std::max(1, h->h_ctr.n_heavy + h->h_ctr.n_big), h->d_ctr, h->dev,
+                             h->st, &item_launches);
   h->launches += item_launches;
   if (ce == cudaSuccess && h->h_ctr.n_dup > 0) {
     ce = spk::launch_num_dup(h->in, h->dup.cols, h->h_ctr.n_dup, h->h_ctr.dup_n, h->d_u, h->d_colptr, out, h->d_ctr, h->dev,

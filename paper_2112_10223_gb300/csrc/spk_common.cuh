@@ -40,6 +40,7 @@ struct Counters {
   int32_t n_big;        // heavy columns with s_j > BIG_S (listed apart, not counted in n_heavy)
   int32_t n_wbig;       // warp columns above WARP_SMALL entries, listed from the list's end
   int32_t max_warp_s;   // largest s_j of a warp column
+  int64_t heavy_sum;    // entries of the heavy columns
   // The symbolic phase's, from n_windows to n_dup: zero when it starts.
   int32_t n_windows;    // Window records of CTA-class columns, from the record array's start
   int32_t n_hwin;       // Window records of heavy columns, from the record array's end

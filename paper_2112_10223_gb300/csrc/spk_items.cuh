@@ -205,6 +205,36 @@ __device__ __forceinline__ int item_seg(const ItemMap<B>& M, const ItemSlots<B>&
   return (int)b.y + __popc(b.x & (0xfffffffeu & (0xffffffffu >> (31 - (threadIdx.x & 31)))));
 }
 
+// Positions [p0, p1) of a published table without chunks or barriers: each warp
+// walks an equal run of them, segment by segment, 32 U at a time.
+// f(rows, vals, n): the lane's entries are at rows[32 t] (and vals[32 t]) for
+// t < U with 32 t < n.
+template <int B, typename V, int U, typename F>
+__device__ __forceinline__ void item_walk(const ItemMap<B>& M, int64_t p0, int64_t p1, F&& f) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t run = (p1 - p0 + ItemMap<B>::NW - 1) / ItemMap<B>::NW;
+  int64_t p = p0 + wid * run;
+  const int64_t pe = min(p1, p + run);
+  int o = 0, oe = M.ne;  // the last segment that starts at or before p
+  while (oe - o > 1) {
+    const int mid = (o + oe) >> 1;
+    if (M.first[mid] <= p) o = mid;
+    else oe = mid;
+  }
+  for (; p < pe; ++o) {
+    const ulonglong2 seg = M.seg[o];
+    const int64_t end = min(pe, (int64_t)M.first[o + 1]);
+    const int32_t* rows = reinterpret_cast<const int32_t*>(seg.x) + p + lane;
+    const V* vals = reinterpret_cast<const V*>(seg.y) + p + lane;
+    for (int n = (int)(end - p); n > 0; n -= 32 * U) {  // (warp-uniform)
+      f(rows, vals, n - lane);
+      rows += 32 * U;
+      vals += 32 * U;
+    }
+    p = end;
+  }
+}
+
 // Issues the loads of the chunk's rows.  Slots are handled in groups; groups
 // past ns are skipped here and by every pass.
 template <int B>

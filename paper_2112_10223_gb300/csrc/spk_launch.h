@@ -82,10 +82,12 @@ cudaError_t launch_kind_sort(const Inputs& in, const Window* win, int cap, Windo
                              const DeviceInfo& dev, cudaStream_t st);
 // One launch per class and kind present: over the n_cta records at win's start
 // and the n_heavy ones at its end (win_cap records) when the batch has one
-// kind, else over the groups of wsort (host copy of kind_n).
+// kind, else over the groups of wsort (host copy of kind_n).  heavy_mean: entries
+// per heavy column.
 cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int64_t win_cap, int n_cta,
                            int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
-                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
+                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator,
+                           int64_t heavy_mean, Counters* ctr_w,
                            const DeviceInfo& dev, cudaStream_t st, int* launches);
 // The n columns of the dup list, n_kind of each problem kind (Counters::n_dup, dup_n).
 cudaError_t launch_num_dup(const Inputs& in, const int32_t* list, int n, const int32_t* n_kind, const int32_t* u,

@@ -21,13 +21,12 @@
 //            item.
 //
 // The bitmap covers a slab of 2^slab_log2 rows (at most 2^20): an item whose
-// rows span more is processed slab by slab, with per-input binary searches
-// for each slab's entries.
+// rows span more is processed slab by slab.
 //
 // k_num_items (below) is this accumulator with the entries' rows in registers,
 // as a flat bitmap or a compact word table; k_num_bitmap, which walks the
 // entries once per pass, runs only for block_accumulator = 1 on slabs of more
-// than 2^17 rows, whose bitmap fills the SM.
+// than 2^17 rows (from 2^20 on the bitmap fills the SM).
 #include <mutex>
 #include <type_traits>
 
@@ -341,6 +340,17 @@ struct ItemSmem {
   int umax;
 };
 
+// Threads per block: 256 for CTA-class columns (at most 4096 entries: one chunk,
+// four blocks per SM), 384 for the windows of heavy columns (window_max distinct
+// rows, mostly under 6144 entries; 512 threads measured 808 against 750 us on 96
+// columns of 480,000 entries, since more warps run with part of their slots).
+constexpr int CTA_ITEM_BLOCK = 256, HEAVY_ITEM_BLOCK = 384;
+// Rows in registers, chunk by chunk (one chunk in CTA-class columns); the same,
+// but items of several chunks and long segments walked in runs; all walked.
+enum : int { ITEM_CHUNK, ITEM_BOTH, ITEM_WALK };
+// Entries per segment from which an item of more than a chunk is walked in runs.
+constexpr int ITEM_LONG = 128;
+
 // Input i's part of the item of window W in column j.
 __device__ __forceinline__ void window_seg(const Inputs& in, const Window& W, const int32_t* offs, int off, int j, int i,
                                            int* beg, int* end) {
@@ -358,11 +368,12 @@ __device__ __forceinline__ void window_seg(const Inputs& in, const Window& W, co
 // One item, the record at sm.win[turn].  F holds the bounds of its first segment
 // table (read while the previous item ran) and leaves with those of the next
 // item, whose record (null: none) goes to sm.win[turn ^ 1].
-template <typename V, typename A, bool PHASED, bool WIDE, int B>
+template <typename V, typename A, bool PHASED, bool WIDE, int B, int MODE>
 __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, int turn, ItemBounds<B>& F,
                                          const int32_t* offs, int32_t* __restrict__ out_row, V* __restrict__ out_val,
                                          const ItemSmem<B>& sm, int slab_log2, int flat_rows, Counters* ctr_w) {
   constexpr int KT = ItemMap<B>::KT, CAP = ItemMap<B>::CAP;
+  constexpr bool WALK = MODE != ITEM_CHUNK, REGS = MODE != ITEM_WALK;
   const int tid = threadIdx.x;
   const Window& W = sm.win[turn];
   const Inst* I = in.inst + inst_of(in, W.col);
@@ -387,6 +398,12 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
   const int64_t S = (int64_t)1 << slab_log2;
   const int64_t span = (int64_t)W.r_hi - W.r_lo;
   const int nsl = span <= 0 ? 0 : (int)((span + S - 1) >> slab_log2);
+  // Several slabs: of a CTA-class column, one chunk, every slab takes all entries
+  // and skips the rows outside it.  A binary search's dozen dependent loads take
+  // longer than reading the rows again (25000 columns of 1200 entries in 16 inputs,
+  // 2^21 rows, float: 2369 -> 1950 us).  (Larger items would search, but the windows
+  // of a heavy column end with its slabs.)
+  constexpr bool KEEP = B == CTA_ITEM_BLOCK && MODE == ITEM_CHUNK;
   int u_done = 0;
   bool bad = false;
   for (int t = 0; t < nsl; ++t) {
@@ -394,11 +411,11 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
     const int hi = (int)min((int64_t)W.r_hi, (int64_t)lo + S);
     const uint32_t width = (uint32_t)(hi - lo);
     const bool flat = !WIDE || width <= (uint32_t)flat_rows;
-    // The item's entries of input i that fall in [lo, hi).
+    // The item's entries of input i.
     auto seg = [&](int i, int* beg, int* end) {
       int b, e;
       window_seg(in, W, offs, off, j, i, &b, &e);
-      if (nsl > 1 && in.sorted) {  // unordered inputs: the whole segment, rows outside the slab skipped
+      if (!KEEP && nsl > 1 && in.sorted) {
         const int32_t* ri = in.ri[off + i];
         b = lower_bound_i32(ri, b, e, lo);
         e = lower_bound_i32(ri, b, e, hi);
@@ -406,7 +423,7 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
       *beg = b;
       *end = e;
     };
-    uint32_t r[ITEM_SLOTS];  // rows less lo
+    uint32_t r[REGS ? ITEM_SLOTS : 1];  // rows less lo
     ItemSlots<B> L;
     int total = 0;  // positions of the current segment table
     L.ns = 0;
@@ -415,27 +432,29 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
     int s_ent = 0;
     auto table = [&](int ib, bool first, int* red) {
       const int k_lo = ib * KT, nk = min(KT, k - k_lo);
-      if (!(first && ib == 0 && nsl == 1)) F = item_bounds<B>(k_lo, nk, seg);
+      if (!(first && ib == 0 && (KEEP ? t == 0 || nib == 1 : nsl == 1))) F = item_bounds<B>(k_lo, nk, seg);
       if (!first) {
         total = item_table<sizeof(V), false, false>(M, in, off, k_lo, nk, F, red);
         return;
       }
-      total = item_table<sizeof(V), true, true>(M, in, off, k_lo, nk, F, red);
+      total = item_table<sizeof(V), true, REGS>(M, in, off, k_lo, nk, F, red);
       if (t == 0 && ib == 0 && next && tid < (int)(sizeof(Window) / 4))  // (every thread is past the previous item)
         reinterpret_cast<int32_t*>(&sm.win[turn ^ 1])[tid] = next_word;
       s_ent += total;
-      single = nib == 1 && total <= CAP;
+      single = REGS && nib == 1 && total <= CAP;
     };
     const uint32_t wmax = width - 1u;
     // Loaded rows to rows less lo; those outside the slab become 0xffffffff.
     auto relative = [&]() {
+      if constexpr (REGS) {
 #pragma unroll
-      for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
-        if (q0 >= L.ns) break;  // (warp-uniform)
+        for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+          if (q0 >= L.ns) break;  // (warp-uniform)
 #pragma unroll
-        for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
-          r[q] -= (uint32_t)lo;
-          r[q] = r[q] <= wmax ? r[q] : 0xffffffffu;
+          for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
+            r[q] -= (uint32_t)lo;
+            r[q] = r[q] <= wmax ? r[q] : 0xffffffffu;
+          }
         }
       }
     };
@@ -444,11 +463,23 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
       const uint32_t wd = c >> 5;
       return (int)spre[wd >> 5] + __popc(summ[wd >> 5] & ((1u << (wd & 31)) - 1u));
     };
-    // Runs op over every chunk of rows.  A single-chunk item is loaded by the
+    // Long segments: barrier-free runs instead of chunks.  (The table is published.)
+    auto long_segments = [&]() { return !REGS || (WALK && total > CAP && total >= ITEM_LONG * M.ne); };
+    // Runs mark(row less lo) over the rows.  A single-chunk item is loaded by the
     // first call only; others reload their rows (and rebuild the map) each time.
-    auto rows_pass = [&](bool first, auto&& op) {
+    auto rows_pass = [&](bool first, auto&& mark) {
+      auto slots = [&]() {
+        if constexpr (REGS) {
+#pragma unroll
+          for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+            if (q0 >= L.ns) break;  // (warp-uniform)
+#pragma unroll
+            for (int q = q0; q < q0 + ITEM_GROUP; ++q) mark(r[q]);
+          }
+        }
+      };
       if (!first && single) {
-        op();
+        slots();
         return;
       }
       for (int ib = 0; ib < nib; ++ib) {
@@ -457,18 +488,40 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
           table(ib, first, M.red[0]);
           if (!first) __syncthreads();
         }
-        for (int c0 = 0; total > 0; c0 += CAP) {
-          if (!first || c0 > 0) item_map(M, c0);
-          __syncthreads();
-          L.init(c0, total);
-          item_rows(M, L, c0, r);
-          relative();
-          op();
-          if (single) break;
-          __syncthreads();
-          item_unmap(M);
-          __syncthreads();
-          if (total - c0 <= CAP) break;
+        if (WALK && (!REGS || total > CAP)) {
+          if (first) __syncthreads();
+          if (long_segments()) {
+            item_walk<B, V, 8>(M, 0, total, [&](const int32_t* rows, const V*, int n) {
+              uint32_t x[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                x[u] = 0xffffffffu;
+                if (32 * u < n) x[u] = (uint32_t)__ldg(rows + 32 * u) - (uint32_t)lo;
+              }
+#pragma unroll
+              for (int u = 0; u < 8; ++u) mark(x[u]);
+            });
+            if (REGS && first) {
+              __syncthreads();
+              item_unmap(M);
+            }
+            continue;
+          }
+        }
+        if constexpr (REGS) {
+          for (int c0 = 0; total > 0; c0 += CAP) {
+            if (!first || c0 > 0) item_map(M, c0);
+            __syncthreads();
+            L.init(c0, total);
+            item_rows(M, L, c0, r);
+            relative();
+            slots();
+            if (single) break;
+            __syncthreads();
+            item_unmap(M);
+            __syncthreads();
+            if (total - c0 <= CAP) break;
+          }
         }
       }
     };
@@ -479,18 +532,11 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
     const int per = nwords <= 4 * B ? 4 : (nwords <= 8 * B ? 8 : 16);
     // The passes have no branches: addresses come from the row clamped into
     // the slab, and only the atomic itself is predicated.
-    rows_pass(true, [&]() {
-#pragma unroll
-      for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
-        if (q0 >= L.ns) break;  // (warp-uniform)
-#pragma unroll
-        for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
-          const uint32_t c = min(r[q], wmax);
-          uint32_t* w = flat ? &bits[pad_word((int)(c >> 5))] : &summ[c >> 10];
-          const uint32_t bit = 1u << (flat ? c & 31 : (c >> 5) & 31);
-          if (r[q] <= wmax) atomicOr(w, bit);
-        }
-      }
+    rows_pass(true, [&](uint32_t x) {
+      const uint32_t c = min(x, wmax);
+      uint32_t* w = flat ? &bits[pad_word((int)(c >> 5))] : &summ[c >> 10];
+      const uint32_t bit = 1u << (flat ? c & 31 : (c >> 5) & 31);
+      if (x <= wmax) atomicOr(w, bit);
     });
     __syncthreads();
     if (t == nsl - 1 && nib == 1 && next) F = next_bounds();  // used when the next item starts
@@ -528,17 +574,10 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
       __syncthreads();
       fits = ne <= sm.umax && !bad;
       if (fits) {
-        rows_pass(false, [&]() {
-#pragma unroll
-          for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
-            if (q0 >= L.ns) break;  // (warp-uniform)
-#pragma unroll
-            for (int q = q0; q < q0 + ITEM_GROUP; ++q) {
-              const uint32_t c = min(r[q], wmax);
-              const int cc = compact(c);
-              if (r[q] <= wmax && cc < ne) atomicOr(&cw[cc], 1u << (c & 31));
-            }
-          }
+        rows_pass(false, [&](uint32_t x) {
+          const uint32_t c = min(x, wmax);
+          const int cc = compact(c);
+          if (x <= wmax && cc < ne) atomicOr(&cw[cc], 1u << (c & 31));
         });
         __syncthreads();
         const int pc = ne <= 4 * B ? 4 : (ne <= 8 * B ? 8 : 16);
@@ -578,51 +617,77 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
         for (int ph = 0; ph < nph; ++ph) {
           const int e_lo = phased ? M.phase[ph] : 0;
           const int e_hi = phased && ph + 1 < nph ? M.phase[ph + 1] : total;
-          for (int c0 = 0; e_lo < e_hi; c0 += CAP) {
+          // Rank of row x less lo (none for rows outside the slab).
+          auto rank_of = [&](uint32_t x) {
+            const uint32_t c = min(x, wmax);
+            uint32_t wbits;
+            int base;
+            if (flat) {
+              wbits = bits[pad_word((int)(c >> 5))];
+              base = wpre[c >> 5];
+            } else {
+              const int cc = min(ne - 1, compact(c));
+              wbits = cw[cc];
+              base = cpre[cc];
+            }
+            const uint32_t rank = (uint32_t)(base + __popc(wbits & ((1u << (c & 31)) - 1u)));
+            return x > wmax ? 0xffffffffu : rank;
+          };
+          const bool walk = !single && long_segments();
+          if (WALK && walk && e_lo < e_hi)
+            item_walk<B, V, 4>(M, e_lo, e_hi, [&](const int32_t* rows, const V* vals, int n) {
+              uint32_t x[4];
+              V v[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                x[u] = 0xffffffffu;
+                v[u] = V(0);
+                if (32 * u < n) {
+                  x[u] = (uint32_t)__ldg(rows + 32 * u) - (uint32_t)lo;
+                  v[u] = __ldg(vals + 32 * u);
+                }
+              }
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const uint32_t rank = rank_of(x[u]);
+                if (rank < (uint32_t)slab_u) atomicAdd(&acc[rank], (A)v[u]);
+              }
+            });
+          for (int c0 = 0; REGS && !walk && e_lo < e_hi; c0 += CAP) {
             if (c0 + (CAP - 1) >= e_lo) {
               if (!single) {
                 item_map(M, c0);
                 __syncthreads();
                 L.init(c0, total);
-                item_rows(M, L, c0, r);
+                if constexpr (REGS) item_rows(M, L, c0, r);
                 relative();
               }
+              if constexpr (REGS) {
 #pragma unroll
-              for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
-                if (q0 >= L.ns) break;  // (warp-uniform)
-                uint32_t rank[ITEM_GROUP];
-                V v[ITEM_GROUP];
+                for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+                  if (q0 >= L.ns) break;  // (warp-uniform)
+                  uint32_t rank[ITEM_GROUP];
+                  V v[ITEM_GROUP];
 #pragma unroll
-                for (int x = 0; x < ITEM_GROUP; ++x)
-                  v[x] = __ldg(reinterpret_cast<const V*>(M.seg[item_seg(M, L, q0 + x)].y) + (c0 + L.pos(q0 + x)));
+                  for (int x = 0; x < ITEM_GROUP; ++x)
+                    v[x] = __ldg(reinterpret_cast<const V*>(M.seg[item_seg(M, L, q0 + x)].y) + (c0 + L.pos(q0 + x)));
 #pragma unroll
-                for (int x = 0; x < ITEM_GROUP; ++x) {
-                  const int q = q0 + x;
-                  const uint32_t c = min(r[q], wmax);
-                  uint32_t wbits;
-                  int base;
-                  if (flat) {
-                    wbits = bits[pad_word((int)(c >> 5))];
-                    base = wpre[c >> 5];
-                  } else {
-                    const int cc = min(ne - 1, compact(c));
-                    wbits = cw[cc];
-                    base = cpre[cc];
+                  for (int x = 0; x < ITEM_GROUP; ++x) {
+                    const int q = q0 + x;
+                    rank[x] = rank_of(r[q]);
+                    // Row and rank together (20 + 12 bits) for the rows' write below.
+                    if (by_entry) r[q] = r[q] <= wmax ? r[q] | (rank[x] << 20) : 0xffffffffu;
+                    bool ok = L.live(q);
+                    if (PHASED && phased) {
+                      const int e = c0 + L.run + 32 * q + (tid & 31);
+                      ok = ok && e >= e_lo && e < e_hi;
+                    }
+                    if (!ok) rank[x] = 0xffffffffu;
                   }
-                  rank[x] = (uint32_t)(base + __popc(wbits & ((1u << (c & 31)) - 1u)));
-                  if (r[q] > wmax) rank[x] = 0xffffffffu;
-                  // Row and rank together (20 + 12 bits) for the rows' write below.
-                  if (by_entry) r[q] = r[q] <= wmax ? c | (rank[x] << 20) : 0xffffffffu;
-                  bool ok = L.live(q);
-                  if (PHASED && phased) {
-                    const int e = c0 + L.run + 32 * q + (tid & 31);
-                    ok = ok && e >= e_lo && e < e_hi;
-                  }
-                  if (!ok) rank[x] = 0xffffffffu;
+#pragma unroll
+                  for (int x = 0; x < ITEM_GROUP; ++x)
+                    if (rank[x] < (uint32_t)slab_u) atomicAdd(&acc[rank[x]], (A)v[x]);
                 }
-#pragma unroll
-                for (int x = 0; x < ITEM_GROUP; ++x)
-                  if (rank[x] < (uint32_t)slab_u) atomicAdd(&acc[rank[x]], (A)v[x]);
               }
               if (!single) {
                 __syncthreads();
@@ -658,16 +723,18 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
       }
       __syncthreads();
       int32_t* rows = reinterpret_cast<int32_t*>(acc);  // slab_u <= umax slots of at least 4 bytes
-      if (by_entry) {
+      if (REGS && by_entry) {
         // Every entry writes its row at its rank (equal rows write the same).
         // All ones marks a slot without a row; its rank, 4095, is below slab_u
         // only for a whole column of 4096 rows, where every entry has one.
+        if constexpr (REGS) {
 #pragma unroll
-        for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
-          if (q0 >= L.ns) break;  // (warp-uniform)
+          for (int q0 = 0; q0 < ITEM_SLOTS; q0 += ITEM_GROUP) {
+            if (q0 >= L.ns) break;  // (warp-uniform)
 #pragma unroll
-          for (int q = q0; q < q0 + ITEM_GROUP; ++q)
-            if ((r[q] >> 20) < (uint32_t)slab_u) rows[r[q] >> 20] = lo + (int)(r[q] & 0xfffffu);
+            for (int q = q0; q < q0 + ITEM_GROUP; ++q)
+              if ((r[q] >> 20) < (uint32_t)slab_u) rows[r[q] >> 20] = lo + (int)(r[q] & 0xfffffu);
+          }
         }
       } else if (flat) {
         for (int w = tid; w < nwords; w += B) {
@@ -705,14 +772,9 @@ __device__ __forceinline__ void reg_item(const Inputs& in, const Window* next, i
 }
 
 // DT: 0 = float values, 1 = double values; ACC: 0 sums in the value type, 1
-// float sums in phases, 2 float values summed in double.  B: threads per block,
-// 256 for CTA-class columns (at most 4096 entries: one chunk, four blocks per
-// SM), 384 for the windows of heavy columns (window_max distinct rows, mostly
-// under 6144 entries; 512 threads measured 808 against 750 us on 96 columns of
-// 480,000 entries, since more warps run with part of their slots).
-constexpr int CTA_ITEM_BLOCK = 256, HEAVY_ITEM_BLOCK = 384;
+// float sums in phases, 2 float values summed in double.
 
-template <int DT, int ACC, bool WIDE, int B>
+template <int DT, int ACC, bool WIDE, int B, int MODE>
 __global__ void __launch_bounds__(B, B == CTA_ITEM_BLOCK ? 4 : 2)
     k_num_items(Inputs in, const Window* __restrict__ win, int nwin, const int32_t* __restrict__ offs,
                 const int64_t* __restrict__ col_ptr, Outs o, int slab_log2, int umax, int flat_rows, int only_dtype,
@@ -769,7 +831,7 @@ __global__ void __launch_bounds__(B, B == CTA_ITEM_BLOCK ? 4 : 2)
       continue;
     }
     const int64_t out = col_ptr[W.col] - (in.col_inst ? col_ptr[I->colbase] : 0) + W.out_off;
-    reg_item<V, A, ACC == 1, WIDE, B>(in, more ? win + wi + step : nullptr, turn, F, offs, out_row_of(o, q) + out,
+    reg_item<V, A, ACC == 1, WIDE, B, MODE>(in, more ? win + wi + step : nullptr, turn, F, offs, out_row_of(o, q) + out,
                                       static_cast<V*>(out_val_of(o, q)) + out, sm, slab_log2, flat_rows, ctr_w);
     if (!more) break;
     wi += step;
@@ -902,11 +964,11 @@ static cudaError_t launch_items(K kern, int block, int blocks_per_sm, const Inpu
   return cudaGetLastError();
 }
 
-template <int DT, int ACC, bool WIDE, int B>
+template <int DT, int ACC, bool WIDE, int B, int MODE>
 static cudaError_t launch_reg_items(const Inputs& in, const Window* win, int n_win, const int32_t* offs,
                                     const int64_t* col_ptr, const Outs& out, int slab_log2, int umax, int flat_rows,
                                     int only_dtype, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
-  auto kern = k_num_items<DT, ACC, WIDE, B>;
+  auto kern = k_num_items<DT, ACC, WIDE, B, MODE>;
   const size_t smem = ItemLayout<WIDE, B>(slab_log2, umax, (DT == 1 || ACC == 2) ? 8 : 4).bytes();
   const int bps = resident_blocks((const void*)kern, B, smem);
   if (bps < 1) return cudaErrorInvalidConfiguration;
@@ -923,23 +985,40 @@ static cudaError_t launch_reg_items(const Inputs& in, const Window* win, int n_w
 template <int DT, int ACC>
 static cudaError_t launch_num_cta_t(const Inputs& in, const Window* win, int n_win, bool heavy, const int32_t* offs,
                                     const int64_t* col_ptr, const Outs& out, int umax, int accumulator,
-                                    int only_dtype, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st) {
+                                    int64_t heavy_mean, int only_dtype, Counters* ctr_w, const DeviceInfo& dev,
+                                    cudaStream_t st) {
   constexpr size_t VS = (DT == 1 || ACC == 2) ? 8 : 4;  // accumulator bytes
   int slab_log2 = 10;
   while (slab_log2 < NUM_SLAB_LOG2_MAX && ((int64_t)1 << slab_log2) < (int64_t)in.mmax) ++slab_log2;
   if (accumulator == 1 && slab_log2 > FLAT_LOG2) {
     const size_t sf = bitmap_smem_bytes(slab_log2, umax, VS);
-    auto kern = k_num_bitmap<DT, ACC, 1024, 4>;
-    const int bf = sf <= (size_t)dev.smem_optin ? resident_blocks((const void*)kern, 1024, sf) : 0;
-    return launch_items(kern, 1024, bf, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sf, only_dtype, ctr_w,
+    const bool small = sf <= (size_t)dev.smem_per_sm / 2 - 2048;  // room for several blocks
+    auto kern = small ? k_num_bitmap<DT, ACC, 256, 8> : k_num_bitmap<DT, ACC, 1024, 4>;
+    const int block = small ? 256 : 1024;
+    const int bf = sf <= (size_t)dev.smem_optin ? resident_blocks((const void*)kern, block, sf) : 0;
+    return launch_items(kern, block, bf, in, win, n_win, offs, col_ptr, out, slab_log2, umax, sf, only_dtype, ctr_w,
                         dev, st);
   }
   const bool wide = accumulator == 2 || slab_log2 > FLAT_LOG2;
   const int flat_rows = accumulator == 2 ? 0 : FLAT_ROWS;
-  auto launch = heavy ? (wide ? launch_reg_items<DT, ACC, true, HEAVY_ITEM_BLOCK>
-                              : launch_reg_items<DT, ACC, false, HEAVY_ITEM_BLOCK>)
-                      : (wide ? launch_reg_items<DT, ACC, true, CTA_ITEM_BLOCK>
-                              : launch_reg_items<DT, ACC, false, CTA_ITEM_BLOCK>);
+  // Heavy windows of flat slabs: blocks of 256 threads, or 384 while there are few
+  // windows (750 columns of 40000 entries in 16 inputs, 2^15 rows, float: 458 us with
+  // 384, 374 with 256; 122 windows of R-MAT scale 14: the call 222 and 232 us).
+  // Compact ones: 384 (tall columns 719 against 903 us with 256), chunk by chunk (12
+  // inputs of 1.7 M rows, 201 columns of 200,000 entries, double: the walk's code
+  // spills, 710 -> 760 us, and windows hold little more than a chunk); but in unordered
+  // inputs, whose windows read whole columns, 256 and walked from the start when the
+  // columns are long and their segments too (2500 columns of 12000 entries in 16
+  // inputs, 2^20 rows, float 1084 -> 981 us; of 6000 entries 1021 -> 1105 us).
+  auto launch = wide ? launch_reg_items<DT, ACC, true, CTA_ITEM_BLOCK, ITEM_CHUNK>
+                     : launch_reg_items<DT, ACC, false, CTA_ITEM_BLOCK, ITEM_CHUNK>;
+  if (heavy && wide)
+    launch = !in.sorted && heavy_mean >= 8192 && heavy_mean >= 100 * (int64_t)in.kmax
+                 ? launch_reg_items<DT, ACC, true, CTA_ITEM_BLOCK, ITEM_WALK>
+                 : launch_reg_items<DT, ACC, true, HEAVY_ITEM_BLOCK, ITEM_CHUNK>;
+  else if (heavy)
+    launch = n_win <= 4 * dev.sms ? launch_reg_items<DT, ACC, false, HEAVY_ITEM_BLOCK, ITEM_BOTH>
+                                  : launch_reg_items<DT, ACC, false, CTA_ITEM_BLOCK, ITEM_BOTH>;
   return launch(in, win, n_win, offs, col_ptr, out, slab_log2, umax, flat_rows, only_dtype, ctr_w, dev, st);
 }
 
@@ -1014,8 +1093,9 @@ cudaError_t launch_kind_sort(const Inputs& in, const Window* win, int cap, Windo
 
 cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window* win, int64_t win_cap, int n_cta,
                            int n_heavy, const Window* wsort, const int32_t* kind_n, const int32_t* offs,
-                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator, Counters* ctr_w,
-                           const DeviceInfo& dev, cudaStream_t st, int* launches) {
+                           const int64_t* col_ptr, const Outs& out, int window_max, int accumulator,
+                           int64_t heavy_mean, Counters* ctr_w, const DeviceInfo& dev, cudaStream_t st,
+                           int* launches) {
   *launches = 0;
   if (n_cta + n_heavy <= 0) return cudaSuccess;
   // Float problems: k <= FP32_ACC_TERMS sum in float, up to
@@ -1041,7 +1121,7 @@ cudaError_t launch_num_cta(const Inputs& in, int dt, int f32_kinds, const Window
     const int f = alone ? -1 : sel[q];
     auto launch = q == 0 ? launch_num_cta_t<0, 0> : q == 1 ? launch_num_cta_t<0, 1>
                   : q == 2 ? launch_num_cta_t<0, 2> : launch_num_cta_t<1, 0>;
-    e = launch(in, w, n, heavy, offs, col_ptr, out, window_max, accumulator, f, ctr_w, dev, st);
+    e = launch(in, w, n, heavy, offs, col_ptr, out, window_max, accumulator, heavy_mean, f, ctr_w, dev, st);
   }
   return e;
 }

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(256) k_bin(Inputs in, int warp_lim, int cta_ma
     // Heavy columns: the largest go to their own list, handed out first.
     warp_append(cls == CLS_HEAVY && s <= BIG_S, heavy_list, &ctr->n_heavy, g, lane);
     warp_append(cls == CLS_HEAVY && s > BIG_S, big_list, &ctr->n_big, g, lane);
+    if (cls == CLS_HEAVY) atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->heavy_sum), (unsigned long long)s);
   }
 }
 
@@ -235,13 +236,16 @@ __device__ __forceinline__ void dup_divide(const Inputs& in, const int32_t* __re
     }
   }
   if (!any) return;  // (block-uniform)
-  const int nw = ctr->n_windows, cap = (int)(win_cap - ctr->n_hwin);
+  // Larger ones than a CTA-class column join the heavy columns' records at the array's end.
+  const int nw = ctr->n_windows, nh = ctr->n_hwin;
+  const bool room = (int64_t)nw + nh + nd <= win_cap;
   __syncthreads();
+  if (threadIdx.x == 0 && !room) atomicOr(&ctr->err, ERR_WINDOW_CAP);
   constexpr int PER = 8;
-  int kept = 0, moved = 0;
+  int kept = 0, moved = 0;  // (moved: to CTA-class records)
   for (int x0 = 0; x0 < nd; x0 += PER * SCAN_BLOCK) {
     int g[PER], kind[PER];
-    unsigned keep = 0u, move = 0u;
+    unsigned keep = 0u, move = 0u, cta = 0u;
 #pragma unroll
     for (int t = 0; t < PER; ++t) {
       const int x = x0 + t * SCAN_BLOCK + (int)threadIdx.x;
@@ -251,11 +255,13 @@ __device__ __forceinline__ void dup_divide(const Inputs& in, const int32_t* __re
     for (int t = 0; t < PER; ++t)
       if (g[t] >= 0) {
         kind[t] = item_kind(in.inst + inst_of(in, g[t]));
-        (s[g[t]] <= limit[kind[t]] ? keep : move) |= 1u << t;
+        const int sg = s[g[t]];
+        (sg <= limit[kind[t]] ? keep : move) |= 1u << t;
+        if (sg > limit[kind[t]] && sg <= CTA_MAX_LIMIT) cta |= 1u << t;
       }
     // Every read of this part of the list comes before the scan's barrier, every write after it and no further on.
     long long total;
-    const long long ex = block_excl_scan64(__popc(keep) | ((long long)__popc(move) << 32), tmp, &total);
+    const long long ex = block_excl_scan64(__popc(keep) | ((long long)__popc(cta) << 32), tmp, &total);
     int at = kept + (int)(ex & 0xffffffff), wi = nw + moved + (int)(ex >> 32);
 #pragma unroll
     for (int t = 0; t < PER; ++t) {
@@ -270,9 +276,7 @@ __device__ __forceinline__ void dup_divide(const Inputs& in, const int32_t* __re
         w.u = u[g[t]];
         w.out_off = 0;
         w.search = -1;
-        if (wi < cap) win[wi] = w;
-        else atomicOr(&ctr->err, ERR_WINDOW_CAP);
-        ++wi;
+        if (room) win[(cta >> t) & 1u ? wi++ : (int)win_cap - 1 - atomicAdd(&ctr->n_hwin, 1)] = w;
       }
     }
     kept += (int)(total & 0xffffffff);
@@ -280,7 +284,7 @@ __device__ __forceinline__ void dup_divide(const Inputs& in, const int32_t* __re
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    ctr->n_windows = nw + moved;
+    ctr->n_windows = nw + (room ? moved : 0);
     ctr->n_dup = kept;
   }
   if (threadIdx.x < 4) ctr->dup_n[threadIdx.x] = left[threadIdx.x];

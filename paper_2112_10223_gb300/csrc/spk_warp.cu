@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(WARPS * 32, (!NUMERIC ? 32 : DT == 0 ? 28 : 24
           if (u < 0) atomicOr(&a.ctr_w->err, ERR_RANGE);  // a row outside [0, m): reported; B is never computed
           a.u_out[cur.g] = u < 0 ? cur.s : u;
           n_unique += u == cur.s;
-          n_bucket += bucket_column(a, cur.s, u, true);
+          if constexpr (RES) n_bucket += bucket_column(a, cur.s, u, true);  // (BUCKET_NEAR; others: k_warp_col counts)
         }
       }
     }

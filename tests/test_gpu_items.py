@@ -281,3 +281,44 @@ def test_rows_out_of_order_stay_inside_the_inputs(m, acc):
     assert info["windows_split"] > 8 and info["status"] in ("SPKADD_OK", "SPKADD_ERR_INTERNAL")
     in_order = [(c, torch.cat([r[:L].sort().values, r[L:].sort().values]), v) for c, r, v in A]
     assert check_full(in_order, m, torch.float64, exact=True)[0]["status"] == "SPKADD_OK"
+
+
+def _spread(k, m, n, L, seed, dtype):
+    """k inputs of n columns of L rows each, one in each of L equal ranges."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    step = m // L
+    cp = torch.arange(n + 1, dtype=torch.int32, device="cuda") * L
+    out = []
+    for _ in range(k):
+        ri = torch.arange(L, device="cuda") * step + torch.randint(0, step, (n, L), generator=g, device="cuda")
+        ri = ri.reshape(-1).to(torch.int32)
+        out.append((cp, ri, torch.randint(-8, 9, (ri.numel(),), generator=g, device="cuda").to(dtype)))
+    return out
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("k, L", [(3, 4000), (16, 800), (40, 300), (41, 300), (200, 45), (180, 130)])
+@pytest.mark.parametrize("m", [40000, 1 << 20, (1 << 21) + 3])
+def test_heavy_windows_of_several_chunks(k, L, m, dtype):
+    """Windows of more entries than a chunk holds, few (one block in two takes none) and more than four to an SM, in
+    and out of order: walked in runs where their segments are long, chunk by chunk where they are not."""
+    for n in (20, 330):
+        A = _spread(k, m, n, L, k, dtype)
+        want = oracle.add(to_np(A))
+        for B, order in ((A, 0), (_flipped(A), 1)):
+            out = spk.spkadd(B, m, info=True, options=spk.default_options(input_order=order))
+            compare(tuple(t.cpu().numpy() for t in out[:3]), want, dtype, exact=True)
+            assert out[3]["cols_heavy"] == n and out[3]["windows"] >= 2 * n
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_columns_over_several_slabs(dtype):
+    """CTA-class columns of problems past 2^20 rows: every slab takes the rows inside it, ends of slabs among them."""
+    m = (1 << 22) + 9
+    A = _spread(7, m, 200, 300, 2, dtype)
+    edge = torch.tensor([0, (1 << 20) - 1, 1 << 20, (1 << 21) - 1, 1 << 21, (1 << 22) - 1, 1 << 22, m - 1], dtype=torch.int32)
+    cp = torch.arange(201, dtype=torch.int32, device="cuda") * 8
+    A.append((cp, edge.cuda().repeat(200), torch.ones(1600, dtype=dtype, device="cuda")))
+    for B, opt in ((A, {}), (_flipped(A), dict(input_order=1)), (A, dict(block_accumulator=2))):
+        info, _ = check_full([tuple(t.cpu() for t in a) for a in B], m, dtype, exact=True, options=spk.default_options(**opt))
+        assert info["cols_cta"] == 200
